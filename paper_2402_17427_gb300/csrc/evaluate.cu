@@ -2,6 +2,11 @@
 // affine colour map fitted in centred form (channel means, then centred second moments; FP32
 // per thread, FP64 across threads and blocks, Cholesky in FP64), the corrected image clipped to
 // [0, 1], then PSNR (peak 1) and the loss's SSIM on the corrected image.
+//
+// Five launches.  Each streaming pass leaves one row of partial sums a block; the blocks of the next
+// pass add those rows up themselves (one 456-row column a warp, all loads independent), so that no
+// one-block reduction stands between two passes.  One thread adding 1,024 rows serially, as a kernel
+// of its own, took 59 to 77 us each (three of them: 206 of 372 us at 1920 x 1080).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -13,95 +18,146 @@
 namespace vg {
 namespace {
 
-constexpr int kEvalBlocks = 1024;
+// Blocks of a streaming pass: three an SM of the 152, so that a pass is one wave and the next one
+// has few rows to add (1,024 blocks: 37 us for the first pass, mostly six serial block sums a block).
+constexpr int kEvalBlocks = 456;
+constexpr int kEvalThreads = 256;
 constexpr int kMeans = 6;      // mean r, g, b of the rendering and of the target
 constexpr int kMoments = 15;   // 6 of the symmetric 3x3 covariance of x, 9 of the cross-covariance x y^T
 
-__device__ __forceinline__ double block_sum_d(double v, double* sm /*[8]*/) {
+__device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+  return v;
+}
+
+// The block's sums of K per-thread values (FP32 inside a warp's first step, FP64 beyond): one row
+// of `part`.
+template <int K>
+__device__ __forceinline__ void write_row(const float (&m)[K], double* __restrict__ part) {
+  __shared__ double sm[kEvalThreads / 32][K];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const double t = warp_sum_d((double)m[k]);
+    if (lane == 0) sm[w][k] = t;
+  }
   __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sm[k];
+  if (threadIdx.x < K) {
+    double t = 0.0;
+#pragma unroll
+    for (int j = 0; j < kEvalThreads / 32; ++j) t += sm[j][threadIdx.x];
+    part[(size_t)blockIdx.x * K + threadIdx.x] = t;
+  }
+}
+
+// tot[k] = sum over the nb rows of `part`, by every block that needs it: a warp takes columns
+// w, w + 8, ...  Ends with a block barrier.
+template <int K>
+__device__ __forceinline__ void sum_rows(const double* __restrict__ part, int nb, double* tot /*shared [K]*/) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int k = w; k < K; k += kEvalThreads / 32) {
+    double t = 0.0;
+#pragma unroll 5
+    for (int b = lane; b < nb; b += 32) t += part[(size_t)b * K + k];
+    t = warp_sum_d(t);
+    if (lane == 0) tot[k] = t;
+  }
   __syncthreads();
-  return t;
+}
+
+// body(x, y, p, n): the three channels of rendering and target at pixels p .. p + n - 1, n = 4 but
+// at the image's end.  WIDE: 16-byte loads, where every plane starts on a 16-byte boundary and the
+// pixel count is a multiple of 4; else the same four pixels by scalar loads (their lines stay in L1).
+template <bool WIDE, typename Body>
+__device__ __forceinline__ void each_quad(const float* __restrict__ img, const float* __restrict__ tgt, long long npx,
+                                          Body body) {
+  for (long long p = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x); p < npx;
+       p += 4 * (long long)gridDim.x * blockDim.x) {
+    float x[3][4], y[3][4];
+    const int n = WIDE ? 4 : (int)(npx - p < 4 ? npx - p : 4);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      if constexpr (WIDE) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(img + c * npx + p));
+        const float4 b = __ldg(reinterpret_cast<const float4*>(tgt + c * npx + p));
+        x[c][0] = a.x; x[c][1] = a.y; x[c][2] = a.z; x[c][3] = a.w;
+        y[c][0] = b.x; y[c][1] = b.y; y[c][2] = b.z; y[c][3] = b.w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          x[c][j] = j < n ? __ldg(img + c * npx + p + j) : 0.f;
+          y[c][j] = j < n ? __ldg(tgt + c * npx + p + j) : 0.f;
+        }
+      }
+    }
+    body(x, y, p, n);
+  }
 }
 
 // pass 1: channel sums of the rendering and the target
-__global__ void __launch_bounds__(256) cc_sums(const float* __restrict__ img, const float* __restrict__ tgt,
-                                               long long npx, double* __restrict__ part) {
-  __shared__ double sm[8];
+template <bool WIDE>
+__global__ void __launch_bounds__(kEvalThreads) cc_sums(const float* __restrict__ img, const float* __restrict__ tgt,
+                                                        long long npx, double* __restrict__ part) {
+  pdl_enter();
   float m[kMeans] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npx; p += (long long)gridDim.x * blockDim.x)
+  each_quad<WIDE>(img, tgt, npx, [&](const float (&x)[3][4], const float (&y)[3][4], long long, int) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      m[c] += img[c * npx + p];
-      m[3 + c] += tgt[c * npx + p];
+    for (int c = 0; c < 3; ++c) {   // absent pixels are 0
+      m[c] += (x[c][0] + x[c][1]) + (x[c][2] + x[c][3]);
+      m[3 + c] += (y[c][0] + y[c][1]) + (y[c][2] + y[c][3]);
     }
-#pragma unroll
-  for (int k = 0; k < kMeans; ++k) {
-    const double t = block_sum_d((double)m[k], sm);
-    if (threadIdx.x == 0) part[(size_t)blockIdx.x * kMeans + k] = t;
-  }
+  });
+  write_row<kMeans>(m, part);
 }
 
-__global__ void cc_means(const double* __restrict__ part, int nb, long long npx, double* __restrict__ mean) {
-  if (threadIdx.x < kMeans) {
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * kMeans + threadIdx.x];
-    mean[threadIdx.x] = s / (double)npx;
-  }
-}
-
-// pass 2: centred second moments (products of centred values are accurate in FP32)
-__global__ void __launch_bounds__(256) cc_moments(const float* __restrict__ img, const float* __restrict__ tgt,
-                                                  long long npx, const double* __restrict__ mean,
-                                                  double* __restrict__ part) {
-  __shared__ double sm[8];
+// pass 2: centred second moments (products of centred values are accurate in FP32).  Block 0 keeps
+// the means for the fit.
+template <bool WIDE>
+__global__ void __launch_bounds__(kEvalThreads) cc_moments(const float* __restrict__ img, const float* __restrict__ tgt,
+                                                           long long npx, const double* __restrict__ sums, int nb,
+                                                           double* __restrict__ mean, double* __restrict__ part) {
+  pdl_enter();
+  __shared__ double tot[kMeans];
+  sum_rows<kMeans>(sums, nb, tot);
   float mu[kMeans];
 #pragma unroll
-  for (int k = 0; k < kMeans; ++k) mu[k] = (float)mean[k];
+  for (int k = 0; k < kMeans; ++k) mu[k] = (float)(tot[k] / (double)npx);
+  if (blockIdx.x == 0 && threadIdx.x < kMeans) mean[threadIdx.x] = tot[threadIdx.x] / (double)npx;
   float m[kMoments];
 #pragma unroll
   for (int k = 0; k < kMoments; ++k) m[k] = 0.f;
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npx; p += (long long)gridDim.x * blockDim.x) {
-    const float x[3] = {img[p] - mu[0], img[npx + p] - mu[1], img[2 * npx + p] - mu[2]};
-    const float y[3] = {tgt[p] - mu[3], tgt[npx + p] - mu[4], tgt[2 * npx + p] - mu[5]};
+  each_quad<WIDE>(img, tgt, npx, [&](const float (&xs)[3][4], const float (&ys)[3][4], long long, int n) {
+    float t[kMoments];     // this quad's sums, added to the thread's once: a quarter of the additions in series
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int e = 0; e < 4; ++e) {
+      if (e >= n) break;
+      const float x[3] = {xs[0][e] - mu[0], xs[1][e] - mu[1], xs[2][e] - mu[2]};
+      const float y[3] = {ys[0][e] - mu[3], ys[1][e] - mu[4], ys[2][e] - mu[5]};
 #pragma unroll
-      for (int j = i; j < 3; ++j) {
-        const int k = i * 3 - i * (i - 1) / 2 + (j - i);   // upper-triangle slot of (i, j)
-        m[k] = fmaf(x[i], x[j], m[k]);
-      }
+      for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+        for (int j = i; j < 3; ++j) {
+          const int k = i * 3 - i * (i - 1) / 2 + (j - i);   // upper-triangle slot of (i, j)
+          t[k] = e == 0 ? x[i] * x[j] : fmaf(x[i], x[j], t[k]);
+        }
 #pragma unroll
-      for (int c = 0; c < 3; ++c) m[6 + 3 * i + c] = fmaf(x[i], y[c], m[6 + 3 * i + c]);
-  }
+      for (int i = 0; i < 3; ++i)
 #pragma unroll
-  for (int k = 0; k < kMoments; ++k) {
-    const double t = block_sum_d((double)m[k], sm);
-    if (threadIdx.x == 0) part[(size_t)blockIdx.x * kMoments + k] = t;
-  }
+        for (int c = 0; c < 3; ++c) t[6 + 3 * i + c] = e == 0 ? x[i] * y[c] : fmaf(x[i], y[c], t[6 + 3 * i + c]);
+    }
+#pragma unroll
+    for (int k = 0; k < kMoments; ++k) m[k] += t[k];
+  });
+  write_row<kMoments>(m, part);
 }
 
 // Least squares in centred form: Cov(x) A^T = Cov(x, y), b = mean(y) - A mean(x), by a Cholesky
 // factorisation that drops a colour direction whose pivot falls below 1e-10 of the trace (its
 // coefficient is 0: the remaining columns span the same space, so the fitted values are those of
 // every least-squares solution; a constant rendering gets A = 0, b = mean(y)).
-__global__ void cc_solve(const double* __restrict__ part, int nb, const double* __restrict__ mean,
-                         double* __restrict__ coef, float* __restrict__ out) {
-  __shared__ double tot[kMoments];
-  if (threadIdx.x < kMoments) {
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * kMoments + threadIdx.x];
-    tot[threadIdx.x] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
+// coef = (A row-major, b); one thread, from the totals and the means.
+__device__ void cc_solve(const double* tot, const double* mean, double* coef) {
   double C[3][3], K[3][3], L[3][3] = {{0}};
   for (int i = 0, k = 0; i < 3; ++i)
     for (int j = i; j < 3; ++j, ++k) C[i][j] = C[j][i] = tot[k];
@@ -138,50 +194,82 @@ __global__ void cc_solve(const double* __restrict__ part, int nb, const double* 
     double b = mean[3 + c];
     for (int i = 0; i < 3; ++i) {
       coef[3 * c + i] = At[i][c];
-      out[2 + 3 * c + i] = (float)At[i][c];
       b -= At[i][c] * mean[i];
     }
     coef[9 + c] = b;
-    out[11 + c] = (float)b;
   }
 }
 
-__global__ void __launch_bounds__(256) cc_apply(const float* __restrict__ img, const float* __restrict__ tgt,
-                                                long long npx, const double* __restrict__ coef,
-                                                float* __restrict__ corr, double* __restrict__ part) {
-  __shared__ double sm[8];
+// pass 3: every block solves the 3 x 3 system for itself (block 0 writes the map out), then the
+// corrected image and its squared error.
+template <bool WIDE>
+__global__ void __launch_bounds__(kEvalThreads) cc_apply(const float* __restrict__ img, const float* __restrict__ tgt,
+                                                         long long npx, const double* __restrict__ mom, int nb,
+                                                         const double* __restrict__ mean, float* __restrict__ corr,
+                                                         double* __restrict__ part, float* __restrict__ out) {
+  pdl_enter();
+  __shared__ double tot[kMoments], coef[12];
+  sum_rows<kMoments>(mom, nb, tot);
+  if (threadIdx.x == 0) cc_solve(tot, mean, coef);
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x < 12) out[2 + threadIdx.x] = (float)coef[threadIdx.x];
   float A[9], b[3];
 #pragma unroll
   for (int k = 0; k < 9; ++k) A[k] = (float)coef[k];
 #pragma unroll
   for (int c = 0; c < 3; ++c) b[c] = (float)coef[9 + c];
-  float se = 0.f;
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < npx; p += (long long)gridDim.x * blockDim.x) {
-    const float x0 = img[p], x1 = img[npx + p], x2 = img[2 * npx + p];
+  float se[1] = {0.f};
+  each_quad<WIDE>(img, tgt, npx, [&](const float (&x)[3][4], const float (&y)[3][4], long long p, int n) {
+    float t = 0.f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float v = fminf(1.f, fmaxf(0.f, fmaf(A[3 * c], x0, fmaf(A[3 * c + 1], x1, fmaf(A[3 * c + 2], x2, b[c])))));
-      corr[c * npx + p] = v;
-      const float d = v - tgt[c * npx + p];
-      se = fmaf(d, d, se);
+      float v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        v[e] = fminf(1.f, fmaxf(0.f, fmaf(A[3 * c], x[0][e], fmaf(A[3 * c + 1], x[1][e], fmaf(A[3 * c + 2], x[2][e], b[c])))));
+        const float d = e < n ? v[e] - y[c][e] : 0.f;
+        t = fmaf(d, d, t);
+      }
+      if constexpr (WIDE) {
+        *reinterpret_cast<float4*>(corr + c * npx + p) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (e < n) corr[c * npx + p + e] = v[e];
+      }
     }
-  }
-  const double t = block_sum_d((double)se, sm);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
+    se[0] += t;
+  });
+  write_row<1>(se, part);
 }
 
-__global__ void cc_finish(const double* __restrict__ part, int nb, long long n, const float* __restrict__ dssim,
-                          float* __restrict__ out) {
+// PSNR from the squared-error rows, SSIM from the moment pass's partial sums (sum S, sum |x - y|).
+__global__ void __launch_bounds__(1024) cc_finish(const double* __restrict__ sq, int nb, const double* __restrict__ ssim,
+                                                  int ns, long long n, float* __restrict__ out) {
+  pdl_enter();
+  __shared__ double sm[2][32];
+  double e = 0.0, t = 0.0;
+  for (int b = threadIdx.x; b < nb; b += 1024) e += sq[b];
+#pragma unroll 4
+  for (int b = threadIdx.x; b < ns; b += 1024) t += ssim[2 * (size_t)b];
+  e = warp_sum_d(e);
+  t = warp_sum_d(t);
+  if ((threadIdx.x & 31) == 0) {
+    sm[0][threadIdx.x >> 5] = e;
+    sm[1][threadIdx.x >> 5] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  e = warp_sum_d(sm[0][threadIdx.x]);
+  t = warp_sum_d(sm[1][threadIdx.x]);
   if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += part[b];
-  const double mse = s / (double)n;
+  const double mse = e / (double)n;
   out[0] = mse > 0.0 ? (float)(-10.0 * log10(mse)) : INFINITY;
-  out[1] = 1.f - *dssim;    // the loss entry point with lambda = 1 gives 1 - SSIM
+  out[1] = (float)(t / (double)n);
 }
 
 struct EvalLayout {
-  size_t corr, sums, mean, mom, coef, sq, dssim, loss, total;
+  size_t corr, sums, mean, mom, sq, ssim, total;
 };
 
 EvalLayout eval_layout(int W, int H) {
@@ -193,12 +281,27 @@ EvalLayout eval_layout(int W, int H) {
   L.sums = take((size_t)kEvalBlocks * kMeans * sizeof(double));
   L.mean = take(kMeans * sizeof(double));
   L.mom = take((size_t)kEvalBlocks * kMoments * sizeof(double));
-  L.coef = take(16 * sizeof(double));
   L.sq = take((size_t)kEvalBlocks * sizeof(double));
-  L.dssim = take(sizeof(float));
-  L.loss = take(vg_loss_workspace_bytes(W, H));
+  L.ssim = take((size_t)ssim_partials(W, H) * 2 * sizeof(double));
   L.total = o;
   return L;
+}
+
+template <bool WIDE>
+cudaError_t launch_eval(const float* img, const float* target, int W, int H, const EvalLayout& L, char* ws, float* out,
+                        cudaStream_t s) {
+  const long long npx = (long long)W * H;
+  const int nb = (int)std::min<long long>(kEvalBlocks, (npx + 4 * kEvalThreads - 1) / (4 * kEvalThreads));
+  auto D = [&](size_t off) { return reinterpret_cast<double*>(ws + off); };
+  float* corr = reinterpret_cast<float*>(ws + L.corr);
+  note_launches(4);
+  cc_sums<WIDE><<<nb, kEvalThreads, 0, s>>>(img, target, npx, D(L.sums));
+  launch_pdl(cc_moments<WIDE>, nb, kEvalThreads, 0, s, img, target, npx, D(L.sums), nb, D(L.mean), D(L.mom));
+  launch_pdl(cc_apply<WIDE>, nb, kEvalThreads, 0, s, img, target, npx, D(L.mom), nb, D(L.mean), corr, D(L.sq), out);
+  const cudaError_t e = launch_ssim_value(corr, target, W, H, D(L.ssim), s);
+  if (e != cudaSuccess) return e;
+  launch_pdl(cc_finish, 1, 1024, 0, s, D(L.sq), nb, D(L.ssim), ssim_partials(W, H), 3 * npx, out);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -219,24 +322,10 @@ extern "C" vg_status vg_eval_color_corrected(const float* img, const float* targ
   if (workspace_bytes < L.total) return VG_ERR_CAPACITY;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
-  const long long npx = (long long)width * height;
-  const int nb = (int)std::min<long long>(kEvalBlocks, (npx + 255) / 256);
-  double* mom = reinterpret_cast<double*>(ws + L.mom);
-  double* coef = reinterpret_cast<double*>(ws + L.coef);
-  double* sq = reinterpret_cast<double*>(ws + L.sq);
-  float* corr = reinterpret_cast<float*>(ws + L.corr);
-  float* dssim = reinterpret_cast<float*>(ws + L.dssim);
-  double* sums = reinterpret_cast<double*>(ws + L.sums);
-  double* mean = reinterpret_cast<double*>(ws + L.mean);
-  cc_sums<<<nb, 256, 0, s>>>(img, target, npx, sums);
-  cc_means<<<1, 32, 0, s>>>(sums, nb, npx, mean);
-  cc_moments<<<nb, 256, 0, s>>>(img, target, npx, mean, mom);
-  cc_solve<<<1, 32, 0, s>>>(mom, nb, mean, coef, out);
-  cc_apply<<<nb, 256, 0, s>>>(img, target, npx, coef, corr, sq);
-  note_launches(6);
-  const vg_status st = vg_loss_l1_dssim(corr, target, width, height, 1.0f, ws + L.loss,
-                                        vg_loss_workspace_bytes(width, height), dssim, nullptr, stream);
-  if (st != VG_OK) return st;
-  cc_finish<<<1, 32, 0, s>>>(sq, nb, 3 * npx, dssim, out);
-  return cudaGetLastError() == cudaSuccess ? VG_OK : VG_ERR_CUDA;
+  // 16-byte loads need the images on 16-byte boundaries and planes of a multiple of 4 pixels
+  const bool wide = ((reinterpret_cast<uintptr_t>(img) | reinterpret_cast<uintptr_t>(target)) & 15u) == 0 &&
+                    ((long long)width * height) % 4 == 0;
+  const cudaError_t e = wide ? launch_eval<true>(img, target, width, height, L, ws, out, s)
+                             : launch_eval<false>(img, target, width, height, L, ws, out, s);
+  return e == cudaSuccess ? VG_OK : VG_ERR_CUDA;
 }

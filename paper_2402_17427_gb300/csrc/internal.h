@@ -292,6 +292,8 @@ size_t ssim_maps_floats(int W, int H);
 int ssim_partials(int W, int H);
 cudaError_t launch_ssim_moments(const float* x, const float* y, int W, int H, float lambda, float* maps,
                                 double* partials, cudaStream_t s);
+// The moment pass alone, without the maps (the evaluation's SSIM): partials as above.
+cudaError_t launch_ssim_value(const float* x, const float* y, int W, int H, double* partials, cudaStream_t s);
 cudaError_t launch_ssim_grad_appearance(const float* x, const float* y, const float* maps, int W, int H,
                                         const float* pool_grad, int pw, int ph, float* grad, cudaStream_t s);
 

@@ -161,6 +161,9 @@ __device__ __forceinline__ void stage_pairs(const float* const (&plane)[F], int 
 // Moments of a 32x32 output tile: x, y staged with a 5-pixel zero-padded halo as row pairs.  The
 // horizontal pass (21 row pairs x 4 groups of 8 columns) slides the window along a row for two
 // rows at once; the vertical pass (32 columns x 4 groups of 8 rows) slides it down a column.
+// kMaps: the derivative maps for the gradient pass are written; without it the pass leaves the
+// partial sums alone (the evaluation needs no gradient).
+template <bool kMaps>
 __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float* __restrict__ x,
                                                                     const float* __restrict__ y, int W, int H,
                                                                     Win win, float dLdS, float* __restrict__ maps,
@@ -241,14 +244,18 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
     const float2 g1 = __fmul2_rn(dl, __fmul2_rn(neg(S), iD2));
     const float2 g2 = __fmul2_rn(dl, __fmul2_rn(__fmul2_rn(two, N1), iD));
     const size_t pix = (size_t)gy * W + gx;
-    maps[(0 * 3 + c) * plane + pix] = g0.x;
-    maps[(1 * 3 + c) * plane + pix] = g1.x;
-    maps[(2 * 3 + c) * plane + pix] = g2.x;
+    if constexpr (kMaps) {
+      maps[(0 * 3 + c) * plane + pix] = g0.x;
+      maps[(1 * 3 + c) * plane + pix] = g1.x;
+      maps[(2 * 3 + c) * plane + pix] = g2.x;
+    }
     ssum += S.x;
     if (in1) {
-      maps[(0 * 3 + c) * plane + pix + W] = g0.y;
-      maps[(1 * 3 + c) * plane + pix + W] = g1.y;
-      maps[(2 * 3 + c) * plane + pix + W] = g2.y;
+      if constexpr (kMaps) {
+        maps[(0 * 3 + c) * plane + pix + W] = g0.y;
+        maps[(1 * 3 + c) * plane + pix + W] = g1.y;
+        maps[(2 * 3 + c) * plane + pix + W] = g2.y;
+      }
       ssum += S.y;
     }
   }
@@ -433,8 +440,15 @@ cudaError_t launch_ssim_moments(const float* x, const float* y, int W, int H, fl
   const dim3 grid((W + LT - 1) / LT, (H + LT - 1) / LT, 3);
   const double inv = 1.0 / (3.0 * (double)W * H);
   note_launches(1);
-  ssim_forward_kernel<<<grid, kLossThreads, 0, s>>>(x, y, W, H, make_window(), (float)(-lambda * inv), maps, partials);
+  ssim_forward_kernel<true><<<grid, kLossThreads, 0, s>>>(x, y, W, H, make_window(), (float)(-lambda * inv), maps, partials);
   return cudaGetLastError();
+}
+
+cudaError_t launch_ssim_value(const float* x, const float* y, int W, int H, double* partials, cudaStream_t s) {
+  const dim3 grid((W + LT - 1) / LT, (H + LT - 1) / LT, 3);
+  note_launches(1);
+  return launch_pdl(ssim_forward_kernel<false>, grid, kLossThreads, 0, s, x, y, W, H, make_window(), 0.f,
+                    static_cast<float*>(nullptr), partials);
 }
 
 cudaError_t launch_ssim_grad_appearance(const float* x, const float* y, const float* maps, int W, int H,
@@ -472,7 +486,7 @@ extern "C" vg_status vg_loss_l1_dssim(const float* img, const float* target, int
   const Win win = make_window();
   note_launches(out_grad ? 3 : 2);
   // the call's first kernel follows whatever the caller queued on s: a plain launch
-  ssim_forward_kernel<<<grid, kLossThreads, 0, s>>>(img, target, width, height, win, (float)(-lambda * inv), maps, partials);
+  ssim_forward_kernel<true><<<grid, kLossThreads, 0, s>>>(img, target, width, height, win, (float)(-lambda * inv), maps, partials);
   cudaEvent_t fork = nullptr, join = nullptr;
   cudaError_t e = finalize_beside(partials, nb, inv, lambda, out_loss, out_grad != nullptr, s, &fork, &join);
   if (out_grad)
@@ -578,7 +592,7 @@ extern "C" vg_status vg_loss_l1_dssim_noalloc(const float* img, const float* tar
   note_launches(out_grad ? 3 : 2);
   // every map entry and partial these kernels read is written earlier in the same call, so the
   // scratch needs no clearing between calls
-  ssim_forward_kernel<<<grid, kLossThreads, 0, s>>>(img, target, width, height, win, (float)(-lambda * inv), maps, partials);
+  ssim_forward_kernel<true><<<grid, kLossThreads, 0, s>>>(img, target, width, height, win, (float)(-lambda * inv), maps, partials);
   loss_finalize<<<1, 1024, 0, s>>>(partials, nb, inv, lambda, out_loss);
   if (out_grad)
     ssim_backward_kernel<false><<<grid, kLossThreads, 0, s>>>(img, target, maps, width, height, win, (float)((1.0 - lambda) * inv), out_grad);
