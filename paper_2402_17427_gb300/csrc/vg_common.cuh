@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "vgrast.h"
@@ -183,6 +185,63 @@ __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long lon
 
 __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Decoupled look-back of ticketed block `blk` whose own count is `tot`, by one whole warp: publishes
+// the block's status word and returns the sum of the counts of all blocks before it (every lane).
+// Blocks only wait on blocks of smaller tickets, which are already running; each wait is bounded by
+// a second, after which bit 0 of *timeout is set (before this block's prefix is published).
+__device__ __forceinline__ unsigned lookback(unsigned long long* status, unsigned blk, unsigned tot,
+                                             unsigned* timeout) {
+  const int lane = threadIdx.x & 31;
+  unsigned excl = 0;
+  if (lane == 0) st_relaxed(status + blk, (blk == 0 ? kFlagPrefix : kFlagAggregate) | tot);
+  if (blk == 0) return 0;
+  long long p = (long long)blk - 1;
+  const uint64_t start = global_timer_ns();
+  for (;;) {
+    const unsigned long long v = p - lane >= 0 ? ld_relaxed(status + (p - lane)) : kFlagPrefix;
+    const unsigned pre = __ballot_sync(0xffffffffu, (v & kFlagPrefix) != 0);
+    const unsigned nr = __ballot_sync(0xffffffffu, (v & (kFlagPrefix | kFlagAggregate)) == 0);
+    const int first_pre = pre ? __ffs(pre) - 1 : 32, first_nr = nr ? __ffs(nr) - 1 : 32;
+    const bool done = first_pre < first_nr;
+    const int take = done ? first_pre + 1 : first_nr;
+    unsigned part = lane < take ? (unsigned)(v & kCountMask) : 0u;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    excl += part;
+    if (done) break;
+    p -= take;
+    if (take == 0 && global_timer_ns() - start > 1000000000ull) {   // a predecessor never published
+      if (lane == 0) {
+        atomicOr(timeout, 1u);
+        __threadfence();      // the flag is visible before this block's prefix is
+      }
+      break;
+    }
+  }
+  if (lane == 0) st_relaxed(status + blk, kFlagPrefix | (excl + tot));
+  return excl;
+}
+
+// Copies `rows` rows of W floats to consecutive rows of dst, row r from src(r) (null: zeros; skip(r):
+// left alone), by the whole block: consecutive threads take consecutive words of the output, so the
+// stores are coalesced whatever rows they come from and a row is read in one run.  VEC: 16-byte
+// words (W a multiple of 4, rows on 16-byte boundaries).
+template <int W, bool VEC, typename Src, typename Skip>
+__device__ __forceinline__ void copy_rows(float* __restrict__ dst, int rows, Src src, Skip skip) {
+  constexpr int U = VEC ? W / 4 : W;
+  using T = typename std::conditional<VEC, float4, float>::type;
+  T* d = reinterpret_cast<T*>(dst);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < rows * U; i += blockDim.x) {
+    const int r = i / U, c = i % U;
+    if (skip(r)) continue;
+    const float* s = src(r);
+    T v{};
+    if (s) v = __ldg(reinterpret_cast<const T*>(s) + c);
+    d[i] = v;
+  }
 }
 
 }  // namespace vg
