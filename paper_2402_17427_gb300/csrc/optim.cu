@@ -128,77 +128,51 @@ __device__ __forceinline__ int decide(const DensIn& in, long long i, float ls[3]
   return max3(ls) > in.tdense ? 3 : 2;
 }
 
-template <int F>
-__device__ void copy_gaussian(const vg_gaussians& src, long long i, const vg_param_ptrs& dst, long long o, bool zero) {
-  for (int a = 0; a < 3; ++a) {
-    dst.means[3 * o + a] = zero ? 0.f : __ldg(src.means + 3 * i + a);
-    dst.log_scales[3 * o + a] = zero ? 0.f : __ldg(src.log_scales + 3 * i + a);
-  }
-  reinterpret_cast<float4*>(dst.quats)[o] =
-      zero ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(reinterpret_cast<const float4*>(src.quats) + i);
-  dst.opacity_logits[o] = zero ? 0.f : __ldg(src.opacity_logits + i);
-  if constexpr (F % 4 == 0) {   // 16-byte rows (checked on the host for degrees 1 and 3)
-    const float4* sv = reinterpret_cast<const float4*>(src.sh + i * F);
-    float4* dv = reinterpret_cast<float4*>(dst.sh + o * F);
-#pragma unroll
-    for (int w = 0; w < F / 4; ++w) dv[w] = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(sv + w);
-  } else {
-    for (int w = 0; w < F; ++w) dst.sh[o * F + w] = zero ? 0.f : __ldg(src.sh + i * F + w);
-  }
-}
-
+// Bound by HBM: the decision inputs of every Gaussian, and 3 x 236 bytes (parameters and two moments,
+// degree 3) read of every Gaussian kept and written of every one emitted.  A block lists what it
+// emits in shared memory and copies the rows together (copy_rows); one thread copying the rows of
+// its own Gaussian took 457 us for 1M Gaussians (0.5 of the measured HBM rate), its 16-byte stores
+// 192 bytes apart.  Two Gaussians a thread halve the blocks that look back one after another.
+constexpr int kDensItems = 2, kDensTile = 256 * kDensItems;
+constexpr unsigned kDensSplit = 1u << 31, kDensSecond = 1u << 30;   // flags beside a 30-bit index in the block
 template <int F>
 __global__ void __launch_bounds__(256) densify_kernel(const DensIn in, long long n, unsigned* ticket,
                                                       unsigned long long* status, unsigned* timeout, const DensOut out) {
   __shared__ unsigned s_blk, s_base;
   __shared__ unsigned s_sm[8];
+  __shared__ unsigned s_row[2 * kDensTile];   // each emitted Gaussian: index in the block's input, flags
   if (threadIdx.x == 0) s_blk = atomicAdd(ticket, 1u);
   __syncthreads();
   const unsigned blk = s_blk;
-  const long long i = (long long)blk * blockDim.x + threadIdx.x;
-  int act = 0;
-  float ls[3] = {0.f, 0.f, 0.f};
-  unsigned emit = 0;
-  if (i < n) {
-    act = decide(in, i, ls);
-    const bool fits = !(max3(ls) > in.tmax);
-    const float lc[3] = {ls[0] - kLn16, ls[1] - kLn16, ls[2] - kLn16};
-    const bool child_fits = !(max3(lc) > in.tmax);
-    emit = act == 1 ? (fits ? 1u : 0u) : act == 2 ? (fits ? 2u : 0u) : act == 3 ? (child_fits ? 2u : 0u) : 0u;
+  const long long first = (long long)blk * kDensTile;
+  unsigned code[kDensItems], emits[kDensItems], mine = 0;
+#pragma unroll
+  for (int j = 0; j < kDensItems; ++j) {      // consecutive Gaussians, so that one scan gives the output order
+    const unsigned local = threadIdx.x * kDensItems + j;
+    const long long i = first + local;
+    code[j] = local;
+    emits[j] = 0;
+    if (i < n) {
+      float ls[3];
+      const int act = decide(in, i, ls);
+      const bool fits = !(max3(ls) > in.tmax);
+      const float lc[3] = {ls[0] - kLn16, ls[1] - kLn16, ls[2] - kLn16};
+      const bool child_fits = !(max3(lc) > in.tmax);
+      emits[j] = act == 1 ? (fits ? 1u : 0u) : act == 2 ? (fits ? 2u : 0u) : act == 3 ? (child_fits ? 2u : 0u) : 0u;
+      if (act == 3) code[j] |= kDensSplit;
+    }
+    mine += emits[j];
   }
   unsigned tot;
-  const unsigned ex = block_exclusive_scan(emit, &tot, s_sm);
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    unsigned excl = 0;
-    if (lane == 0) st_relaxed(status + blk, (blk == 0 ? kFlagPrefix : kFlagAggregate) | tot);
-    if (blk > 0) {
-      long long p = (long long)blk - 1;
-      const uint64_t start = global_timer_ns();
-      for (;;) {
-        const unsigned long long v = p - lane >= 0 ? ld_relaxed(status + (p - lane)) : kFlagPrefix;
-        const unsigned pre = __ballot_sync(0xffffffffu, (v & kFlagPrefix) != 0);
-        const unsigned nr = __ballot_sync(0xffffffffu, (v & (kFlagPrefix | kFlagAggregate)) == 0);
-        const int first_pre = pre ? __ffs(pre) - 1 : 32, first_nr = nr ? __ffs(nr) - 1 : 32;
-        const bool done = first_pre < first_nr;
-        const int take = done ? first_pre + 1 : first_nr;
-        unsigned part = lane < take ? (unsigned)(v & kCountMask) : 0u;
+  unsigned at = block_exclusive_scan(mine, &tot, s_sm);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        excl += part;
-        if (done) break;
-        p -= take;
-        if (take == 0 && global_timer_ns() - start > 1000000000ull) {   // a predecessor never published
-          if (lane == 0) {
-            atomicOr(timeout, 1u);
-            __threadfence();
-          }
-          break;
-        }
-      }
-      if (lane == 0) st_relaxed(status + blk, kFlagPrefix | (excl + tot));
-    }
-    if (lane == 0) {
+  for (int j = 0; j < kDensItems; ++j) {
+    if (emits[j] > 0) s_row[at++] = code[j];
+    if (emits[j] > 1) s_row[at++] = code[j] | kDensSecond;
+  }
+  if (threadIdx.x < 32) {
+    const unsigned excl = lookback(status, blk, tot, timeout);
+    if (threadIdx.x == 0) {
       s_base = excl;
       if (blk == gridDim.x - 1) {
         __threadfence();
@@ -207,33 +181,53 @@ __global__ void __launch_bounds__(256) densify_kernel(const DensIn in, long long
     }
   }
   __syncthreads();
-  if (emit == 0) return;
-  const long long o = (long long)s_base + ex;
-  if (act == 1 || act == 2) {
-    copy_gaussian<F>(in.p, i, out.p, o, false);
-    copy_gaussian<F>(in.m, i, out.m, o, false);
-    copy_gaussian<F>(in.v, i, out.v, o, false);
-    if (act == 2) {
-      copy_gaussian<F>(in.p, i, out.p, o + 1, false);
-      copy_gaussian<F>(in.m, i, out.m, o + 1, true);
-      copy_gaussian<F>(in.v, i, out.v, o + 1, true);
-    }
-    return;
-  }
+  const size_t o = s_base;
+  const int rows = (int)tot;
+  auto local_of = [&](int r) { return s_row[r] & (kDensSecond - 1u); };
+  auto none = [](int) { return false; };
+  auto is_split = [&](int r) { return (s_row[r] & kDensSplit) != 0; };
+  // a parameter row comes from its Gaussian; a moment row too, but is zero for a clone's copy and
+  // for the children of a split
+  auto param = [&](const float* a, int w) {
+    return [=](int r) { return a + (size_t)(first + local_of(r)) * w; };
+  };
+  auto moment = [&](const float* a, int w) {
+    return [=](int r) {
+      const unsigned c = s_row[r];
+      return (c & (kDensSplit | kDensSecond)) ? nullptr : a + (size_t)(first + (c & (kDensSecond - 1u))) * w;
+    };
+  };
+  constexpr bool V = F % 4 == 0;     // 16-byte SH rows (checked on the host for degrees 1 and 3)
+  copy_rows<F, V>(out.p.sh + o * F, rows, param(in.p.sh, F), none);
+  copy_rows<F, V>(out.m.sh + o * F, rows, moment(in.m.sh, F), none);
+  copy_rows<F, V>(out.v.sh + o * F, rows, moment(in.v.sh, F), none);
+  copy_rows<4, true>(out.p.quats + o * 4, rows, param(in.p.quats, 4), none);
+  copy_rows<4, true>(out.m.quats + o * 4, rows, moment(in.m.quats, 4), none);
+  copy_rows<4, true>(out.v.quats + o * 4, rows, moment(in.v.quats, 4), none);
+  copy_rows<3, false>(out.p.means + o * 3, rows, param(in.p.means, 3), is_split);
+  copy_rows<3, false>(out.m.means + o * 3, rows, moment(in.m.means, 3), none);
+  copy_rows<3, false>(out.v.means + o * 3, rows, moment(in.v.means, 3), none);
+  copy_rows<3, false>(out.p.log_scales + o * 3, rows, param(in.p.log_scales, 3), is_split);
+  copy_rows<3, false>(out.m.log_scales + o * 3, rows, moment(in.m.log_scales, 3), none);
+  copy_rows<3, false>(out.v.log_scales + o * 3, rows, moment(in.v.log_scales, 3), none);
+  copy_rows<1, false>(out.p.opacity_logits + o, rows, param(in.p.opacity_logits, 1), none);
+  copy_rows<1, false>(out.m.opacity_logits + o, rows, moment(in.m.opacity_logits, 1), none);
+  copy_rows<1, false>(out.v.opacity_logits + o, rows, moment(in.v.opacity_logits, 1), none);
   // split: two children, mean mu + R(q) (s * z_j), log-scale - ln 1.6
-  const float4 q = __ldg(reinterpret_cast<const float4*>(in.p.quats) + i);
-  const float qi = rsqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
-  const float w = q.x * qi, x = q.y * qi, y = q.z * qi, z = q.w * qi;
-  const float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y),
-                      2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
-                      2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)};
-  const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
-  for (int j = 0; j < 2; ++j) {
-    const long long oj = o + j;
-    copy_gaussian<F>(in.p, i, out.p, oj, false);
-    copy_gaussian<F>(in.m, i, out.m, oj, true);
-    copy_gaussian<F>(in.v, i, out.v, oj, true);
-    const float* zz = in.normals + (6 * i + 3 * j);
+  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+    if (!is_split(r)) continue;
+    const long long i = first + local_of(r);
+    const size_t oj = o + r;
+    const float4 q = __ldg(reinterpret_cast<const float4*>(in.p.quats) + i);
+    const float qi = rsqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
+    const float w = q.x * qi, x = q.y * qi, y = q.z * qi, z = q.w * qi;
+    const float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y),
+                        2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
+                        2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)};
+    const float ls[3] = {__ldg(in.p.log_scales + 3 * i), __ldg(in.p.log_scales + 3 * i + 1),
+                         __ldg(in.p.log_scales + 3 * i + 2)};
+    const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
+    const float* zz = in.normals + (6 * i + (s_row[r] & kDensSecond ? 3 : 0));
     const float d[3] = {s[0] * __ldg(zz), s[1] * __ldg(zz + 1), s[2] * __ldg(zz + 2)};
     for (int a = 0; a < 3; ++a) {
       out.p.means[3 * oj + a] = __ldg(in.p.means + 3 * i + a) + (R[3 * a] * d[0] + R[3 * a + 1] * d[1] + R[3 * a + 2] * d[2]);
@@ -262,7 +256,7 @@ DensLayout dens_layout(long long n) {
   size_t o = 0;
   auto take = [&](size_t b) { size_t at = o; o = align_up(o + b); return at; };
   L.ticket = take(2 * sizeof(unsigned));
-  L.status = take(sizeof(unsigned long long) * (size_t)((n + 255) / 256 + 1));
+  L.status = take(sizeof(unsigned long long) * (size_t)((n + kDensTile - 1) / kDensTile + 1));
   L.total = o;
   return L;
 }
@@ -362,7 +356,7 @@ extern "C" vg_status vg_densify(const vg_gaussians* in, const vg_gaussians* m_in
            (float)std::log((double)opts->min_opacity / (1.0 - (double)opts->min_opacity)),
            (float)std::log((double)opts->max_world_scale)};
   char* ws = static_cast<char*>(workspace);
-  const unsigned blocks = (unsigned)((n + 255) / 256);
+  const unsigned blocks = (unsigned)((n + kDensTile - 1) / kDensTile);
   if (cudaMemsetAsync(ws + L.ticket, 0, 2 * sizeof(unsigned), s) != cudaSuccess ||
       cudaMemsetAsync(ws + L.status, 0, sizeof(unsigned long long) * blocks, s) != cudaSuccess)
     return VG_ERR_CUDA;
