@@ -47,25 +47,25 @@ __global__ void publish_counters(const WsHeader* hdr, int64_t* c) {
   c[VG_CNT_EVALS_RUN_BWD] = (int64_t)hdr->evals_run_bwd;
 }
 
+// Lists, records and touch counts by Gaussian id, from the slots (positions among the visible
+// Gaussians, in index order) that the workspace keeps them by.  `proj` starts cleared.
 __global__ void read_state(const uint32_t* __restrict__ lists, const Splat* __restrict__ splats,
                            const uint32_t* __restrict__ touched_in, const WsHeader* __restrict__ hdr, int n,
-                           const uint32_t* d0, const uint32_t* d1, uint32_t* __restrict__ ids,
-                           float* __restrict__ proj, uint32_t* __restrict__ touched) {
-  const unsigned np = render_dead(hdr) ? 0u : hdr->pair_n;   // lists of a render that gave up are not read
+                           const uint32_t* d0, const uint32_t* d1, const uint32_t* __restrict__ vis_ids,
+                           uint32_t* __restrict__ ids, float* __restrict__ proj, uint32_t* __restrict__ touched) {
+  const bool dead = render_dead(hdr);                // lists of a render that gave up are not read
+  const unsigned np = dead ? 0u : hdr->pair_n, nv = dead ? 0u : hdr->visible;
   const uint32_t* dorder = depth_order(hdr, d0, d1);
   const float k = -1.3862943611198906f;   // scaled conic -> inverse covariance
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < np || i < (unsigned)n; i += gridDim.x * blockDim.x) {
-    if (ids && i < np) ids[i] = dorder[lists[i]];
-    if (i < (unsigned)n) {
-      if (touched) touched[i] = touched_in[i];
-      if (proj) {
-        const Splat s = splats[i];
-        const bool vis = touched_in[i] > 0;
-        const float ulo = __half2float(__ushort_as_half((unsigned short)(s.uvlo & 0xFFFFu)));
-        const float vlo = __half2float(__ushort_as_half((unsigned short)(s.uvlo >> 16)));
-        float v[12] = {s.u, s.v, s.ca * k, s.cb * 0.5f * k, s.cc * k, exp2f(s.lo), s.r, s.g, s.b, (float)s.rank, ulo, vlo};
-        for (int f = 0; f < 12; ++f) proj[(size_t)i * 12 + f] = vis ? v[f] : 0.f;
-      }
+    if (ids && i < np) ids[i] = vis_ids[dorder[lists[i]]];
+    if (i < (unsigned)n && touched) touched[i] = touched_in[i];
+    if (i < nv && proj) {
+      const Splat s = splats[i];
+      const float ulo = __half2float(__ushort_as_half((unsigned short)(s.uvlo & 0xFFFFu)));
+      const float vlo = __half2float(__ushort_as_half((unsigned short)(s.uvlo >> 16)));
+      float v[12] = {s.u, s.v, s.ca * k, s.cb * 0.5f * k, s.cc * k, exp2f(s.lo), s.r, s.g, s.b, (float)s.rank, ulo, vlo};
+      for (int f = 0; f < 12; ++f) proj[(size_t)vis_ids[i] * 12 + f] = v[f];
     }
   }
 }
@@ -640,12 +640,15 @@ extern "C" vg_status vg_read_render_state(const void* workspace, size_t workspac
   const char* ws = static_cast<const char*>(workspace);
   if (ranges && cudaMemcpyAsync(ranges, ws + L.ranges, (size_t)tiles * 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return VG_ERR_CUDA;
+  if (projected && n > 0 && cudaMemsetAsync(projected, 0, (size_t)n * 12 * sizeof(float), s) != cudaSuccess)
+    return VG_ERR_CUDA;
   note_launches(1);
   read_state<<<1024, 256, 0, s>>>(reinterpret_cast<const uint32_t*>(ws + L.pvals[0]), reinterpret_cast<const Splat*>(ws + L.splats),
                                   reinterpret_cast<const uint32_t*>(ws + L.touched),
                                   reinterpret_cast<const WsHeader*>(ws + L.header), (int)n,
                                   reinterpret_cast<const uint32_t*>(ws + L.vvals[0]),
-                                  reinterpret_cast<const uint32_t*>(ws + L.vvals[1]), ids, projected, touched);
+                                  reinterpret_cast<const uint32_t*>(ws + L.vvals[1]),
+                                  reinterpret_cast<const uint32_t*>(ws + L.vis_ids), ids, projected, touched);
   return cuda_status(cudaGetLastError());
 }
 
@@ -666,12 +669,15 @@ extern "C" vg_status vg_read_batch_state(const void* workspace, size_t workspace
   const char* ws = static_cast<const char*>(workspace);
   if (ranges && cudaMemcpyAsync(ranges, ws + L.ranges, (size_t)c.total_tiles * 8, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return VG_ERR_CUDA;
+  if (projected && c.total_n > 0 && cudaMemsetAsync(projected, 0, (size_t)c.total_n * 12 * sizeof(float), s) != cudaSuccess)
+    return VG_ERR_CUDA;
   note_launches(1);
   read_state<<<1024, 256, 0, s>>>(reinterpret_cast<const uint32_t*>(ws + L.pvals[0]), reinterpret_cast<const Splat*>(ws + L.splats),
                                   reinterpret_cast<const uint32_t*>(ws + L.touched),
                                   reinterpret_cast<const WsHeader*>(ws + L.header), c.total_n,
                                   reinterpret_cast<const uint32_t*>(ws + L.vvals[0]),
-                                  reinterpret_cast<const uint32_t*>(ws + L.vvals[1]), ids, projected, touched);
+                                  reinterpret_cast<const uint32_t*>(ws + L.vvals[1]),
+                                  reinterpret_cast<const uint32_t*>(ws + L.vis_ids), ids, projected, touched);
   return cuda_status(cudaGetLastError());
 }
 

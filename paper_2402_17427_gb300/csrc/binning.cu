@@ -38,6 +38,12 @@ __device__ __forceinline__ void segment(unsigned n, unsigned& begin, unsigned& e
   end = min(n, begin + seg);
 }
 
+// View of the visible Gaussian in slot `slot` (the Gaussian's id is read only where views differ).
+__device__ __forceinline__ int slot_view(const DevTables* __restrict__ tab, const uint32_t* __restrict__ vis_ids,
+                                         unsigned slot) {
+  return tab->h.n_views == 1 ? 0 : tseg(tab, find_seg(tab, (int)vis_ids[slot])).view;
+}
+
 // ---- look-back sort helpers ------------------------------------------------------------------
 
 constexpr int kLookback = 8;                                 // status rows read per look-back step
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_pass(
 // themselves evenly over its blocks, so that the nearest (largest) Gaussians, which the depth
 // order puts together, do not serialise one block.
 __global__ void __launch_bounds__(256) pairs_count(const DevTables* __restrict__ tab, const uint32_t* order0,
-                                                   const uint32_t* order1, const uint32_t* __restrict__ touched,
+                                                   const uint32_t* order1, const uint32_t* __restrict__ vis_ids,
                                                    const uint2* __restrict__ rects, const WsHeader* __restrict__ hdr,
                                                    unsigned long long* __restrict__ blocksums,
                                                    Splat* __restrict__ splats, Splat* __restrict__ vsplats,
@@ -236,18 +242,18 @@ __global__ void __launch_bounds__(256) pairs_count(const DevTables* __restrict__
     const unsigned s = t0 + threadIdx.x;
     uint32_t cnt = 0;
     if (s < end) {
-      const uint32_t id = order[s];
-      cnt = touched[id];
+      const uint32_t slot = order[s];
       // the record in depth order (what the blend kernels gather), carrying its rank
-      const float4* src = reinterpret_cast<const float4*>(splats + id);
+      const float4* src = reinterpret_cast<const float4*>(splats + slot);
       float4 r0 = src[0], r1 = src[1], r2 = src[2];
       r2.y = __uint_as_float(s);
       float4* dst = reinterpret_cast<float4*>(vsplats + s);
       dst[0] = r0; dst[1] = r1; dst[2] = r2;
-      splats[id].rank = s;
-      const KView& vw = tview(tab, tseg(tab, find_seg(tab, (int)id)).view);
-      const uint2 rc = rects[id];
+      splats[slot].rank = s;
+      const KView& vw = tview(tab, slot_view(tab, vis_ids, slot));
+      const uint2 rc = rects[slot];
       const unsigned tx0 = rc.x & 0xFFFFu, ty0 = rc.y & 0xFFFFu, w = (rc.x >> 16) - tx0 + 1u;
+      cnt = w * ((rc.y >> 16) - ty0 + 1u);
       first_key[s] = (uint32_t)vw.tile_base + ty0 * (uint32_t)vw.tiles_x + tx0;
       shape[s] = w | ((uint32_t)vw.tiles_x << 16);   // both below 2^16 (width <= 16384 pixels)
     }
@@ -485,7 +491,7 @@ __global__ void __launch_bounds__(256) order_scatter(const DevTables* __restrict
 // atomics on the words many rectangles share.
 constexpr int kCountCopies = 8;
 __global__ void __launch_bounds__(256) tile_count(const DevTables* __restrict__ tab, const uint32_t* __restrict__ vis_ids,
-                                                  const uint32_t* __restrict__ touched, const uint2* __restrict__ rects,
+                                                  const uint2* __restrict__ rects,
                                                   const WsHeader* __restrict__ hdr, unsigned* __restrict__ tdiff,
                                                   int tiles) {
   pdl_enter();
@@ -499,14 +505,11 @@ __global__ void __launch_bounds__(256) tile_count(const DevTables* __restrict__ 
     const unsigned t = t0 + threadIdx.x;
     int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1, base = 0, txn = 0;
     if (t < nv) {
-      const uint32_t id = vis_ids[t];
-      if (touched[id]) {
-        const KView& vw = tview(tab, tseg(tab, find_seg(tab, (int)id)).view);
-        const uint2 rc = rects[id];
-        tx0 = (int)(rc.x & 0xFFFF); tx1 = (int)(rc.x >> 16);
-        ty0 = (int)(rc.y & 0xFFFF); ty1 = (int)(rc.y >> 16);
-        base = vw.tile_base; txn = vw.tiles_x;
-      }
+      const KView& vw = tview(tab, slot_view(tab, vis_ids, t));
+      const uint2 rc = rects[t];
+      tx0 = (int)(rc.x & 0xFFFF); tx1 = (int)(rc.x >> 16);
+      ty0 = (int)(rc.y & 0xFFFF); ty1 = (int)(rc.y >> 16);
+      base = vw.tile_base; txn = vw.tiles_x;
     }
     for (int r = 0;; ++r) {
       const bool act = ty0 + r <= ty1;
@@ -817,7 +820,7 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
       if (known) opted_ctx[dev] = ctx;
     }
     cudaMemsetAsync(tdiff, 0, (size_t)kCountCopies * tiles * sizeof(unsigned), side);
-    tile_count<<<2 * std::max(1, sort_blocks()), 256, 0, side>>>(tab, U(L.vis_ids), U(L.touched), rects, hdr, tdiff,
+    tile_count<<<2 * std::max(1, sort_blocks()), 256, 0, side>>>(tab, U(L.vis_ids), rects, hdr, tdiff,
                                                                 tiles);
     tile_prep<<<1, kPrepThreads, smem, side>>>(tab, tiles, cap, tpasses, tdiff, ranges, ctl->hist[1][0], U(L.order));
     if (join) cudaEventRecord(join, side);
@@ -836,7 +839,7 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
   const int BP = kMaxSortBlocks < 6 * B / 2 ? kMaxSortBlocks : 6 * B / 2;   // 6 blocks per SM
   // per Gaussian in depth order: first tile key and rectangle shape in the depth keys' buffers,
   // free once the depth sort is done
-  launch_pdl(pairs_count, BP, 256, 0, s, tab, U(L.vvals[0]), U(L.vvals[1]), U(L.touched), rects, hdr, bsum64,
+  launch_pdl(pairs_count, BP, 256, 0, s, tab, U(L.vvals[0]), U(L.vvals[1]), U(L.vis_ids), rects, hdr, bsum64,
              splats, vsplats, U(L.vkeys[0]), U(L.vkeys[1]));
   launch_pdl(pairs_scan, 1, 256, 0, s, bsum64, BP, hdr, (unsigned long long)cap);
   launch_pdl(pairs_emit, 2 * B, 256, 0, s, U(L.vvals[0]), U(L.vvals[1]), hdr, bsum64, BP, U(L.vkeys[0]),

@@ -400,7 +400,8 @@ __global__ void __launch_bounds__(TileShape<TS, true>::kThreads, TS == 16 ? 16 :
 blend_backward_kernel(const DevTables* __restrict__ tab, const Splat* __restrict__ vsplats,
                       const uint32_t* __restrict__ lists, const uint2* __restrict__ ranges,
                       const uint32_t* __restrict__ order, int item_begin, int item_count, float* __restrict__ g2d,
-                      const uint32_t* dorder0, const uint32_t* dorder1, WsHeader* __restrict__ hdr) {
+                      const uint32_t* dorder0, const uint32_t* dorder1, const uint32_t* __restrict__ vis_ids,
+                      WsHeader* __restrict__ hdr) {
   pdl_enter();
   using S = TileShape<TS, true>;
   const uint32_t* __restrict__ dorder = depth_order(hdr, dorder0, dorder1);
@@ -648,7 +649,7 @@ blend_backward_kernel(const DevTables* __restrict__ tab, const Splat* __restrict
             const uint32_t rank = __float_as_uint(f2.y);
             if ((lane & 1) == 0 && field >= 0 && field < 9) red_add_f32(g2d + (size_t)rank * 9 + field, tot);
             if (ABS && (lane & 1) == 0 && field == 9) {
-              const int id = (int)dorder[rank];
+              const int id = (int)vis_ids[dorder[rank]];
               const KSeg& sg = tseg(tab, find_seg(tab, id));
               if (sg.gabs) red_add_f32(sg.gabs + (id - sg.offset), tot);
             }
@@ -709,26 +710,26 @@ cudaError_t fwd_class(const DevTables* tab, const HostPlan& plan, const Splat* v
 template <int TS, bool ABS, bool COUNT>
 void bwd_launch(const DevTables* tab, const Splat* vsplats, const uint32_t* lists, const uint2* ranges,
                 const uint32_t* order, int begin, int items, float* g2d, const uint32_t* d0, const uint32_t* d1,
-                WsHeader* hdr, cudaStream_t s) {
+                const uint32_t* vis_ids, WsHeader* hdr, cudaStream_t s) {
   using S = TileShape<TS, true>;
   auto k = blend_backward_kernel<TS, ABS, COUNT>;
   launch_pdl(k, resident_grid(k, S::kThreads, items), S::kThreads, 0, s, tab, vsplats, lists, ranges, order, begin, items, g2d,
-                                                                 d0, d1, hdr);
+                                                                 d0, d1, vis_ids, hdr);
 }
 
 template <int TS>
 cudaError_t bwd_class(const DevTables* tab, const HostPlan& plan, const Splat* vsplats, const uint32_t* lists,
                       const uint2* ranges, const uint32_t* order, float* g2d, const uint32_t* d0, const uint32_t* d1,
-                      WsHeader* hdr, bool abs, bool count, cudaStream_t s) {
+                      const uint32_t* vis_ids, WsHeader* hdr, bool abs, bool count, cudaStream_t s) {
   using S = TileShape<TS, true>;
   const int items = plan.class_tiles[S::kClass];
   if (items == 0) return cudaSuccess;
   note_launches(1);
   const int begin = plan.class_begin[S::kClass];
-  if (abs && count) bwd_launch<TS, true, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, hdr, s);
-  else if (abs) bwd_launch<TS, true, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, hdr, s);
-  else if (count) bwd_launch<TS, false, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, hdr, s);
-  else bwd_launch<TS, false, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, hdr, s);
+  if (abs && count) bwd_launch<TS, true, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
+  else if (abs) bwd_launch<TS, true, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
+  else if (count) bwd_launch<TS, false, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
+  else bwd_launch<TS, false, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
   return cudaGetLastError();
 }
 
@@ -759,9 +760,10 @@ cudaError_t launch_blend_backward(const DevTables* tab, const HostPlan& plan, co
   note_launches(1);
   const uint32_t* d0 = reinterpret_cast<const uint32_t*>(ws + L.vvals[0]);
   const uint32_t* d1 = reinterpret_cast<const uint32_t*>(ws + L.vvals[1]);
-  cudaError_t e = bwd_class<8>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, hdr, abs, count, s);
-  if (e == cudaSuccess) e = bwd_class<16>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, hdr, abs, count, s);
-  if (e == cudaSuccess) e = bwd_class<32>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, hdr, abs, count, s);
+  const uint32_t* vis_ids = reinterpret_cast<const uint32_t*>(ws + L.vis_ids);
+  cudaError_t e = bwd_class<8>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, s);
+  if (e == cudaSuccess) e = bwd_class<16>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, s);
+  if (e == cudaSuccess) e = bwd_class<32>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, s);
   return e;
 }
 

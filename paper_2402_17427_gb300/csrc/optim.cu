@@ -81,12 +81,13 @@ __global__ void __launch_bounds__(256) adam_kernel(const AdamArgs a) {
 
 __global__ void __launch_bounds__(256) accumulate_kernel(const float* __restrict__ g2d, const Splat* __restrict__ vsplats,
                                                          const WsHeader* __restrict__ hdr,
-                                                         const uint32_t* d0, const uint32_t* d1, float hw, float hh,
+                                                         const uint32_t* d0, const uint32_t* d1,
+                                                         const uint32_t* __restrict__ vis_ids, float hw, float hh,
                                                          float* __restrict__ accum, int* __restrict__ count) {
   const uint32_t* __restrict__ dorder = depth_order(hdr, d0, d1);
   const unsigned V = hdr->visible;
   for (unsigned s = blockIdx.x * blockDim.x + threadIdx.x; s < V; s += gridDim.x * blockDim.x) {
-    const unsigned id = dorder[s];
+    const unsigned id = vis_ids[dorder[s]];
     // the 2D gradient from the compositing adjoint's power moments (slots 0-5), by depth rank
     float mom[6], d2[6];
 #pragma unroll
@@ -318,7 +319,7 @@ extern "C" vg_status vg_densify_accumulate(const void* workspace, size_t workspa
   accumulate_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 4096), 256, 0, s>>>(
       reinterpret_cast<const float*>(ws + L.g2d), reinterpret_cast<const Splat*>(ws + L.vsplats),
       reinterpret_cast<const WsHeader*>(ws + L.header), reinterpret_cast<const uint32_t*>(ws + L.vvals[0]), reinterpret_cast<const uint32_t*>(ws + L.vvals[1]),
-      0.5f * (float)width, 0.5f * (float)height, accum, reinterpret_cast<int*>(count));
+      reinterpret_cast<const uint32_t*>(ws + L.vis_ids), 0.5f * (float)width, 0.5f * (float)height, accum, reinterpret_cast<int*>(count));
   note_launches(1);
   return cudaGetLastError() == cudaSuccess ? VG_OK : VG_ERR_CUDA;
 }

@@ -240,98 +240,233 @@ __device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const K
   P.valid = true;
 }
 
-// 256 threads a block (the shared arrays below are sized for it), held to 48 registers so that
-// 5 blocks share an SM: the kernel is latency-bound (1M Gaussians at 1080p: 79 -> 77 us).
-template <int DEG>
-__global__ void __launch_bounds__(256, 5) preprocess_kernel(const DevTables* __restrict__ tab, int total_n,
-                                                         Splat* __restrict__ splats, uint2* __restrict__ rects,
-                                                         uint32_t* __restrict__ touched, const Compact cp,
-                                                         WsHeader* __restrict__ hdr) {
+// Whether Gaussian i may touch the image, from its mean and its largest scale alone: false only if
+// project() and the rectangle rule would cull it.  lambda_max(T Sigma T^T) <= |T|_F^2 max(s)^2 bounds the
+// radius; the margins (1e-3 relative, 0.01 px + 1e-6 |u|) are far above the rounding of either side.
+// Comparisons are written so that a NaN or an infinity passes on to project().
+__device__ __forceinline__ bool may_touch(const KGauss& g, const KCam& cm, const KOpts& op, int i, const float* m) {
+  float p[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+    p[r] = __fmaf_rn(cm.R[3 * r], m[0], __fmaf_rn(cm.R[3 * r + 1], m[1], __fmaf_rn(cm.R[3 * r + 2], m[2], cm.t[r])));
+  const float z = p[2];
+  if (!(z > cm.near_plane)) return false;
+  const float smax = expf(fmaxf(fmaxf(__ldg(g.log_scales + 3 * i), __ldg(g.log_scales + 3 * i + 1)),
+                                __ldg(g.log_scales + 3 * i + 2)));
+  const float xz = __fdiv_rn(p[0], z), yz = __fdiv_rn(p[1], z);
+  const float u = __fmaf_rn(cm.fx, xz, cm.cx), v = __fmaf_rn(cm.fy, yz, cm.cy);
+  const float xzc = fminf(cm.limx, fmaxf(-cm.limx, xz)), yzc = fminf(cm.limy, fmaxf(-cm.limy, yz));
+  const float iz = 1.f / z;
+  const float j00 = cm.fx * iz, j02 = -cm.fx * xzc * iz, j11 = cm.fy * iz, j12 = -cm.fy * yzc * iz;
+  float f2 = 0.f;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float a = j00 * cm.R[c] + j02 * cm.R[6 + c], b = j11 * cm.R[3 + c] + j12 * cm.R[6 + c];
+    f2 = fmaf(a, a, fmaf(b, b, f2));
+  }
+  const float rb = 3.003f * sqrtf(fmaf(1.001f * f2, smax * smax, op.dilation)) + 0.01f;
+  const float ru = fmaf(1e-6f, fabsf(u), rb), rv = fmaf(1e-6f, fabsf(v), rb);
+  return !(u + ru < 0.f || u - ru > (float)(cm.W - 1) || v + rv < 0.f || v - rv > (float)(cm.H - 1));
+}
+
+// Projection, first half: the visible Gaussians, compacted in index order (slot = position in that
+// order), with their depth keys and tile rectangles.
+//
+// A block takes 512 Gaussians in ticket order (so the look-back only waits on running blocks), four
+// a thread with their loads in flight together.  Only ~1 in 5 is visible (1 in 25 in the 20M-Gaussian
+// city), in no order, so may_touch() first thins them out on 24 bytes a Gaussian, the candidates are packed
+// densely in shared memory, and whole warps of them go through project().  The colours and records, which need
+// no order, are left to record_kernel over the dense list of visible Gaussians: with the spherical
+// harmonics in this kernel its blocks waited at their barriers for a few busy warps and for the
+// look-back (one Gaussian a thread, 256 a block: 58 us for 1M Gaussians and 963 us for 20M).
+constexpr int kCullThreads = 128, kCullItems = 4, kCullTile = kCullThreads * kCullItems, kCullWarps = kCullThreads / 32;
+__global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* __restrict__ tab, int total_n,
+                                                                uint2* __restrict__ rects,
+                                                                uint32_t* __restrict__ touched, const Compact cp,
+                                                                WsHeader* __restrict__ hdr) {
   pdl_enter();
-  // blocks take their Gaussians in ticket order, so the look-back below only ever waits on
-  // blocks that are already running
   __shared__ unsigned s_blk, s_base;
-  __shared__ unsigned s_sm[8];
-  __shared__ unsigned s_dlo, s_dhi;   // the block's min / max depth key
+  __shared__ unsigned s_dlo, s_dhi;                      // the block's min / max depth key
+  __shared__ unsigned s_wc[2][kCullItems * kCullWarps];  // counts a warp (and item) leaves for the others
   __shared__ unsigned s_h[kMaxPasses][kRadix];
-  // the visible Gaussians' stage-3 inputs, packed densely in index order: Gaussian, segment,
-  // mean, conic, and the 2D covariance's diagonal
-  __shared__ float s_job[10][256];
-  if (threadIdx.x == 0) {
+  __shared__ uint16_t s_cand[kCullTile], s_local[kCullTile];
+  __shared__ unsigned s_key[kCullTile];
+  __shared__ uint2 s_rect[kCullTile];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) {
     s_blk = atomicAdd(cp.ticket, 1u);
     s_dlo = 0xFFFFFFFFu;
     s_dhi = 0u;
   }
-#pragma unroll
-  for (int p = 0; p < kMaxPasses; ++p) s_h[p][threadIdx.x] = 0;
+  for (int k = tid; k < kMaxPasses * kRadix; k += kCullThreads) s_h[k / kRadix][k % kRadix] = 0;
   __syncthreads();
   const unsigned blk = s_blk;
-  const int i = (int)(blk * blockDim.x + threadIdx.x);
-  uint32_t key = 0xFFFFFFFFu, lo_key = 0xFFFFFFFFu, hi_key = 0u;
-  // 1. projection, tile rectangle and visibility
-  int segi = 0;
-  Proj P;
-  P.valid = false;
-  bool vis = false;
-  if (i < total_n) {
-    segi = find_seg(tab, i);
-    const KSeg* sg = &tseg(tab, segi);
-    const KView& vw = tview(tab, sg->view);
-    const int li = i - sg->offset;
-    project(sg->g, vw.cam, vw.op, li, P);
-    uint32_t cnt = 0;
-    if (P.valid) {
-      const int T = vw.op.tile;
-      int xlo = rect_lo(P.u, P.r, vw.cam.W), xhi = rect_hi(P.u, P.r, vw.cam.W);
-      int ylo = rect_lo(P.v, P.r, vw.cam.H), yhi = rect_hi(P.v, P.r, vw.cam.H);
-      if (xlo <= xhi && ylo <= yhi) {
-        const int tx0 = xlo / T, tx1 = xhi / T, ty0 = ylo / T, ty1 = yhi / T;
-        cnt = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
-        rects[i] = make_uint2((uint32_t)tx0 | ((uint32_t)tx1 << 16), (uint32_t)ty0 | ((uint32_t)ty1 << 16));
-        vis = true;
-        key = __float_as_uint(P.depth);
-        lo_key = hi_key = key;
-      }
+  const int base = (int)(blk * kCullTile), last = min(total_n - 1, base + (kCullTile - 1));
+  const int seg0 = find_seg(tab, base);
+  const bool one = seg0 == tab->h.n_segs - 1 || tseg(tab, seg0 + 1).offset > last;   // one segment in this block
+  // 1. candidates: a mean each, all four requested together, then the largest scales
+  float m[kCullItems][3];
+#pragma unroll
+  for (int j = 0; j < kCullItems; ++j) {
+    const int i = base + j * kCullThreads + tid;
+    if (i <= last) {
+      const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
+      const float* q = sg.g.means + 3 * (size_t)(i - sg.offset);
+      m[j][0] = __ldg(q); m[j][1] = __ldg(q + 1); m[j][2] = __ldg(q + 2);
     }
-    touched[i] = cnt;
-    if (cp.key_inputs)
-      cp.key_inputs[i] = P.valid ? make_float4(P.u, P.v, P.r, P.depth) : make_float4(0.f, 0.f, -1.f, 0.f);
   }
-  // 2. the block's visible count, published before the heavy per-Gaussian work so that later
-  //    blocks rarely wait in their look-back
-  unsigned tot;
-  const unsigned ex = block_exclusive_scan((unsigned)vis, &tot, s_sm);
-  const bool publish = (int)blk != cp.stall_block;
-  if (threadIdx.x == 0 && publish) st_relaxed(cp.status + blk, (blk == 0 ? kFlagPrefix : kFlagAggregate) | tot);
-  // 3. the splat record: colour from spherical harmonics along the viewing direction, opacity,
-  //    the accurate blending position and the alpha >= alpha_min box.  Only ~1 in 5 Gaussians is
-  //    visible, so the visible ones are packed densely first: slot k is taken by thread 255 - k,
-  //    which leaves warp 0 free for the look-back below while the last warps do this stage.
-  if (vis) {
-    s_job[0][ex] = __int_as_float(i);
-    s_job[1][ex] = __int_as_float(segi);
-    s_job[2][ex] = P.m[0]; s_job[3][ex] = P.m[1]; s_job[4][ex] = P.m[2];
-    s_job[5][ex] = P.ca; s_job[6][ex] = P.cb; s_job[7][ex] = P.cc;
-    s_job[8][ex] = P.A; s_job[9][ex] = P.C;
+  unsigned votes[kCullItems];
+#pragma unroll
+  for (int j = 0; j < kCullItems; ++j) {
+    const int i = base + j * kCullThreads + tid;
+    bool c = false;
+    if (i <= last) {
+      const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
+      const KView& vw = tview(tab, sg.view);
+      c = cp.key_inputs != nullptr || may_touch(sg.g, vw.cam, vw.op, i - sg.offset, m[j]);
+      if (!c) touched[i] = 0;
+    }
+    votes[j] = __ballot_sync(0xffffffffu, c);
+    if (lane == 0) s_wc[0][j * kCullWarps + warp] = __popc(votes[j]);
   }
   __syncthreads();
-  const unsigned slot = blockDim.x - 1 - threadIdx.x;
-  if (slot < tot) {
-    const int i = __float_as_int(s_job[0][slot]);
-    const KSeg* sg = &tseg(tab, __float_as_int(s_job[1][slot]));
+  const uint32_t lt = lanemask_lt();
+  int ncand = 0;
+#pragma unroll
+  for (int k = 0; k < kCullItems * kCullWarps; ++k) {      // counts in index order: item, then warp
+    const int j = k / kCullWarps;
+    if (k % kCullWarps == warp && (votes[j] >> lane & 1u))
+      s_cand[ncand + __popc(votes[j] & lt)] = (uint16_t)(j * kCullThreads + tid);
+    ncand += (int)s_wc[0][k];
+  }
+  __syncthreads();
+  // 2. projection, tile rectangle and visibility of the candidates, the visible ones packed in order
+  unsigned tot = 0, lo_key = 0xFFFFFFFFu, hi_key = 0u;
+  for (int r = 0, odd = 1; r < ncand; r += kCullThreads, odd ^= 1) {
+    bool vis = false;
+    uint32_t key = 0;
+    uint2 rect = make_uint2(0u, 0u);
+    int local = 0;
+    if (r + tid < ncand) {
+      local = s_cand[r + tid];
+      const int i = base + local;
+      const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
+      const KView& vw = tview(tab, sg.view);
+      Proj P;
+      project(sg.g, vw.cam, vw.op, i - sg.offset, P);
+      uint32_t cnt = 0;
+      if (P.valid) {
+        const int T = vw.op.tile;
+        const int xlo = rect_lo(P.u, P.r, vw.cam.W), xhi = rect_hi(P.u, P.r, vw.cam.W);
+        const int ylo = rect_lo(P.v, P.r, vw.cam.H), yhi = rect_hi(P.v, P.r, vw.cam.H);
+        if (xlo <= xhi && ylo <= yhi) {
+          const int tx0 = xlo / T, tx1 = xhi / T, ty0 = ylo / T, ty1 = yhi / T;
+          cnt = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
+          rect = make_uint2((uint32_t)tx0 | ((uint32_t)tx1 << 16), (uint32_t)ty0 | ((uint32_t)ty1 << 16));
+          vis = true;
+          key = __float_as_uint(P.depth);
+          lo_key = min(lo_key, key);
+          hi_key = max(hi_key, key);
+        }
+      }
+      touched[i] = cnt;
+      if (cp.key_inputs)
+        cp.key_inputs[i] = P.valid ? make_float4(P.u, P.v, P.r, P.depth) : make_float4(0.f, 0.f, -1.f, 0.f);
+    }
+    const unsigned vote = __ballot_sync(0xffffffffu, vis);
+    if (lane == 0) s_wc[odd][warp] = __popc(vote);
+    __syncthreads();                      // the other buffer is written in the next round
+    unsigned at = tot + __popc(vote & lt);
+#pragma unroll
+    for (int w = 0; w < kCullWarps; ++w) {
+      const unsigned c = s_wc[odd][w];
+      if (w < warp) at += c;
+      tot += c;
+    }
+    if (vis) {
+      s_key[at] = key;
+      s_rect[at] = rect;
+      s_local[at] = (uint16_t)local;
+    }
+  }
+  // min / max depth key over visible Gaussians (they fix the bits the depth sort needs): per warp,
+  // then per block in shared memory, then one global atomic each per block (one per warp put
+  // ~31K same-address atomics per render on two words)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo_key = min(lo_key, __shfl_xor_sync(0xffffffffu, lo_key, o));
+    hi_key = max(hi_key, __shfl_xor_sync(0xffffffffu, hi_key, o));
+  }
+  if (lane == 0 && lo_key <= hi_key) {
+    atomicMin(&s_dlo, lo_key);
+    atomicMax(&s_dhi, hi_key);
+  }
+  __syncthreads();
+  // 3. the block's offset among all visible Gaussians (warp 0) beside the digit histograms (the others)
+  if (warp == 0) {
+    const unsigned excl = lookback(cp.status, blk, tot, &hdr->status, (unsigned)VG_STATUS_WAIT_TIMEOUT, cp.wait_ns,
+                                   (int)blk != cp.stall_block);
+    if (lane == 0) {
+      s_base = excl;
+      if (blk == gridDim.x - 1) hdr->visible = excl + tot;
+      if (s_dlo <= s_dhi) {
+        atomicMin(&hdr->dmin, s_dlo);
+        atomicMax(&hdr->dmax, s_dhi);
+      }
+    }
+  } else {
+    for (unsigned k = tid - 32; k < tot; k += kCullThreads - 32) {
+      const unsigned key = s_key[k];
+#pragma unroll
+      for (int p = 0; p < kMaxPasses; ++p) atomicAdd(&s_h[p][(key >> (p * kRadixBits)) & (kRadix - 1)], 1u);
+    }
+  }
+  __syncthreads();
+  for (unsigned k = tid; k < tot; k += kCullThreads) {
+    const unsigned at = s_base + k;
+    cp.vkeys[at] = s_key[k];
+    cp.vvals[at] = at;
+    cp.vis_ids[at] = (uint32_t)(base + s_local[k]);
+    rects[at] = s_rect[k];
+  }
+  if (tot > 0)
+    for (int k = tid; k < kMaxPasses * kRadix; k += kCullThreads) {
+      const unsigned c = s_h[k / kRadix][k % kRadix];
+      if (c) atomicAdd(&cp.hist[k], c);
+    }
+  // clear the look-back rows of the first depth-sort pass
+  for (size_t z = (size_t)blk * kCullThreads + tid; z < cp.zero_words; z += (size_t)gridDim.x * kCullThreads)
+    cp.zero[z] = 0ull;
+}
+
+// Projection, second half: the splat record of every visible Gaussian, by slot: colour from
+// spherical harmonics along the viewing direction, opacity, the accurate blending position and the
+// alpha >= alpha_min box.  Bound by the latency of the scattered parameter rows, with no barrier and
+// nothing to wait for, so it runs at whatever occupancy its registers leave.
+template <int DEG>
+__global__ void __launch_bounds__(128) record_kernel(const DevTables* __restrict__ tab,
+                                                     const uint32_t* __restrict__ vis_ids,
+                                                     const WsHeader* __restrict__ hdr, Splat* __restrict__ splats) {
+  pdl_enter();
+  const bool dead = render_dead(hdr);   // the compacted list may hold unwritten slots
+  const unsigned nv = hdr->visible;
+  if (dead) return;
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += gridDim.x * blockDim.x) {
+    const int i = (int)vis_ids[t];
+    const KSeg* sg = &tseg(tab, find_seg(tab, i));
     const int li = i - sg->offset;
-    P.m[0] = s_job[2][slot]; P.m[1] = s_job[3][slot]; P.m[2] = s_job[4][slot];
-    P.ca = s_job[5][slot]; P.cb = s_job[6][slot]; P.cc = s_job[7][slot];
-    P.A = s_job[8][slot]; P.C = s_job[9][slot];
     const KView& vw = tview(tab, sg->view);
     const KCam& cm = vw.cam;
     constexpr int K = (DEG + 1) * (DEG + 1);
+    float Y[16], c[3 * K];
+    load_sh<DEG>(sg->g.sh, li, c);
+    const float logit = __ldg(sg->g.logits + li);
+    Proj P;
+    project(sg->g, cm, vw.op, li, P);
     float d0 = P.m[0] - cm.cam_pos[0], d1 = P.m[1] - cm.cam_pos[1], d2 = P.m[2] - cm.cam_pos[2];
     const float il = rsqrtf(d0 * d0 + d1 * d1 + d2 * d2);
     d0 *= il; d1 *= il; d2 *= il;
-    float Y[16], c[3 * K];
     sh_basis<DEG>(d0, d1, d2, Y);
-    load_sh<DEG>(sg->g.sh, li, c);
     float rgb[3];
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
@@ -340,7 +475,7 @@ __global__ void __launch_bounds__(256, 5) preprocess_kernel(const DevTables* __r
       for (int k = 0; k < K; ++k) acc = fmaf(c[3 * k + ch], Y[k], acc);
       rgb[ch] = fmaxf(0.f, acc);
     }
-    const float o = 1.f / (1.f + expf(-__ldg(sg->g.logits + li)));
+    const float o = 1.f / (1.f + expf(-logit));
     // the mean's projection for blending, as a double-float (see df_dot3)
     float xh, xl, yh, yl, zh, zl;
     df_dot3(cm.R, cm.t[0], P.m, xh, xl);
@@ -370,77 +505,10 @@ __global__ void __launch_bounds__(256, 5) preprocess_kernel(const DevTables* __r
       hy = sqrtf(k2 * P.C) * 1.001f + 0.01f;
     }
     sp.hxy = (uint32_t)__half_as_ushort(__float2half_ru(hx)) | ((uint32_t)__half_as_ushort(__float2half_ru(hy)) << 16);
-    float4* dst = reinterpret_cast<float4*>(splats + i);
+    float4* dst = reinterpret_cast<float4*>(splats + t);
     const float4* src = reinterpret_cast<const float4*>(&sp);
     dst[0] = src[0]; dst[1] = src[1]; dst[2] = src[2];
   }
-  // min / max depth key over visible Gaussians (they fix the bits the depth sort needs): per warp,
-  // then per block in shared memory, then one global atomic each per block (one per warp put
-  // ~31K same-address atomics per render on two words)
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo_key = min(lo_key, __shfl_xor_sync(0xffffffffu, lo_key, o));
-    hi_key = max(hi_key, __shfl_xor_sync(0xffffffffu, hi_key, o));
-  }
-  if ((threadIdx.x & 31) == 0 && lo_key <= hi_key) {
-    atomicMin(&s_dlo, lo_key);
-    atomicMax(&s_dhi, hi_key);
-  }
-  // 4. stable compaction of the visible Gaussians (index order): offsets within the block from
-  //    the scan above, the block's offset by a decoupled look-back over the blocks before it
-  if (vis) {
-#pragma unroll
-    for (int p = 0; p < kMaxPasses; ++p) atomicAdd(&s_h[p][(key >> (p * kRadixBits)) & (kRadix - 1)], 1u);
-  }
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    unsigned excl = 0;
-    if (blk > 0) {
-      // 32 predecessors per step; rows below 0 read as an empty prefix
-      long long p = (long long)blk - 1;
-      const uint64_t start = global_timer_ns();
-      for (;;) {
-        const unsigned long long v = p - lane >= 0 ? ld_relaxed(cp.status + (p - lane)) : kFlagPrefix;
-        const unsigned pre = __ballot_sync(0xffffffffu, (v & kFlagPrefix) != 0);
-        const unsigned nr = __ballot_sync(0xffffffffu, (v & (kFlagPrefix | kFlagAggregate)) == 0);
-        const int first_pre = pre ? __ffs(pre) - 1 : 32, first_nr = nr ? __ffs(nr) - 1 : 32;
-        const bool done = first_pre < first_nr;
-        const int take = done ? first_pre + 1 : first_nr;       // rows consumed this step
-        unsigned part = lane < take ? (unsigned)(v & kCountMask) : 0u;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        excl += part;
-        if (done) break;
-        p -= take;
-        if (take == 0 && global_timer_ns() - start > cp.wait_ns) {   // a predecessor never published
-          if (lane == 0) atomicOr(&hdr->status, (unsigned)VG_STATUS_WAIT_TIMEOUT);
-          break;
-        }
-      }
-      if (lane == 0 && publish) st_relaxed(cp.status + blk, kFlagPrefix | (excl + tot));
-    }
-    if (lane == 0) {
-      s_base = excl;
-      if (blk == gridDim.x - 1) hdr->visible = excl + tot;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && s_dlo <= s_dhi) {
-    atomicMin(&hdr->dmin, s_dlo);
-    atomicMax(&hdr->dmax, s_dhi);
-  }
-  if (vis) {
-    const unsigned at = s_base + ex;
-    cp.vkeys[at] = key;
-    cp.vvals[at] = (uint32_t)i;
-    cp.vis_ids[at] = (uint32_t)i;     // index order, for the adjoint of the projection
-  }
-#pragma unroll
-  for (int p = 0; p < kMaxPasses; ++p)
-    if (s_h[p][threadIdx.x]) atomicAdd(&cp.hist[p * kRadix + threadIdx.x], s_h[p][threadIdx.x]);
-  // clear the look-back rows of the first depth-sort pass
-  for (size_t z = (size_t)blk * blockDim.x + threadIdx.x; z < cp.zero_words; z += (size_t)gridDim.x * blockDim.x)
-    cp.zero[z] = 0ull;
 }
 
 // Zero gradients of the Gaussians that touch no tile (skipped when accumulating).  A warp owns
@@ -490,7 +558,7 @@ __global__ void __launch_bounds__(256) zero_culled_grads(const DevTables* __rest
 // Adjoint of the projection for visible Gaussian i: writes (or, accumulating, adds) the gradients
 // of its mean, log-scale, quaternion, logit and SH coefficients.
 template <int DEG>
-__device__ __forceinline__ void project_adjoint(const DevTables* __restrict__ tab, const Splat* __restrict__ splats,
+__device__ __forceinline__ void project_adjoint(const DevTables* __restrict__ tab, const Splat& rec,
                                                 const float* __restrict__ g2d, int accumulate, int i) {
   constexpr int K = (DEG + 1) * (DEG + 1);
   constexpr int F = 3 * K;
@@ -512,7 +580,6 @@ __device__ __forceinline__ void project_adjoint(const DevTables* __restrict__ ta
   const KCam cm = tview(tab, sg.view).cam;
   const KOpts op = tview(tab, sg.view).op;
   const int li = (int)l;
-  const Splat& rec = splats[i];
   const uint32_t rank = rec.rank;
   float d2[9];
   {
@@ -689,7 +756,7 @@ __global__ void __launch_bounds__(128, 4) preprocess_backward_kernel(
   const int nv = (int)hdr->visible;
   if (dead) return;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += gridDim.x * blockDim.x)
-    project_adjoint<DEG>(tab, splats, g2d, accumulate, (int)vis_ids[t]);
+    project_adjoint<DEG>(tab, splats[t], g2d, accumulate, (int)vis_ids[t]);
 }
 
 }  // namespace
@@ -697,16 +764,18 @@ __global__ void __launch_bounds__(128, 4) preprocess_backward_kernel(
 cudaError_t launch_preprocess(const DevTables* tab, int total_n, int degree, Splat* splats, uint2* rects,
                               uint32_t* touched, const Compact& cp, WsHeader* hdr, cudaStream_t s) {
   if (total_n == 0) return cudaSuccess;
-  note_launches(1);
-  const int blocks = (total_n + 255) / 256;
+  note_launches(2);
+  const int blocks = (total_n + kCullTile - 1) / kCullTile;
   // the compaction's look-back words (one per block) start cleared
   if (cudaMemsetAsync(cp.status, 0, (size_t)blocks * sizeof(unsigned long long), s) != cudaSuccess)
     return cudaGetLastError();
+  launch_pdl(cull_kernel, blocks, kCullThreads, 0, s, tab, total_n, rects, touched, cp, hdr);
+  const int rb = std::min((total_n + 127) / 128, 8 * sort_blocks());
   switch (degree) {
-    case 0: launch_pdl(preprocess_kernel<0>, blocks, 256, 0, s, tab, total_n, splats, rects, touched, cp, hdr); break;
-    case 1: launch_pdl(preprocess_kernel<1>, blocks, 256, 0, s, tab, total_n, splats, rects, touched, cp, hdr); break;
-    case 2: launch_pdl(preprocess_kernel<2>, blocks, 256, 0, s, tab, total_n, splats, rects, touched, cp, hdr); break;
-    default: launch_pdl(preprocess_kernel<3>, blocks, 256, 0, s, tab, total_n, splats, rects, touched, cp, hdr); break;
+    case 0: launch_pdl(record_kernel<0>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
+    case 1: launch_pdl(record_kernel<1>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
+    case 2: launch_pdl(record_kernel<2>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
+    default: launch_pdl(record_kernel<3>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
   }
   return cudaGetLastError();
 }
