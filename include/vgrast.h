@@ -137,9 +137,9 @@ typedef struct {
 
 #define VG_FLAG_ACCUMULATE_GRADS 1  /* backward adds into the gradient arrays (else writes)  */
 #define VG_FLAG_COUNT_BLENDS 2      /* forward counts evaluations / blends into counters     */
-/* Diagnostic for tests of the bounded-wait error path, never set in normal use: the first block
- * of the projection kernel's stream compaction withholds its look-back status, and that
- * look-back's waits give up after 2 ms instead of 1 s.  The render then reports
+/* Diagnostic for tests of the bounded-wait error path, never set in normal use: the first partition
+ * of the depth sort withholds its look-back status, and that look-back's waits give up after 2 ms
+ * instead of 1 s (more than 1,024 visible Gaussians make a second partition, which waits).  The render then reports
  * VG_STATUS_WAIT_TIMEOUT: every later stage of that render sees the status and treats every tile
  * list as empty (image = background, final T = 1, last = 0), and a backward pass on its
  * workspace writes no gradient of a visible Gaussian.  Nothing waits longer than the limit and

@@ -283,13 +283,13 @@ vg_status run_forward(Call& c, const vg_raster_opts* opts0, void* workspace, siz
   launch_pdl(init_header, 1, 256, 0, s, hdr, reinterpret_cast<SortCtl*>(ws + L.sortctl));
   note_launches(2);   // init_header + publish_counters
   stage_event(ev, VG_STAGE_PROJECT, true, s);
-  cudaError_t e = launch_preprocess(tab, c.total_n, c.degree, reinterpret_cast<Splat*>(ws + L.splats),
-                                    reinterpret_cast<uint2*>(ws + L.rects), reinterpret_cast<uint32_t*>(ws + L.touched),
-                                    make_compact(L, ws, c.total_n, opts0), hdr, s);
+  cudaError_t e = launch_preprocess(tab, c.total_n, reinterpret_cast<uint2*>(ws + L.rects),
+                                    reinterpret_cast<uint32_t*>(ws + L.touched), make_compact(L, ws, opts0), hdr, s);
   if (e != cudaSuccess) return VG_ERR_CUDA;
   stage_event(ev, VG_STAGE_PROJECT, false, s);
   stage_event(ev, VG_STAGE_SORT, true, s);
-  e = launch_binning(tab, c.total_n, c.total_tiles, pair_capacity, L, ws, s);
+  e = launch_binning(tab, c.total_n, c.degree, c.total_tiles, pair_capacity, L, ws,
+                     (opts0->flags & VG_FLAG_TEST_STALL_LOOKBACK) != 0, s);
   if (e != cudaSuccess) return VG_ERR_CUDA;
   stage_event(ev, VG_STAGE_SORT, false, s);
   stage_event(ev, VG_STAGE_BLEND, true, s);

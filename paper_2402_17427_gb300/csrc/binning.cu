@@ -9,7 +9,7 @@
 //      id only (ceil(log2 tiles) bits), which keeps the depth order inside every tile.
 // Both sorts are least-significant-digit radix sorts with 8-bit digits and one kernel per
 // digit pass: the digit histograms of all passes are known before the first pass (the
-// projection kernel accumulates the depth keys'; the tile keys' follow from the per-tile pair
+// projection's compaction accumulates the depth keys'; the tile keys' follow from the per-tile pair
 // counts, which the tile rectangles fix before any pair is emitted, or, for renders of more
 // tiles than one block holds, from the emitted keys), and every pass finds the
 // output offset of each partition by a decoupled look-back over the partitions before it (each
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_pass(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, const unsigned* n_ptr, unsigned cap, bool depth, int shift,
     const unsigned* __restrict__ hist, unsigned* next_part, unsigned long long* status_cur,
-    unsigned long long* __restrict__ status_next, WsHeader* hdr) {
+    unsigned long long* __restrict__ status_next, WsHeader* hdr, bool stall) {
   pdl_enter();
   constexpr int TILE = kSortThreads * ITEMS;
   // the prologue's loads are issued together, then tested
@@ -151,13 +151,13 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_pass(
     unsigned long long* row = status_cur + (size_t)part * kRadix;
     unsigned excl = 0;
     if (part == 0) {
-      st_relaxed(row + d, kFlagPrefix | c);
+      if (!stall) st_relaxed(row + d, kFlagPrefix | c);   // withheld in a test of the bounded wait
     } else {
       st_relaxed(row + d, kFlagAggregate | c);
       // look back kLookback rows at a time (independent loads); rows below 0 read as an empty
       // prefix, so the walk always ends at a prefix
       int p = (int)part - 1;
-      const uint64_t start = global_timer_ns();
+      const uint64_t start = global_timer_ns(), limit = stall ? 2000000ull : 1000000000ull;
       for (;;) {
         unsigned long long v[kLookback];
 #pragma unroll
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kSortThreads) onesweep_pass(
         }
         if (done) break;
         p -= used;
-        if (used == 0 && global_timer_ns() - start > 1000000000ull) {   // a predecessor never published
+        if (used == 0 && global_timer_ns() - start > limit) {   // a predecessor never published
           atomicOr(&hdr->status, (unsigned)VG_STATUS_WAIT_TIMEOUT);
           break;
         }
@@ -738,21 +738,18 @@ Layout make_layout(int64_t total_n, int64_t total_tiles, int64_t cap) {
   return L;
 }
 
-Compact make_compact(const Layout& L, char* ws, int total_n, const vg_raster_opts* opts0) {
+Compact make_compact(const Layout& L, char* ws, const vg_raster_opts* opts0) {
   Compact c;
   c.key_inputs = reinterpret_cast<float4*>(opts0 ? opts0->key_inputs : nullptr);
-  const bool stall = opts0 && (opts0->flags & VG_FLAG_TEST_STALL_LOOKBACK) != 0;
-  c.stall_block = stall ? 0 : -1;
-  c.wait_ns = stall ? 2000000ull : 1000000000ull;
+  // scratch in regions that are written only later: the depth-ordered records (48 bytes a Gaussian)
+  // and the look-back rows of the second depth pass (2 bytes a Gaussian and more)
+  c.entries = reinterpret_cast<uint4*>(ws + L.vsplats);
+  c.counts = reinterpret_cast<unsigned*>(ws + L.status[1]);
   c.vkeys = reinterpret_cast<uint32_t*>(ws + L.vkeys[0]);
   c.vvals = reinterpret_cast<uint32_t*>(ws + L.vvals[0]);
   c.vis_ids = reinterpret_cast<uint32_t*>(ws + L.vis_ids);
-  SortCtl* ctl = reinterpret_cast<SortCtl*>(ws + L.sortctl);
-  c.hist = ctl->hist[0][0];
-  c.ticket = &ctl->ticket;
-  c.status = reinterpret_cast<unsigned long long*>(ws + L.status[1]);
+  c.hist = reinterpret_cast<SortCtl*>(ws + L.sortctl)->hist[0][0];
   c.zero = reinterpret_cast<unsigned long long*>(ws + L.status[0]);
-  c.zero_words = (size_t)((total_n + kDepthTile - 1) / kDepthTile) * kRadix;
   return c;
 }
 
@@ -773,8 +770,8 @@ int onesweep_blocks() {
   return v;
 }
 
-cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capacity, const Layout& L, char* ws,
-                           cudaStream_t s) {
+cudaError_t launch_binning(const DevTables* tab, int n, int degree, int tiles, int64_t capacity, const Layout& L, char* ws,
+                           bool stall, cudaStream_t s) {
   const int B = sort_blocks();
   WsHeader* hdr = reinterpret_cast<WsHeader*>(ws + L.header);
   SortCtl* ctl = reinterpret_cast<SortCtl*>(ws + L.sortctl);
@@ -797,16 +794,21 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
   const bool prep = tiles <= kPrepTiles;
   const uint2* rects = reinterpret_cast<const uint2*>(ws + L.rects);
   uint2* ranges = reinterpret_cast<uint2*>(ws + L.ranges);
-  cudaEvent_t fork = nullptr, join = nullptr;
+  // The records, and for small tile grids the tile counts, need nothing of the depth sort and run on
+  // a side stream beside it (the sort's passes leave most of the chip idle).
+  cudaStream_t side = side_stream_for(s);
+  cudaEvent_t fork = nullptr, join = nullptr, rec_join = nullptr;
+  if (side && (fork = call_event(kEvBinningFork)) && (join = call_event(kEvBinningJoin)) &&
+      (rec_join = call_event(kEvRecordJoin))) {
+    cudaEventRecord(fork, s);
+    cudaStreamWaitEvent(side, fork, 0);
+  } else {
+    side = s;
+    join = rec_join = nullptr;
+  }
+  cudaError_t re = launch_records(tab, n, degree, U(L.vis_ids), hdr, splats, side);
+  if (rec_join) cudaEventRecord(rec_join, side);
   if (prep) {
-    cudaStream_t side = side_stream_for(s);
-    if (side && (fork = call_event(kEvBinningFork)) && (join = call_event(kEvBinningJoin))) {
-      cudaEventRecord(fork, s);
-      cudaStreamWaitEvent(side, fork, 0);
-    } else {
-      side = s;
-      join = nullptr;
-    }
     unsigned* tdiff = U(L.tcount);
     const size_t smem = (size_t)2 * tiles * sizeof(unsigned);
     // the shared-memory opt-in, once per device and context (function attributes live in the
@@ -824,6 +826,8 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
                                                                 tiles);
     tile_prep<<<1, kPrepThreads, smem, side>>>(tab, tiles, cap, tpasses, tdiff, ranges, ctl->hist[1][0], U(L.order));
     if (join) cudaEventRecord(join, side);
+  } else {
+    join = nullptr;                     // the side stream's last work is the records: rec_join
   }
   // 1. depth sort of the visible Gaussians (compacted by the projection kernel); passes beyond
   //    the bits the keys differ in return at once, and the result sits in the buffer
@@ -832,15 +836,17 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
     const int src = pass & 1, dst = src ^ 1;
     launch_pdl(onesweep_pass<kDepthItems>, OBD, kSortThreads, 0, s, U(L.vkeys[src]), U(L.vvals[src]), U(L.vkeys[dst]), U(L.vvals[dst]),
                                               &hdr->visible, 0xFFFFFFFFu, true, pass * kRadixBits,
-                                              ctl->hist[0][pass], &ctl->next_part[0][pass], S64(src), S64(dst), hdr);
+                                              ctl->hist[0][pass], &ctl->next_part[0][pass], S64(src), S64(dst), hdr,
+                                              stall && pass == 0);
   }
   // 2. pairs in depth order, written where the tile sort's passes leave the result in buffer 0
   const int p0 = tpasses & 1;
   const int BP = kMaxSortBlocks < 6 * B / 2 ? kMaxSortBlocks : 6 * B / 2;   // 6 blocks per SM
   // per Gaussian in depth order: first tile key and rectangle shape in the depth keys' buffers,
   // free once the depth sort is done
-  launch_pdl(pairs_count, BP, 256, 0, s, tab, U(L.vvals[0]), U(L.vvals[1]), U(L.vis_ids), rects, hdr, bsum64,
-             splats, vsplats, U(L.vkeys[0]), U(L.vkeys[1]));
+  if (rec_join) cudaStreamWaitEvent(s, rec_join, 0);
+  pairs_count<<<BP, 256, 0, s>>>(tab, U(L.vvals[0]), U(L.vvals[1]), U(L.vis_ids), rects, hdr, bsum64, splats, vsplats,
+                                 U(L.vkeys[0]), U(L.vkeys[1]));   // plainly: the first after a join
   launch_pdl(pairs_scan, 1, 256, 0, s, bsum64, BP, hdr, (unsigned long long)cap);
   launch_pdl(pairs_emit, 2 * B, 256, 0, s, U(L.vvals[0]), U(L.vvals[1]), hdr, bsum64, BP, U(L.vkeys[0]),
              U(L.vkeys[1]), U(L.pkeys[p0]), U(L.pvals[p0]), prep ? S64(0) : nullptr);
@@ -855,15 +861,15 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
     if (pass == 0 && join)
       k<<<OBT, kSortThreads, 0, s>>>(U(L.pkeys[src]), U(L.pvals[src]), U(L.pkeys[dst]), U(L.pvals[dst]), &hdr->pair_n, cap,
                                      false, pass * kRadixBits, ctl->hist[1][pass], &ctl->next_part[1][pass],
-                                     S64(pass & 1), nxt, hdr);
+                                     S64(pass & 1), nxt, hdr, false);
     else
       launch_pdl(k, OBT, kSortThreads, 0, s, U(L.pkeys[src]), U(L.pvals[src]), U(L.pkeys[dst]), U(L.pvals[dst]),
                  &hdr->pair_n, cap, false, pass * kRadixBits, ctl->hist[1][pass], &ctl->next_part[1][pass],
-                 S64(pass & 1), nxt, hdr);
+                 S64(pass & 1), nxt, hdr, false);
   }
   if (prep) {
     note_launches(kMaxPasses + 3 + tpasses + 2);
-    return cudaGetLastError();
+    return re == cudaSuccess ? cudaGetLastError() : re;
   }
   note_launches(kMaxPasses + 4 + tpasses + 1);
   cudaMemsetAsync(ranges, 0, (size_t)tiles * sizeof(uint2), s);
@@ -878,7 +884,7 @@ cudaError_t launch_binning(const DevTables* tab, int n, int tiles, int64_t capac
     launch_pdl(order_scatter, tgrid, 256, 0, s, tab, ranges, tiles, buckets, U(L.order));
     note_launches(3);
   }
-  return cudaGetLastError();
+  return re == cudaSuccess ? cudaGetLastError() : re;
 }
 
 }  // namespace vg

@@ -159,7 +159,6 @@ constexpr int kMaxPasses = 4;                           // 32-bit keys
 struct SortCtl {
   unsigned hist[2][kMaxPasses][kRadix];
   unsigned next_part[2][kMaxPasses];
-  unsigned ticket;                 // block tickets of the projection kernel's compaction
 };
 
 inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
@@ -190,19 +189,17 @@ struct HostPlan {
 };
 
 // ---- launchers (each returns the first CUDA error it hits) ----
-// Outputs of the compaction fused into the projection kernel.
+// What the projection leaves for the sorts: the visible Gaussians in index order, by slot.
+constexpr int kCullRun = 512;      // Gaussians a block of the projection takes
 struct Compact {
-  uint32_t* vkeys;                 // depth keys (FP32 bits) of the visible Gaussians, index order
-  uint32_t* vvals;                 // their ids (the depth sort's values)
-  uint32_t* vis_ids;               // their ids again (kept in index order for the adjoint)
+  uint4* entries;                  // [total_n] scratch: each run's visible Gaussians (key, id, rectangle)
+  unsigned* counts;                // [runs, padded to 4] their numbers
+  uint32_t* vkeys;                 // depth keys (FP32 bits) of the visible Gaussians, by slot
+  uint32_t* vvals;                 // the slots (the depth sort's values)
+  uint32_t* vis_ids;               // Gaussian of each slot
   unsigned* hist;                  // [kMaxPasses][kRadix] digit histograms of the depth keys
-  unsigned* ticket;                // block ticket counter (cleared per render)
-  unsigned long long* status;      // one look-back word per block (cleared by the launcher)
   unsigned long long* zero;        // look-back rows of the first depth pass, cleared here
-  size_t zero_words;
   float4* key_inputs;              // optional [total_n]: (u, v, r, depth) the keys were decided from
-  int stall_block;                 // block that withholds its look-back status (tests only), else -1
-  unsigned long long wait_ns;      // limit of each look-back wait
 };
 // Every kernel after the first look-back of a render checks this once: after a wait gave up the
 // compacted and sorted arrays may hold unwritten slots, so no stage may index with them.  The flag
@@ -221,10 +218,13 @@ __device__ __forceinline__ void pdl_enter() {
 __device__ __forceinline__ bool render_dead(const WsHeader* hdr) {
   return (hdr->status & VG_STATUS_WAIT_TIMEOUT) != 0u;
 }
-cudaError_t launch_preprocess(const DevTables* tab, int total_n, int degree, Splat* splats, uint2* rects,
-                              uint32_t* touched, const Compact& cp, WsHeader* hdr, cudaStream_t s);
-// Regions of the workspace; opts0 supplies the optional key-input record and the test stall.
-Compact make_compact(const Layout& L, char* ws, int total_n, const vg_raster_opts* opts0);
+cudaError_t launch_preprocess(const DevTables* tab, int total_n, uint2* rects, uint32_t* touched, const Compact& cp,
+                              WsHeader* hdr, cudaStream_t s);
+// Splat records of the visible Gaussians, by slot (launched plainly).
+cudaError_t launch_records(const DevTables* tab, int total_n, int degree, const uint32_t* vis_ids, const WsHeader* hdr,
+                           Splat* splats, cudaStream_t s);
+// Regions of the workspace; opts0 supplies the optional key-input record.
+Compact make_compact(const Layout& L, char* ws, const vg_raster_opts* opts0);
 // Adjoint of the projection for the visible Gaussians (gradients of the culled ones are left
 // to launch_zero_culled, or untouched when accumulating).  Sized to leave launch_zero_culled
 // room to run beside it when not accumulating.
@@ -235,10 +235,11 @@ cudaError_t launch_preprocess_backward(const DevTables* tab, int total_n, int de
 cudaError_t launch_zero_culled(const DevTables* tab, int total_n, int degree, const uint32_t* touched,
                                cudaStream_t s);
 
-// Depth order of the visible Gaussians, pair generation (with the depth-ordered splat records),
-// tile sort, ranges and the largest-first order of the tiles.
-cudaError_t launch_binning(const DevTables* tab, int total_n, int total_tiles, int64_t capacity, const Layout& L,
-                           char* ws, cudaStream_t s);
+// Depth order of the visible Gaussians beside their splat records, pair generation (with the
+// depth-ordered records), tile sort, ranges and the largest-first order of the tiles.  stall (tests
+// only): the first partition of the depth sort withholds its look-back words.
+cudaError_t launch_binning(const DevTables* tab, int total_n, int degree, int total_tiles, int64_t capacity,
+                           const Layout& L, char* ws, bool stall, cudaStream_t s);
 
 cudaError_t launch_blend_forward(const DevTables* tab, const HostPlan& plan, const Layout& L, char* ws, bool count,
                                  cudaStream_t s);
@@ -263,7 +264,7 @@ cudaStream_t side_stream_for(cudaStream_t caller);
 // is legal, since each cudaStreamWaitEvent takes the record that precedes it in host order, and
 // one thread's calls are issued one after another.  nullptr if creation fails.
 enum CallEventSlot {
-  kEvBackwardFork, kEvBackwardJoin, kEvBinningFork, kEvBinningJoin, kEvLossFork, kEvLossJoin,
+  kEvBackwardFork, kEvBackwardJoin, kEvBinningFork, kEvBinningJoin, kEvRecordJoin, kEvLossFork, kEvLossJoin,
   kEvAppearance, kCallEvents = kEvAppearance + 16
 };
 cudaEvent_t call_event(int slot);

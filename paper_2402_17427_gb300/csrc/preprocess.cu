@@ -269,41 +269,30 @@ __device__ __forceinline__ bool may_touch(const KGauss& g, const KCam& cm, const
   return !(u + ru < 0.f || u - ru > (float)(cm.W - 1) || v + rv < 0.f || v - rv > (float)(cm.H - 1));
 }
 
-// Projection, first half: the visible Gaussians, compacted in index order (slot = position in that
-// order), with their depth keys and tile rectangles.
+// Projection, first part: the visible Gaussians of every run of 512, in index order, each as one
+// entry (depth key, Gaussian, tile rectangle) in the run's own part of `entries`, and their number.
 //
-// A block takes 512 Gaussians in ticket order (so the look-back only waits on running blocks), four
-// a thread with their loads in flight together.  Only ~1 in 5 is visible (1 in 25 in the 20M-Gaussian
-// city), in no order, so may_touch() first thins them out on 24 bytes a Gaussian, the candidates are packed
-// densely in shared memory, and whole warps of them go through project().  The colours and records, which need
-// no order, are left to record_kernel over the dense list of visible Gaussians: with the spherical
-// harmonics in this kernel its blocks waited at their barriers for a few busy warps and for the
-// look-back (one Gaussian a thread, 256 a block: 58 us for 1M Gaussians and 963 us for 20M).
-constexpr int kCullThreads = 128, kCullItems = 4, kCullTile = kCullThreads * kCullItems, kCullWarps = kCullThreads / 32;
+// Only ~1 in 5 Gaussians is visible (1 in 25 in the 20M-Gaussian city), in no order, so may_touch()
+// first thins them out on 24 bytes a Gaussian, four a thread with their loads in flight together; the
+// candidates are packed densely in shared memory, and whole warps of them go through project().  No
+// block waits for another: compact_kernel closes the gaps between the runs.  In one kernel with a
+// look-back over the runs (and the spherical harmonics, which now follow in record_kernel) a block
+// spent most of its ~19 us waiting: 963 us for the 20M Gaussians of the city and 58 us for 1M; with
+// the harmonics moved out 550 and 44 us.
+constexpr int kCullThreads = 128, kCullItems = 4, kCullWarps = kCullThreads / 32;
+static_assert(kCullThreads * kCullItems == kCullRun, "a block takes one run");
 __global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* __restrict__ tab, int total_n,
-                                                                uint2* __restrict__ rects,
-                                                                uint32_t* __restrict__ touched, const Compact cp,
-                                                                WsHeader* __restrict__ hdr) {
+                                                               uint4* __restrict__ entries,
+                                                               unsigned* __restrict__ counts,
+                                                               uint32_t* __restrict__ touched,
+                                                               float4* __restrict__ key_inputs) {
   pdl_enter();
-  __shared__ unsigned s_blk, s_base;
-  __shared__ unsigned s_dlo, s_dhi;                      // the block's min / max depth key
   __shared__ unsigned s_wc[2][kCullItems * kCullWarps];  // counts a warp (and item) leaves for the others
-  __shared__ unsigned s_h[kMaxPasses][kRadix];
-  __shared__ uint16_t s_cand[kCullTile], s_local[kCullTile];
-  __shared__ unsigned s_key[kCullTile];
-  __shared__ uint2 s_rect[kCullTile];
+  __shared__ uint16_t s_cand[kCullRun];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
-    s_blk = atomicAdd(cp.ticket, 1u);
-    s_dlo = 0xFFFFFFFFu;
-    s_dhi = 0u;
-  }
-  for (int k = tid; k < kMaxPasses * kRadix; k += kCullThreads) s_h[k / kRadix][k % kRadix] = 0;
-  __syncthreads();
-  const unsigned blk = s_blk;
-  const int base = (int)(blk * kCullTile), last = min(total_n - 1, base + (kCullTile - 1));
+  const int base = (int)blockIdx.x * kCullRun, last = min(total_n - 1, base + (kCullRun - 1));
   const int seg0 = find_seg(tab, base);
-  const bool one = seg0 == tab->h.n_segs - 1 || tseg(tab, seg0 + 1).offset > last;   // one segment in this block
+  const bool one = seg0 == tab->h.n_segs - 1 || tseg(tab, seg0 + 1).offset > last;   // one segment in this run
   // 1. candidates: a mean each, all four requested together, then the largest scales
   float m[kCullItems][3];
 #pragma unroll
@@ -323,7 +312,7 @@ __global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* 
     if (i <= last) {
       const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
       const KView& vw = tview(tab, sg.view);
-      c = cp.key_inputs != nullptr || may_touch(sg.g, vw.cam, vw.op, i - sg.offset, m[j]);
+      c = key_inputs != nullptr || may_touch(sg.g, vw.cam, vw.op, i - sg.offset, m[j]);
       if (!c) touched[i] = 0;
     }
     votes[j] = __ballot_sync(0xffffffffu, c);
@@ -340,16 +329,13 @@ __global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* 
     ncand += (int)s_wc[0][k];
   }
   __syncthreads();
-  // 2. projection, tile rectangle and visibility of the candidates, the visible ones packed in order
-  unsigned tot = 0, lo_key = 0xFFFFFFFFu, hi_key = 0u;
+  // 2. projection, tile rectangle and visibility of the candidates, the visible ones written in order
+  unsigned tot = 0;
   for (int r = 0, odd = 1; r < ncand; r += kCullThreads, odd ^= 1) {
     bool vis = false;
-    uint32_t key = 0;
-    uint2 rect = make_uint2(0u, 0u);
-    int local = 0;
+    uint4 e = make_uint4(0u, 0u, 0u, 0u);
     if (r + tid < ncand) {
-      local = s_cand[r + tid];
-      const int i = base + local;
+      const int i = base + s_cand[r + tid];
       const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
       const KView& vw = tview(tab, sg.view);
       Proj P;
@@ -362,16 +348,14 @@ __global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* 
         if (xlo <= xhi && ylo <= yhi) {
           const int tx0 = xlo / T, tx1 = xhi / T, ty0 = ylo / T, ty1 = yhi / T;
           cnt = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
-          rect = make_uint2((uint32_t)tx0 | ((uint32_t)tx1 << 16), (uint32_t)ty0 | ((uint32_t)ty1 << 16));
           vis = true;
-          key = __float_as_uint(P.depth);
-          lo_key = min(lo_key, key);
-          hi_key = max(hi_key, key);
+          e = make_uint4(__float_as_uint(P.depth), (uint32_t)i, (uint32_t)tx0 | ((uint32_t)tx1 << 16),
+                         (uint32_t)ty0 | ((uint32_t)ty1 << 16));
         }
       }
       touched[i] = cnt;
-      if (cp.key_inputs)
-        cp.key_inputs[i] = P.valid ? make_float4(P.u, P.v, P.r, P.depth) : make_float4(0.f, 0.f, -1.f, 0.f);
+      if (key_inputs)
+        key_inputs[i] = P.valid ? make_float4(P.u, P.v, P.r, P.depth) : make_float4(0.f, 0.f, -1.f, 0.f);
     }
     const unsigned vote = __ballot_sync(0xffffffffu, vis);
     if (lane == 0) s_wc[odd][warp] = __popc(vote);
@@ -383,66 +367,103 @@ __global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* 
       if (w < warp) at += c;
       tot += c;
     }
-    if (vis) {
-      s_key[at] = key;
-      s_rect[at] = rect;
-      s_local[at] = (uint16_t)local;
+    if (vis) entries[(size_t)base + at] = e;
+  }
+  if (tid == 0) counts[blockIdx.x] = tot;
+}
+
+// Projection, second part: the runs' entries moved together in index order (slot = position among all
+// visible Gaussians): depth keys and sort values (the slots), ids and rectangles, with the digit
+// histograms and the range of the keys.  Each block owns consecutive runs and adds up the counts of
+// the runs before it itself (L2 reads, a few us even for the 39K runs of 20M Gaussians), so there is
+// neither a look-back nor a scan kernel.
+constexpr int kCompactThreads = 256;
+__global__ void __launch_bounds__(kCompactThreads) compact_kernel(const uint4* __restrict__ entries,
+                                                                  const unsigned* __restrict__ counts, int runs,
+                                                                  int per_block, uint2* __restrict__ rects,
+                                                                  const Compact cp, WsHeader* __restrict__ hdr) {
+  pdl_enter();
+  __shared__ unsigned s_sm[8];
+  __shared__ unsigned s_off[kCompactThreads];
+  __shared__ unsigned s_h[kMaxPasses][kRadix];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+  for (int p = 0; p < kMaxPasses; ++p) s_h[p][tid] = 0;
+  const int first = (int)blockIdx.x * per_block, end = min(runs, first + per_block);
+  unsigned before = 0, all = 0;     // visible Gaussians before this block's runs, and in total
+#pragma unroll 4
+  for (int k = 4 * tid; k < runs; k += 4 * kCompactThreads) {
+    const uint4 c = __ldg(reinterpret_cast<const uint4*>(counts + k));     // padded to 4
+    const unsigned v[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (k + j < runs) all += v[j];
+      if (k + j < first) before += v[j];
     }
   }
-  // min / max depth key over visible Gaussians (they fix the bits the depth sort needs): per warp,
-  // then per block in shared memory, then one global atomic each per block (one per warp put
-  // ~31K same-address atomics per render on two words)
+  unsigned total;
+  block_exclusive_scan(all, &total, s_sm);
+  unsigned base;
+  block_exclusive_scan(before, &base, s_sm);
+  if (blockIdx.x == 0 && tid == 0) hdr->visible = total;
+  unsigned lo_key = 0xFFFFFFFFu, hi_key = 0u;
+  for (int r0 = first; r0 < end; r0 += kCompactThreads) {
+    unsigned sum;
+    s_off[tid] = base + block_exclusive_scan(r0 + tid < end ? counts[r0 + tid] : 0u, &sum, s_sm);
+    __syncthreads();
+    base += sum;
+    for (int r = r0 + warp; r < min(end, r0 + kCompactThreads); r += kCompactThreads / 32) {
+      const unsigned o = s_off[r - r0];
+      const unsigned n = (r + 1 - r0 < kCompactThreads ? s_off[r + 1 - r0] : base) - o;   // absent runs count 0
+      for (unsigned k = lane; k < n; k += 32) {
+        const uint4 e = __ldg(entries + (size_t)r * kCullRun + k);
+        cp.vkeys[o + k] = e.x;
+        cp.vvals[o + k] = o + k;
+        cp.vis_ids[o + k] = e.y;
+        rects[o + k] = make_uint2(e.z, e.w);
+        lo_key = min(lo_key, e.x);
+        hi_key = max(hi_key, e.x);
+#pragma unroll
+        for (int p = 0; p < kMaxPasses; ++p) atomicAdd(&s_h[p][(e.x >> (p * kRadixBits)) & (kRadix - 1)], 1u);
+      }
+    }
+    __syncthreads();
+  }
+  // min / max depth key (they fix the bits the depth sort needs): one global atomic each a block
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lo_key = min(lo_key, __shfl_xor_sync(0xffffffffu, lo_key, o));
     hi_key = max(hi_key, __shfl_xor_sync(0xffffffffu, hi_key, o));
   }
-  if (lane == 0 && lo_key <= hi_key) {
-    atomicMin(&s_dlo, lo_key);
-    atomicMax(&s_dhi, hi_key);
+  __shared__ unsigned s_lo[kCompactThreads / 32], s_hi[kCompactThreads / 32];
+  if (lane == 0) {
+    s_lo[warp] = lo_key;
+    s_hi[warp] = hi_key;
   }
   __syncthreads();
-  // 3. the block's offset among all visible Gaussians (warp 0) beside the digit histograms (the others)
-  if (warp == 0) {
-    const unsigned excl = lookback(cp.status, blk, tot, &hdr->status, (unsigned)VG_STATUS_WAIT_TIMEOUT, cp.wait_ns,
-                                   (int)blk != cp.stall_block);
-    if (lane == 0) {
-      s_base = excl;
-      if (blk == gridDim.x - 1) hdr->visible = excl + tot;
-      if (s_dlo <= s_dhi) {
-        atomicMin(&hdr->dmin, s_dlo);
-        atomicMax(&hdr->dmax, s_dhi);
-      }
+  if (tid == 0) {
+    for (int w = 1; w < kCompactThreads / 32; ++w) {
+      lo_key = min(lo_key, s_lo[w]);
+      hi_key = max(hi_key, s_hi[w]);
     }
-  } else {
-    for (unsigned k = tid - 32; k < tot; k += kCullThreads - 32) {
-      const unsigned key = s_key[k];
+    if (lo_key <= hi_key) {
+      atomicMin(&hdr->dmin, lo_key);
+      atomicMax(&hdr->dmax, hi_key);
+    }
+  }
 #pragma unroll
-      for (int p = 0; p < kMaxPasses; ++p) atomicAdd(&s_h[p][(key >> (p * kRadixBits)) & (kRadix - 1)], 1u);
-    }
-  }
-  __syncthreads();
-  for (unsigned k = tid; k < tot; k += kCullThreads) {
-    const unsigned at = s_base + k;
-    cp.vkeys[at] = s_key[k];
-    cp.vvals[at] = at;
-    cp.vis_ids[at] = (uint32_t)(base + s_local[k]);
-    rects[at] = s_rect[k];
-  }
-  if (tot > 0)
-    for (int k = tid; k < kMaxPasses * kRadix; k += kCullThreads) {
-      const unsigned c = s_h[k / kRadix][k % kRadix];
-      if (c) atomicAdd(&cp.hist[k], c);
-    }
+  for (int p = 0; p < kMaxPasses; ++p)
+    if (s_h[p][tid]) atomicAdd(&cp.hist[p * kRadix + tid], s_h[p][tid]);
   // clear the look-back rows of the first depth-sort pass
-  for (size_t z = (size_t)blk * kCullThreads + tid; z < cp.zero_words; z += (size_t)gridDim.x * kCullThreads)
+  const size_t zero_words = (size_t)((total + kDepthTile - 1) / kDepthTile) * kRadix;
+  for (size_t z = (size_t)blockIdx.x * kCompactThreads + tid; z < zero_words; z += (size_t)gridDim.x * kCompactThreads)
     cp.zero[z] = 0ull;
 }
 
-// Projection, second half: the splat record of every visible Gaussian, by slot: colour from
+// Projection, third part: the splat record of every visible Gaussian, by slot: colour from
 // spherical harmonics along the viewing direction, opacity, the accurate blending position and the
 // alpha >= alpha_min box.  Bound by the latency of the scattered parameter rows, with no barrier and
-// nothing to wait for, so it runs at whatever occupancy its registers leave.
+// nothing to wait for; launched beside the depth sort, which needs only the keys.
 template <int DEG>
 __global__ void __launch_bounds__(128) record_kernel(const DevTables* __restrict__ tab,
                                                      const uint32_t* __restrict__ vis_ids,
@@ -761,21 +782,29 @@ __global__ void __launch_bounds__(128, 4) preprocess_backward_kernel(
 
 }  // namespace
 
-cudaError_t launch_preprocess(const DevTables* tab, int total_n, int degree, Splat* splats, uint2* rects,
-                              uint32_t* touched, const Compact& cp, WsHeader* hdr, cudaStream_t s) {
+cudaError_t launch_preprocess(const DevTables* tab, int total_n, uint2* rects, uint32_t* touched, const Compact& cp,
+                              WsHeader* hdr, cudaStream_t s) {
   if (total_n == 0) return cudaSuccess;
   note_launches(2);
-  const int blocks = (total_n + kCullTile - 1) / kCullTile;
-  // the compaction's look-back words (one per block) start cleared
-  if (cudaMemsetAsync(cp.status, 0, (size_t)blocks * sizeof(unsigned long long), s) != cudaSuccess)
-    return cudaGetLastError();
-  launch_pdl(cull_kernel, blocks, kCullThreads, 0, s, tab, total_n, rects, touched, cp, hdr);
-  const int rb = std::min((total_n + 127) / 128, 8 * sort_blocks());
+  const int runs = (total_n - 1) / kCullRun + 1;
+  launch_pdl(cull_kernel, runs, kCullThreads, 0, s, tab, total_n, cp.entries, cp.counts, touched, cp.key_inputs);
+  // a warp a run on small scenes, up to 2 blocks an SM
+  const int blocks = std::max(1, std::min((runs + kCompactThreads / 32 - 1) / (kCompactThreads / 32), sort_blocks()));
+  const int per = (runs + blocks - 1) / blocks;
+  launch_pdl(compact_kernel, (runs + per - 1) / per, kCompactThreads, 0, s, cp.entries, cp.counts, runs, per, rects, cp, hdr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_records(const DevTables* tab, int total_n, int degree, const uint32_t* vis_ids, const WsHeader* hdr,
+                           Splat* splats, cudaStream_t s) {
+  if (total_n == 0) return cudaSuccess;
+  note_launches(1);
+  const int rb = std::min((total_n - 1) / 128 + 1, 8 * sort_blocks());
   switch (degree) {
-    case 0: launch_pdl(record_kernel<0>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
-    case 1: launch_pdl(record_kernel<1>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
-    case 2: launch_pdl(record_kernel<2>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
-    default: launch_pdl(record_kernel<3>, rb, 128, 0, s, tab, cp.vis_ids, hdr, splats); break;
+    case 0: record_kernel<0><<<rb, 128, 0, s>>>(tab, vis_ids, hdr, splats); break;
+    case 1: record_kernel<1><<<rb, 128, 0, s>>>(tab, vis_ids, hdr, splats); break;
+    case 2: record_kernel<2><<<rb, 128, 0, s>>>(tab, vis_ids, hdr, splats); break;
+    default: record_kernel<3><<<rb, 128, 0, s>>>(tab, vis_ids, hdr, splats); break;
   }
   return cudaGetLastError();
 }
