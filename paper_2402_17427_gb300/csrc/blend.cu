@@ -673,18 +673,20 @@ __global__ void prepare_backward(float* __restrict__ g2d, WsHeader* __restrict__
   if (blockIdx.x == 0) {
     if (threadIdx.x < kTileClasses) hdr->work_bwd[threadIdx.x] = 0;
     if (threadIdx.x == 0) hdr->evals_run_bwd = 0;
+    if (threadIdx.x == 0) hdr->zero_next = 0;
   }
   const size_t n = (size_t)hdr->visible * 9;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) g2d[i] = 0.f;
 }
 
+// Resident blocks of a persistent kernel, `spare` an SM left for another kernel's.
 template <typename K>
-int resident_grid(K kernel, int threads, int items) {
+int resident_grid(K kernel, int threads, int items, int spare = 0) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0);
-  if (per < 1) per = 1;
+  per = per - spare < 1 ? 1 : per - spare;
   const int g = sms * per;
   return items < g ? items : g;
 }
@@ -710,26 +712,29 @@ cudaError_t fwd_class(const DevTables* tab, const HostPlan& plan, const Splat* v
 template <int TS, bool ABS, bool COUNT>
 void bwd_launch(const DevTables* tab, const Splat* vsplats, const uint32_t* lists, const uint2* ranges,
                 const uint32_t* order, int begin, int items, float* g2d, const uint32_t* d0, const uint32_t* d1,
-                const uint32_t* vis_ids, WsHeader* hdr, cudaStream_t s) {
+                const uint32_t* vis_ids, WsHeader* hdr, bool share, cudaStream_t s) {
   using S = TileShape<TS, true>;
   auto k = blend_backward_kernel<TS, ABS, COUNT>;
-  launch_pdl(k, resident_grid(k, S::kThreads, items), S::kThreads, 0, s, tab, vsplats, lists, ranges, order, begin, items, g2d,
+  // The 8 x 8 and 16 x 16 kernels fill an SM with 16 blocks or more, so one fewer costs little and
+  // gives zero_ahead its registers and shared memory; the 32 x 32 kernel holds only a few.
+  launch_pdl(k, resident_grid(k, S::kThreads, items, share && TS <= 16 ? 1 : 0), S::kThreads, 0, s, tab, vsplats, lists, ranges, order, begin, items, g2d,
                                                                  d0, d1, vis_ids, hdr);
 }
 
 template <int TS>
 cudaError_t bwd_class(const DevTables* tab, const HostPlan& plan, const Splat* vsplats, const uint32_t* lists,
                       const uint2* ranges, const uint32_t* order, float* g2d, const uint32_t* d0, const uint32_t* d1,
-                      const uint32_t* vis_ids, WsHeader* hdr, bool abs, bool count, cudaStream_t s) {
+                      const uint32_t* vis_ids, WsHeader* hdr, bool abs, bool count, bool share,
+                      cudaStream_t s) {
   using S = TileShape<TS, true>;
   const int items = plan.class_tiles[S::kClass];
   if (items == 0) return cudaSuccess;
   note_launches(1);
   const int begin = plan.class_begin[S::kClass];
-  if (abs && count) bwd_launch<TS, true, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
-  else if (abs) bwd_launch<TS, true, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
-  else if (count) bwd_launch<TS, false, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
-  else bwd_launch<TS, false, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, s);
+  if (abs && count) bwd_launch<TS, true, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
+  else if (abs) bwd_launch<TS, true, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
+  else if (count) bwd_launch<TS, false, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
+  else bwd_launch<TS, false, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
   return cudaGetLastError();
 }
 
@@ -748,22 +753,26 @@ cudaError_t launch_blend_forward(const DevTables* tab, const HostPlan& plan, con
   return e;
 }
 
+cudaError_t launch_prepare_backward(const Layout& L, char* ws, cudaStream_t s) {
+  note_launches(1);
+  return launch_pdl(prepare_backward, sort_blocks() * 2, 256, 0, s, reinterpret_cast<float*>(ws + L.g2d),
+                    reinterpret_cast<WsHeader*>(ws + L.header));
+}
+
 cudaError_t launch_blend_backward(const DevTables* tab, const HostPlan& plan, const Layout& L, char* ws, bool abs,
-                                  bool count, cudaStream_t s) {
+                                  bool count, bool share, cudaStream_t s) {
   const Splat* vsplats = reinterpret_cast<const Splat*>(ws + L.vsplats);
   const uint32_t* lists = reinterpret_cast<const uint32_t*>(ws + L.pvals[0]);   // final tile-sorted ranks
   const uint2* ranges = reinterpret_cast<const uint2*>(ws + L.ranges);
   const uint32_t* order = reinterpret_cast<const uint32_t*>(ws + L.order);
   WsHeader* hdr = reinterpret_cast<WsHeader*>(ws + L.header);
   float* g2d = reinterpret_cast<float*>(ws + L.g2d);
-  launch_pdl(prepare_backward, sort_blocks() * 2, 256, 0, s, g2d, hdr);
-  note_launches(1);
   const uint32_t* d0 = reinterpret_cast<const uint32_t*>(ws + L.vvals[0]);
   const uint32_t* d1 = reinterpret_cast<const uint32_t*>(ws + L.vvals[1]);
   const uint32_t* vis_ids = reinterpret_cast<const uint32_t*>(ws + L.vis_ids);
-  cudaError_t e = bwd_class<8>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, s);
-  if (e == cudaSuccess) e = bwd_class<16>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, s);
-  if (e == cudaSuccess) e = bwd_class<32>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, s);
+  cudaError_t e = bwd_class<8>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, share, s);
+  if (e == cudaSuccess) e = bwd_class<16>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, share, s);
+  if (e == cudaSuccess) e = bwd_class<32>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, share, s);
   return e;
 }
 

@@ -532,16 +532,72 @@ __global__ void __launch_bounds__(128) record_kernel(const DevTables* __restrict
   }
 }
 
-// Zero gradients of the Gaussians that touch no tile (skipped when accumulating).  A warp owns
-// 32 consecutive Gaussians and writes their SH gradient rows cooperatively, so consecutive
-// lanes store consecutive 16-byte words.
+// Dense gradient outputs are zero for every Gaussian that touches no tile: 236 bytes a Gaussian, most of
+// the bytes of a step (4.7 GB for 20M Gaussians, 0.80 ms at the write rate).  The compositing adjoint before
+// it leaves HBM idle (2% of its bandwidth), so one warp an SM zeroes whole runs of 512 Gaussians, visible or
+// not, while it runs: bulk copies (cp.async.bulk) of a zeroed shared buffer, which take no issue slots.
+// It stops when the adjoint's queues are empty; zero_culled_grads does the rest beside the projection
+// adjoint, which writes the visible rows afterwards.  Which kernel zeroes a run depends on timing, the
+// result does not.  Evict-first, so that the adjoint's records and images stay in L2.
+constexpr uint32_t kZeroBytes = 8192;
+__device__ __forceinline__ void bulk_zero(float* dst, size_t bytes, uint32_t src, uint64_t policy) {
+  char* p = reinterpret_cast<char*>(dst);
+  char* const e = p + bytes;
+  while (p < e && (reinterpret_cast<uintptr_t>(p) & 15u)) {     // to a 16-byte boundary by plain stores
+    *reinterpret_cast<float*>(p) = 0.f;
+    p += 4;
+  }
+  while (p + 16 <= e) {
+    const uint32_t n = (uint32_t)min((size_t)kZeroBytes, (size_t)(e - p) & ~(size_t)15);
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(p), "r"(src),
+                 "r"(n), "l"(policy)
+                 : "memory");
+    p += n;
+  }
+  for (; p < e; p += 4) *reinterpret_cast<float*>(p) = 0.f;
+}
+
+__global__ void __launch_bounds__(32) zero_ahead(const DevTables* __restrict__ tab, int total_n, int F, int items0,
+                                                 int items1, int items2, WsHeader* __restrict__ hdr) {
+  __shared__ __align__(128) float4 s_zero[kZeroBytes / 16];
+  for (int k = threadIdx.x; k < (int)(kZeroBytes / 16); k += 32) s_zero[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  // after a wait of the forward gave up, no gradient of a visible Gaussian is written
+  if (threadIdx.x != 0 || render_dead(hdr)) return;
+  uint64_t policy;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  const uint32_t src = smem_u32(s_zero);
+  const int runs = (total_n - 1) / kCullRun + 1;
+  const volatile unsigned* q = hdr->work_bwd;
+  for (;;) {
+    // every tile has been taken: the rest is left to zero_culled_grads
+    if (q[0] >= (unsigned)items0 && q[1] >= (unsigned)items1 && q[2] >= (unsigned)items2) break;
+    const unsigned run = atomicAdd(&hdr->zero_next, 1u);
+    if (run >= (unsigned)runs) break;
+    const int first = (int)run * kCullRun, last = min(total_n - 1, first + (kCullRun - 1));
+    for (int k = find_seg(tab, first); k < tab->h.n_segs && tseg(tab, k).offset <= last; ++k) {
+      const KSeg& sg = tseg(tab, k);
+      const int lo = max(first, sg.offset), hi = min(last + 1, sg.offset + sg.g.n);
+      if (lo >= hi || !sg.gm) continue;
+      const size_t l = (size_t)(lo - sg.offset), n = (size_t)(hi - lo) * 4;
+      bulk_zero(sg.gsh + l * F, n * F, src, policy);
+      bulk_zero(sg.gq + l * 4, n * 4, src, policy);
+      bulk_zero(sg.gm + l * 3, n * 3, src, policy);
+      bulk_zero(sg.gs + l * 3, n * 3, src, policy);
+      bulk_zero(sg.gl + l, n, src, policy);
+    }
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group 2;" ::: "memory");      // a few runs in flight
+  }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // written before the kernel ends
+}
+
+// Zero gradients of the culled ones of Gaussians base .. base + 31, by one warp.
 template <int DEG>
-__global__ void __launch_bounds__(256) zero_culled_grads(const DevTables* __restrict__ tab, int total_n,
-                                                         const uint32_t* __restrict__ touched) {
-  pdl_enter();
+__device__ __forceinline__ void zero_rows(const DevTables* __restrict__ tab, int total_n,
+                                          const uint32_t* __restrict__ touched, int base, int lane) {
   constexpr int F = 3 * (DEG + 1) * (DEG + 1);
-  const int lane = threadIdx.x & 31;
-  const int base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
   const int i = base + lane;
   bool zero = false;
   float* gsh = nullptr;
@@ -574,6 +630,21 @@ __global__ void __launch_bounds__(256) zero_culled_grads(const DevTables* __rest
       if ((any >> src) & 1u) reinterpret_cast<float*>(p)[f % F] = 0.f;
     }
   }
+}
+
+// Zero gradients of the Gaussians that touch no tile (skipped when accumulating), in the runs that
+// zero_ahead did not take.  A warp owns 32 consecutive Gaussians and writes their SH gradient rows
+// cooperatively, so consecutive lanes store consecutive 16-byte words.
+template <int DEG>
+__global__ void __launch_bounds__(256) zero_culled_grads(const DevTables* __restrict__ tab, int total_n,
+                                                         const uint32_t* __restrict__ touched,
+                                                         const WsHeader* __restrict__ hdr) {
+  constexpr int F = 3 * (DEG + 1) * (DEG + 1);
+  const int lane = threadIdx.x & 31;
+  const long long begin = min((long long)total_n, (long long)hdr->zero_next * kCullRun);
+  for (long long base = begin + ((blockIdx.x * blockDim.x + threadIdx.x) & ~31u); base < total_n;
+       base += (long long)gridDim.x * blockDim.x)
+    zero_rows<DEG>(tab, total_n, touched, (int)base, lane);
 }
 
 // Adjoint of the projection for visible Gaussian i: writes (or, accumulating, adds) the gradients
@@ -809,16 +880,26 @@ cudaError_t launch_records(const DevTables* tab, int total_n, int degree, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_zero_culled(const DevTables* tab, int total_n, int degree, const uint32_t* touched,
-                               cudaStream_t s) {
+cudaError_t launch_zero_ahead(const DevTables* tab, const HostPlan& plan, int total_n, int degree, WsHeader* hdr,
+                              cudaStream_t s) {
   if (total_n == 0) return cudaSuccess;
-  const int zb = (total_n + 255) / 256;
+  const int runs = (total_n - 1) / kCullRun + 1, F = 3 * (degree + 1) * (degree + 1);
+  note_launches(1);
+  zero_ahead<<<std::min(runs, sort_blocks() / 2), 32, 0, s>>>(tab, total_n, F, plan.class_tiles[0], plan.class_tiles[1],
+                                                              plan.class_tiles[2], hdr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_zero_culled(const DevTables* tab, int total_n, int degree, const uint32_t* touched,
+                               const WsHeader* hdr, cudaStream_t s) {
+  if (total_n == 0) return cudaSuccess;
+  const int zb = std::min((total_n - 1) / 256 + 1, 4 * sort_blocks());
   note_launches(1);
   switch (degree) {
-    case 0: zero_culled_grads<0><<<zb, 256, 0, s>>>(tab, total_n, touched); break;
-    case 1: zero_culled_grads<1><<<zb, 256, 0, s>>>(tab, total_n, touched); break;
-    case 2: zero_culled_grads<2><<<zb, 256, 0, s>>>(tab, total_n, touched); break;
-    default: zero_culled_grads<3><<<zb, 256, 0, s>>>(tab, total_n, touched); break;
+    case 0: zero_culled_grads<0><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
+    case 1: zero_culled_grads<1><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
+    case 2: zero_culled_grads<2><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
+    default: zero_culled_grads<3><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
   }
   return cudaGetLastError();
 }
@@ -838,11 +919,15 @@ cudaError_t launch_preprocess_backward(const DevTables* tab, int total_n, int de
   const int per_sm = accumulate ? 4 : 3;
   const int blocks = std::max(1, std::min((total_n + 127) / 128, per_sm * std::max(sms, 1)));
   note_launches(1);
+  auto go = [&](auto kernel) {
+    if (accumulate) launch_pdl(kernel, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc);
+    else kernel<<<blocks, 128, 0, s>>>(tab, vis_ids, hdr, splats, g2d, acc);
+  };
   switch (degree) {
-    case 0: launch_pdl(preprocess_backward_kernel<0>, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc); break;
-    case 1: launch_pdl(preprocess_backward_kernel<1>, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc); break;
-    case 2: launch_pdl(preprocess_backward_kernel<2>, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc); break;
-    default: launch_pdl(preprocess_backward_kernel<3>, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc); break;
+    case 0: go(preprocess_backward_kernel<0>); break;
+    case 1: go(preprocess_backward_kernel<1>); break;
+    case 2: go(preprocess_backward_kernel<2>); break;
+    default: go(preprocess_backward_kernel<3>); break;
   }
   return cudaGetLastError();
 }
