@@ -859,8 +859,9 @@ cudaError_t launch_preprocess(const DevTables* tab, int total_n, uint2* rects, u
   note_launches(2);
   const int runs = (total_n - 1) / kCullRun + 1;
   launch_pdl(cull_kernel, runs, kCullThreads, 0, s, tab, total_n, cp.entries, cp.counts, touched, cp.key_inputs);
-  // a warp a run on small scenes, up to 2 blocks an SM
-  const int blocks = std::max(1, std::min((runs + kCompactThreads / 32 - 1) / (kCompactThreads / 32), sort_blocks()));
+  // a warp a run on small scenes, up to 4 blocks an SM (2 an SM left a block of a merged scene, whose
+  // visible Gaussians sit in few runs, with a long tail: 41 us for four views; more add up more counts)
+  const int blocks = std::max(1, std::min((runs + kCompactThreads / 32 - 1) / (kCompactThreads / 32), 2 * sort_blocks()));
   const int per = (runs + blocks - 1) / blocks;
   launch_pdl(compact_kernel, (runs + per - 1) / per, kCompactThreads, 0, s, cp.entries, cp.counts, runs, per, rects, cp, hdr);
   return cudaGetLastError();
