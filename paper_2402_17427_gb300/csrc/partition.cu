@@ -1,10 +1,13 @@
 // Scene-partition kernels (paper Sec. 4.1 airspace-aware visibility, Sec. 4.3 seamless merging).
 //
 //  - Airspace boxes: per cell, min / max of the points' x and z and max of y, by block
-//    reductions and order-preserving integer atomics (one launch per cell, chunks of 64K points).
-//  - Visibility: one thread per (camera, cell) pair, in FP64: the box is clipped by the near
-//    plane, projected, its convex hull (monotone chain) clipped to the image rectangle
-//    (Sutherland-Hodgman), and the shoelace area divided by the image area.
+//    reductions and order-preserving integer atomics (one launch per 256 cells, chunks of 4K points).
+//  - Visibility: one thread per (camera, cell) pair, in double-floats: the area of the projected box inside the
+//    image rectangle over the image area, as edge integrals: of the silhouette for a box in front of
+//    the near plane, of the faces turned away (clipped by it) for one that the plane cuts.  Where the
+//    faces have no orientation (a singular camera) or the magnitudes are extreme the box is clipped in FP64,
+//    projected, its convex hull (monotone chain) clipped to the image rectangle (Sutherland-Hodgman),
+//    and the shoelace area taken.
 //  - Merge: one pass over all cells' Gaussians.  Blocks take 1,024 Gaussians in ticket order, test
 //    the region, find their output offset by a decoupled look-back over the blocks before them,
 //    and copy the kept Gaussians' parameters straight into the merged arrays.
@@ -32,7 +35,9 @@ __device__ __forceinline__ float ord2f(unsigned o) {
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-constexpr int kBoxChunk = 1 << 14;     // points per block
+// Points per block: 16K made 1,232 blocks of the 20M points of 16 cells, one wave of 8 an SM and a second
+// wave of 16 blocks (53 us); short chunks even that out.
+constexpr int kBoxChunk = 1 << 12;
 constexpr int kBoxCellsPerLaunch = 256;
 
 // Chunk table of one launch: cell c of the launch owns blocks [chunk[c], chunk[c+1]) and points
@@ -63,15 +68,32 @@ __global__ void __launch_bounds__(256) box_reduce(const float* __restrict__ pts,
   const int c = lo_c;
   unsigned v[6] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0u, 0u, 0u};
   const long long lo = (long long)(blockIdx.x - job.chunk[c]) * kBoxChunk;
-  const long long hi = lo + kBoxChunk < job.count[c] ? lo + kBoxChunk : job.count[c];
-  const float* p = pts + 3 * job.first[c];
-  for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+  const int n = (int)(lo + kBoxChunk < job.count[c] ? kBoxChunk : job.count[c] - lo);
+  const float* p = pts + 3 * (job.first[c] + lo);
+  auto put = [&](int a, float f) {
+    const unsigned o = f2ord(f);
+    v[a] = min(v[a], o);
+    v[3 + a] = max(v[3 + a], o);
+  };
+  // four points are three 16-byte words once the address allows (a multiple of 4 bytes plus 12 k, so
+  // after at most three points); the points before that and after the last four by scalar loads
+  int head = 0;
+  while (head < n && head < 4 && (reinterpret_cast<uintptr_t>(p + 3 * head) & 15u)) ++head;
+  const int quads = (n - head) / 4, tail = head + 4 * quads;
+  const int loose = head + (n - tail);
+  if ((int)threadIdx.x < loose) {
+    const int i = (int)threadIdx.x < head ? (int)threadIdx.x : tail + ((int)threadIdx.x - head);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const unsigned o = f2ord(__ldg(p + 3 * i + a));
-      v[a] = min(v[a], o);
-      v[3 + a] = max(v[3 + a], o);
-    }
+    for (int a = 0; a < 3; ++a) put(a, __ldg(p + 3 * i + a));
+  }
+  const float4* w = reinterpret_cast<const float4*>(p + 3 * head);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < quads; i += blockDim.x) {
+    const float4 x = __ldg(w + 3 * i), y = __ldg(w + 3 * i + 1), z = __ldg(w + 3 * i + 2);
+    put(0, x.x); put(1, x.y); put(2, x.z);
+    put(0, x.w); put(1, y.x); put(2, y.y);
+    put(0, y.z); put(1, y.w); put(2, z.x);
+    put(0, z.y); put(1, z.z); put(2, z.w);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -223,16 +245,287 @@ __device__ double box_visibility(const float* box, const vg_camera& cam) {
   return 0.5 * fabs(a2) / (W * H);
 }
 
-__global__ void __launch_bounds__(128) visibility_kernel(const float* __restrict__ boxes, int n_cells,
-                                                         const vg_camera* __restrict__ cams, int n_cams,
-                                                         double threshold, float* out_vis, uint8_t* out_sel) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)n_cams * n_cells) return;
-  const int ci = (int)(idx / n_cells), k = (int)(idx % n_cells);
-  const vg_camera cam = cams[ci];
-  const double v = box_visibility(boxes + 6 * k, cam);
-  if (out_vis) out_vis[idx] = (float)v;
-  if (out_sel) out_sel[idx] = v > threshold ? 1 : 0;
+// Silhouette of a box by which of its faces are turned away from the camera: bit 2a + side for the
+// face of axis a on its lower (0) or upper (1) side.  An edge along axis a, on side kb of axis b and kc
+// of axis c (a, b, c cyclic), lies on the silhouette if just one of its two faces is turned away, and
+// runs along that face's boundary as seen from outside: upwards for face (b, kb) if kb == kc.  Corner k
+// has its x, y, z sides in bits 0, 1, 2.
+struct Silhouette {
+  unsigned char n[64];
+  unsigned char edge[64][6];      // first corner | second corner << 3
+};
+constexpr Silhouette make_silhouettes() {
+  Silhouette t{};
+  for (int mask = 0; mask < 64; ++mask) {
+    int n = 0;
+    unsigned char e[12] = {};
+    for (int a = 0; a < 3; ++a)
+      for (int q = 0; q < 4; ++q) {
+        const int b = (a + 1) % 3, c = (a + 2) % 3, kb = q & 1, kc = q >> 1;
+        const bool away_b = (mask >> (2 * b + kb)) & 1, away_c = (mask >> (2 * c + kc)) & 1;
+        if (away_b == away_c) continue;
+        const int base = (kb << b) | (kc << c), top = base | (1 << a);
+        const bool up = (kb == kc) == away_b;
+        e[n++] = (unsigned char)(up ? base | (top << 3) : top | (base << 3));
+      }
+    // the faces of one axis are never both turned towards a camera outside: other masks are rounding
+    const bool seen = (mask & 3) != 0 && (mask & 12) != 0 && (mask & 48) != 0 && n <= 6;
+    t.n[mask] = (unsigned char)(seen ? n : 0);
+    for (int k = 0; k < 6; ++k) t.edge[mask][k] = seen && k < n ? e[k] : 0;
+  }
+  return t;
+}
+__constant__ Silhouette c_silhouette = make_silhouettes();
+
+// Double-float: a value as an unevaluated sum of two FP32 numbers (48 bits), by the classical
+// error-free transformations (Dekker, Knuth).  An operation is 6 to 20 FP32 instructions; FP64 issues at
+// 1/64 of FP32's rate on this part, so this is the faster way to the ~14 digits the areas need.
+struct dd {
+  float h, l;
+  __device__ dd() {}
+  __device__ dd(float a, float b = 0.f) : h(a), l(b) {}
+};
+__device__ __forceinline__ dd dd_norm(float h, float l) {        // |h| >= |l|
+  const float s = __fadd_rn(h, l);
+  return dd(s, __fsub_rn(l, __fsub_rn(s, h)));
+}
+__device__ __forceinline__ dd operator+(dd a, dd b) {
+  const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+  return dd_norm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ dd operator-(dd a) { return dd(-a.h, -a.l); }
+__device__ __forceinline__ dd operator-(dd a, dd b) { return a + (-b); }
+__device__ __forceinline__ dd operator*(dd a, dd b) {
+  const float p = __fmul_rn(a.h, b.h), e = __fmaf_rn(a.h, b.h, -p);
+  return dd_norm(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e)));
+}
+__device__ __forceinline__ dd operator/(dd a, dd b) {
+  const float q = __fdiv_rn(a.h, b.h);
+  const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));     // a - q b: the first term is exact
+  return dd_norm(q, __fdividef(r, b.h));
+}
+__device__ __forceinline__ bool operator<(dd a, dd b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
+__device__ __forceinline__ bool operator==(dd a, dd b) { return a.h == b.h && a.l == b.l; }
+__device__ __forceinline__ dd dd_clamp(dd v, float lo, float hi) {
+  return v < dd(lo) ? dd(lo) : dd(hi) < v ? dd(hi) : v;
+}
+
+// Signed area between the image of the edge p -> n (camera coordinates, both in front) and the y axis,
+// with x clamped to [-1/2, W - 1/2] and y to [-1/2, H - 1/2]: the integral of clamp(x(y)) dy over the
+// edge.  Summed over a closed polygon's edges it is the signed area of its intersection with that
+// rectangle.  The bounds of y are met in space, where they are linear, not on the image, where the end
+// of an edge beside the camera lies a million pixels off and takes the digits with it.
+__device__ __forceinline__ dd edge_area(const dd* p, const dd* n, const vg_camera& cam) {
+  const float xh = (float)cam.width - 0.5f, yh = (float)cam.height - 0.5f;
+  const dd fx(cam.fx), fy(cam.fy), cx(cam.cx), cy(cam.cy), below = cy + dd(0.5f), above = dd(yh) - cy;
+  const dd ph = fy * p[1], nh = fy * n[1];
+  const dd lo0 = ph + below * p[2], lo1 = nh + below * n[2];       // >= 0: at or above the lower bound
+  const dd hi0 = above * p[2] - ph, hi1 = above * n[2] - nh;       // >= 0: at or below the upper bound
+  if ((lo0.h <= 0.f && lo1.h <= 0.f) || (hi0.h <= 0.f && hi1.h <= 0.f)) return dd(0.f);
+  auto at = [&](const dd* e, dd eh, dd lo, dd hi, dd& x, dd& y) {
+    dd q0 = e[0], q2 = e[2];
+    const bool under = lo.h < 0.f, over = hi.h < 0.f;
+    if (under || over) {
+      const dd t = under ? lo0 / (lo0 - lo1) : hi0 / (hi0 - hi1);
+      q0 = p[0] + t * (n[0] - p[0]);
+      q2 = p[2] + t * (n[2] - p[2]);
+    }
+    x = fx * q0 / q2 + cx;
+    y = under ? dd(-0.5f) : over ? dd(yh) : eh / q2 + cy;
+  };
+  dd xa, ya, xb, yb;
+  at(p, ph, lo0, hi0, xa, ya);
+  at(n, nh, lo1, hi1, xb, yb);
+  const dd dy = yb - ya, ca = dd_clamp(xa, -0.5f, xh), cb = dd_clamp(xb, -0.5f, xh);
+  if (ca == cb) return dy * ca;
+  const dd mean = dd(0.5f) * (ca + cb);
+  if (ca == xa && cb == xb) return dy * mean;
+  // constant before x enters the range at ca and after it leaves at cb; as ca plus a part of cb - ca, so
+  // that an end a million pixels off does not cancel against itself
+  return dy * (ca + (cb - ca) * ((xb - mean) / (xb - xa)));
+}
+
+// A box in camera coordinates: the lower corner and the edges; which faces are turned away (bits as in
+// Silhouette, 0 if that has no meaning here: a singular camera, or magnitudes that double-floats or
+// the areas formed from them would not hold).
+struct CamBox {
+  dd c0[3], e[3][3];
+  int away;
+};
+constexpr float kFarBox = 1e9f, kNearest = 1e-6f, kLongest = 1e7f;   // metres, metres, pixels
+__device__ __forceinline__ CamBox cam_box(const float* __restrict__ box, const vg_camera& cam) {
+  CamBox q;
+  dd lo[3], len[3];
+  float R[3][3], top = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float u = fminf(box[a], box[a + 3]), v = fmaxf(box[a], box[a + 3]);
+    lo[a] = dd(u);
+    len[a] = dd(v) - dd(u);
+    top = fmaxf(top, fmaxf(fabsf(u), fabsf(v)));
+  }
+  bool ok = top < kFarBox && cam.near_plane > kNearest && cam.fx < kLongest && cam.fy < kLongest &&
+            fabsf(cam.cx) < kLongest && fabsf(cam.cy) < kLongest;
+#pragma unroll
+  for (int a = 0; a < 6; ++a) ok = ok && fabsf(box[a]) < kFarBox;     // false for a NaN
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    dd t(cam.world_to_cam[4 * r + 3]);
+    ok = ok && fabsf(t.h) < kFarBox;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      R[a][r] = cam.world_to_cam[4 * r + a];
+      ok = ok && fabsf(R[a][r]) < 1e3f;
+      t = t + dd(R[a][r]) * lo[a];
+      q.e[a][r] = dd(R[a][r]) * len[a];
+    }
+    q.c0[r] = t;
+  }
+  // the camera (the origin) against the planes of each axis's two faces, normal R_b x R_c (so that a
+  // flat box has two faces too, one of them turned away)
+  q.away = 0;
+  dd det(0.f);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float* f = R[(a + 1) % 3];
+    const float* g = R[(a + 2) % 3];
+    dd n[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+      n[r] = dd(f[(r + 1) % 3]) * dd(g[(r + 2) % 3]) - dd(f[(r + 2) % 3]) * dd(g[(r + 1) % 3]);
+    if (a == 0) det = dd(R[0][0]) * n[0] + dd(R[0][1]) * n[1] + dd(R[0][2]) * n[2];
+    const dd s = q.c0[0] * n[0] + q.c0[1] * n[1] + q.c0[2] * n[2], u = s + len[a] * det;
+    const bool lower = det.h > 0.f ? s.h <= 0.f : s.h >= 0.f, upper = det.h > 0.f ? u.h >= 0.f : u.h <= 0.f;
+    q.away |= (lower ? 1 : 0) << (2 * a) | (upper ? 2 : 0) << (2 * a);
+  }
+  if (!ok || !(fabsf(det.h) > 1e-6f)) q.away = 0;
+  return q;
+}
+__device__ __forceinline__ void cam_corner(const CamBox& q, int k, dd* p) {
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    dd v = q.c0[r];
+    if (k & 1) v = v + q.e[0][r];
+    if (k & 2) v = v + q.e[1][r];
+    if (k & 4) v = v + q.e[2][r];
+    p[r] = v;
+  }
+}
+// Signed image area of face `face` (2 axis + side) of a box, clipped by the near plane, if it is turned
+// away from the camera, else 0.  The faces turned away tile the silhouette whether or not the near plane
+// cuts it: what the plane uncovers is seen from inside.
+__device__ dd face_area(const CamBox& q, int face, const vg_camera& cam) {
+  if (!((q.away >> face) & 1)) return dd(0.f);
+  const int b = 1 << ((face >> 1) + 1) % 3, c = 1 << ((face >> 1) + 2) % 3, base = (face & 1) << (face >> 1);
+  const dd near(cam.near_plane);
+  // corners in the order b, c: counter-clockwise from outside on the upper face, clockwise on the lower
+  const int around[4] = {base, base | b, base | b | c, base | c};
+  dd p[3], area(0.f), out[3], in[3];
+  bool cuts = false;
+  cam_corner(q, around[3], p);
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    dd n[3];
+    cam_corner(q, around[k], n);
+    const bool in0 = !(p[2] < near), in1 = !(n[2] < near);
+    if (in0 || in1) {
+      dd u[3] = {p[0], p[1], p[2]}, v[3] = {n[0], n[1], n[2]};
+      if (in0 != in1) {
+        const dd s = (near - p[2]) / (n[2] - p[2]);
+        const dd w[3] = {p[0] + s * (n[0] - p[0]), p[1] + s * (n[1] - p[1]), near};
+        cuts = true;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          if (in0) v[r] = out[r] = w[r];
+          else u[r] = in[r] = w[r];
+        }
+      }
+      area = area + edge_area(u, v, cam);
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) p[r] = n[r];
+  }
+  if (cuts) area = area + edge_area(out, in, cam);       // along the near plane
+  return (face & 1) ? area : -area;
+}
+
+// Bound by instruction issue.  A box wholly in front of the near plane (most) takes no arrays, sorts or
+// hull: eight corners, three cross products, at most six edge integrals.  Boxes that the near plane cuts
+// are gathered, and a block's threads take one face of one of them each, since one such lane would
+// hold up its warp.  All in double-floats: 4,000 cameras x 16 cells took 188 us on the general path in
+// FP64, and 295 us on these paths in FP64 (about 1,000 instructions a pair at 16 clocks a warp).
+constexpr int kVisThreads = 128;
+__global__ void __launch_bounds__(kVisThreads) visibility_kernel(const float* __restrict__ boxes, int n_cells,
+                                                                 const vg_camera* __restrict__ cams, int n_cams,
+                                                                 double threshold, float* out_vis, uint8_t* out_sel) {
+  __shared__ float2 s_p[8][3][kVisThreads];     // corners (boxes in front)
+  __shared__ float2 s_area[6 * kVisThreads];    // faces (boxes that the near plane cuts)
+  __shared__ int s_cut[kVisThreads];
+  __shared__ int s_ncut;
+  if (threadIdx.x == 0) s_ncut = 0;
+  __syncthreads();
+  const long long first = (long long)blockIdx.x * kVisThreads, idx = first + threadIdx.x;
+  const long long pairs = (long long)n_cams * n_cells;
+  auto put = [&](long long i, double v) {
+    if (out_vis) out_vis[i] = (float)v;
+    if (out_sel) out_sel[i] = v > threshold ? 1 : 0;
+  };
+  auto share = [](dd a, const vg_camera& cam) {
+    return fabs((double)a.h + (double)a.l) / ((double)cam.width * (double)cam.height);
+  };
+  if (idx < pairs) {
+    const vg_camera& cam = cams[idx / n_cells];
+    const float* box = boxes + 6 * (idx % n_cells);
+    const CamBox q = cam_box(box, cam);
+    int in = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      dd p[3];
+      cam_corner(q, k, p);
+      in += p[2] < dd(cam.near_plane) ? 0 : 1;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) s_p[k][r][threadIdx.x] = make_float2(p[r].h, p[r].l);
+    }
+    const int edges = c_silhouette.n[q.away];
+    if (q.away == 0) {
+      put(idx, box_visibility(box, cam));
+    } else if (in == 0) {
+      put(idx, 0.0);
+    } else if (in == 8 && edges > 0) {
+      dd area(0.f);
+#pragma unroll 1
+      for (int k = 0; k < edges; ++k) {
+        const int w = c_silhouette.edge[q.away][k];
+        dd p[3], n[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          const float2 a = s_p[w & 7][r][threadIdx.x], b = s_p[w >> 3][r][threadIdx.x];
+          p[r] = dd(a.x, a.y);
+          n[r] = dd(b.x, b.y);
+        }
+        area = area + edge_area(p, n, cam);
+      }
+      put(idx, share(area, cam));
+    } else {
+      s_cut[atomicAdd(&s_ncut, 1)] = threadIdx.x;
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int t = threadIdx.x; t < 6 * s_ncut; t += kVisThreads) {
+    const long long i = first + s_cut[t / 6];
+    const vg_camera& cam = cams[i / n_cells];
+    const dd a = face_area(cam_box(boxes + 6 * (i % n_cells), cam), t % 6, cam);
+    s_area[t] = make_float2(a.h, a.l);
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < s_ncut) {
+    const long long i = first + s_cut[threadIdx.x];
+    dd area(0.f);
+    for (int f = 0; f < 6; ++f) area = area + dd(s_area[6 * threadIdx.x + f].x, s_area[6 * threadIdx.x + f].y);
+    put(i, share(area, cams[i / n_cells]));
+  }
 }
 
 // ---------------------------------------------------------------- merge
@@ -398,8 +691,8 @@ extern "C" vg_status vg_camera_visibility(const float* boxes, int32_t n_cells, c
   if (cudaMemcpyAsync(dcams, cams, sizeof(vg_camera) * (size_t)n_cams, cudaMemcpyHostToDevice, s) != cudaSuccess)
     return VG_ERR_CUDA;
   const long long pairs = (long long)n_cams * n_cells;
-  visibility_kernel<<<(unsigned)((pairs + 127) / 128), 128, 0, s>>>(boxes, n_cells, dcams, n_cams, (double)threshold,
-                                                                   out_visibility, out_selected);
+  visibility_kernel<<<(unsigned)((pairs + kVisThreads - 1) / kVisThreads), kVisThreads, 0, s>>>(
+      boxes, n_cells, dcams, n_cams, (double)threshold, out_visibility, out_selected);
   note_launches(1);
   return cudaGetLastError() == cudaSuccess ? VG_OK : VG_ERR_CUDA;
 }

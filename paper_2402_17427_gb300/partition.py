@@ -47,7 +47,7 @@ def camera_visibility(boxes: torch.Tensor, cameras, threshold: float = VISIBILIT
     sel = torch.empty((len(cams), n_cells), dtype=torch.uint8, device=boxes.device)
     B.vg_camera_visibility(boxes.data_ptr(), n_cells, cams, threshold, ws.data_ptr(), need, vis.data_ptr(),
                            sel.data_ptr(), _stream())
-    return vis, sel.bool()
+    return vis, sel.view(torch.bool)      # 0 or 1 a byte
 
 
 def merge_cells(cells, regions, degree: int):
