@@ -659,37 +659,46 @@ __global__ void __launch_bounds__(256) conv0_embed_grad_kernel(const float* __re
 // the head.
 //
 // The convolutions are implicit GEMMs on the fifth-generation tensor cores (tcgen05.mma,
-// kind::tf32): M = 128 output pixels (an M-tile of 16 rows x 8 columns), N = 16 output channels
-// (conv6's 3 padded with zero weights), K = 9 taps x the input's channels, accumulated in tensor
-// memory.  Every operand is split into two TF32 parts, x = hi + lo with hi = tf32(x) and
-// lo = tf32(x - hi), and each product is formed as lo.hi + hi.lo + hi.hi, so the products are
-// FP32-accurate (relative error about 2^-21; the dropped lo.lo term is below FP32 rounding).
+// kind::tf32), accumulated in tensor memory.  Every operand is split into two TF32 parts, x = hi + lo
+// with hi = tf32(x) and lo = tf32(x - hi), and each product is formed as lo.hi + hi.lo + hi.hi, so the
+// products are FP32-accurate (relative error about 2^-21; the dropped lo.lo term is below FP32 rounding).
+//
+// What bounds them is the shared-memory traffic of the activation operand, so one read of it serves as
+// many products as possible: M = 128 input pixels (4 rows of 32), K = the 3 rows of taps x the input's
+// channels, and N holds all three columns of taps, 3 x NO outputs, hi and lo weights side by side:
+//   D[p][dx][o] = sum over dy, c of X(y + dy - 1, x)[c] W[o][c][dy][dx],
+// one MMA with A_hi against [W_hi | W_lo] and one with A_lo against W_hi into the second half.  The
+// epilogue adds the halves and gathers the taps, out(y, x) = sum over dx of D[(y, x + dx - 1)][dx]: lanes are
+// consecutive pixels of a row, so the neighbours' parts come by one shuffle each and 30 of a row's
+// 32 pixels are outputs.  With the nine taps one after another (N = 32, the activations read 18 times
+// instead of 6 for 16 channels) a pass at 1080p took 119 us.
 //
 // Shared-memory operands use the no-swizzle K-major layout: a core matrix is 8 rows of 16 bytes
-// (4 channels), rows 16 bytes apart.  The input patch of an M-tile (18 x 10 pixels with its halo)
-// is stored as [part][channel group][18][10][4 floats], so the 8 pixels of one output row segment
-// are one core matrix, the next output row is 160 bytes further (the stride between core matrices
-// along M) and the next channel group one plane further (the stride along K); a tap (dy, dx) only
-// moves the start address by (10 dy + dx) x 16 bytes.  Weights are [tap][group][part][16][4]: for
-// one tap and channel group the hi rows are followed by the lo rows, so that one N = 32 operand
-// holds [W_hi | W_lo] and a k-step takes two MMAs, A_hi [W_hi | W_lo] into accumulator columns
-// 0..31 and A_lo W_hi into columns 16..31 (the products hi.hi | hi.lo + lo.hi), reading each part
-// of the activations from shared memory once; the epilogue adds the two halves.
+// (4 channels).  The patch (10 rows x 32 pixels for 8 rows of outputs) is stored [part][channel
+// group][10][32][4 floats]: core matrices follow one another along M, the next channel group is one
+// plane further, a tap row dy moves the start address by 512 bytes.  Planes are 128 / groups bytes
+// longer than their data, so that the groups of the pixels that eight lanes write fall on distinct banks.
+// Weights are [dy][group][part][dx][o][4 channels].
 
-constexpr int kTcThreads = 128;                      // four warps: staging, epilogue; one thread issues
-constexpr int kTcRows = 16, kTcCols = 8;             // output pixels of an M-tile
-constexpr int kPatchH = kTcRows + 2, kPatchW = kTcCols + 2, kPatchPx = kPatchH * kPatchW;
-constexpr uint32_t kPatchPlane = kPatchPx * 16;      // bytes of one channel group of a patch part
+constexpr int kTcThreads = 256;                      // eight warps, an output row each; one thread issues
+constexpr int kTcRows = 8, kTcCols = 30;             // outputs of a tile (two M-tiles of 4 rows x 32 pixels)
+constexpr int kPatchH = kTcRows + 2, kPatchW = 32, kPatchPx = kPatchH * kPatchW;
 constexpr uint64_t kTcWaitNs = 1000000000ull;        // bounded wait for the MMAs of one tile (1 s)
 enum : int { kEpiRelu = 0, kEpiL1 = 1, kEpiMask = 2, kEpiStore = 3 };
 
-template <int C>
+template <int C, int NO>
 struct TcShape {
   static constexpr int CG = C / 4;                           // channel groups (K = 8 per MMA: 2 groups)
-  static constexpr uint32_t PartA = CG * kPatchPlane;
+  static constexpr int N1 = 3 * NO;                          // outputs of the three tap columns
+  static constexpr int N2 = (N1 + 15) / 16 * 16;             // N of the A_lo MMA (past N1: columns nobody reads)
+  static constexpr uint32_t Plane = kPatchPx * 16 + 128 / CG;   // one channel group of a patch part
+  static constexpr uint32_t PartA = CG * Plane;
   static constexpr uint32_t BufA = 2 * PartA;                // hi and lo parts of one patch
-  static constexpr uint32_t SizeB = 9 * CG * 2 * 16 * 16;    // the weights, both parts
+  static constexpr uint32_t GroupB = 2 * N1 * 16;            // one tap row and channel group, both parts
+  static constexpr uint32_t SizeB = 3 * CG * GroupB;
   static constexpr uint32_t Smem = 2 * BufA + SizeB;         // two patch buffers + weights
+  static constexpr uint32_t Acc = N1 + N2 <= 64 ? 64 : 128;  // tensor-memory columns of an M-tile
+  static_assert(2 * N1 % 16 == 0 && N1 + N2 <= Acc, "accumulator layout");
 };
 
 struct TcArgs {
@@ -700,7 +709,7 @@ struct TcArgs {
   const float* act;                // kEpiMask: Hh
   float* out;                      // Hh, gM', gZ5' or gU (null: not written)
   float *map, *gimg;               // kEpiL1 (null: not written)
-  float* dbias;                    // kEpiL1: db6, kEpiMask: db5 (null: not formed)
+  float* dbias;                    // kEpiL1, kEpiMask: a row of 16 sums for each CTA (null: not formed)
   double* partials;                // kEpiL1: the L1 sum of each CTA
   unsigned* status;                // bit 0: a bounded wait gave up
   int H, W, tiles_x, tiles, wo, wc;     // wo x wc: the layer's output x input channels
@@ -715,11 +724,11 @@ __device__ __forceinline__ float4 split_lo(float4 v, float4 h) {
 
 // B[n][tap][k]: forward W[n][k][tap]; adjoint W[k][n][8 - tap] (n = the layer's input channel).
 // Entries past the layer's channels are zero.
-template <int C>
+template <int C, int NO>
 __device__ void tc_stage_weights(unsigned char* sB, const TcArgs& a) {
-  using S = TcShape<C>;
-  for (int i = threadIdx.x; i < 9 * S::CG * 16; i += kTcThreads) {
-    const int n = i & 15, cg = (i >> 4) % S::CG, tap = i / (16 * S::CG);
+  using S = TcShape<C, NO>;
+  for (int i = threadIdx.x; i < 9 * S::CG * NO; i += kTcThreads) {
+    const int n = i % NO, cg = (i / NO) % S::CG, tap = i / (NO * S::CG);
     float v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -728,15 +737,15 @@ __device__ void tc_stage_weights(unsigned char* sB, const TcArgs& a) {
       else v[j] = (k < a.wo && n < a.wc) ? __ldg(a.w + ((size_t)k * a.wc + n) * 9 + (8 - tap)) : 0.f;
     }
     const float4 x = make_float4(v[0], v[1], v[2], v[3]), h = split_hi(x);
-    const uint32_t off = (uint32_t)(((tap * S::CG + cg) * 32 + n) * 16);
+    const uint32_t off = (uint32_t)((tap / 3) * S::CG + cg) * S::GroupB + (uint32_t)((tap % 3) * NO + n) * 16;
     *reinterpret_cast<float4*>(sB + off) = h;
-    *reinterpret_cast<float4*>(sB + off + 256) = split_lo(x, h);
+    *reinterpret_cast<float4*>(sB + off + S::N1 * 16) = split_lo(x, h);
   }
 }
 
-// The M-tile's input patch, rows Y0 - 1 .. Y0 + 16 and columns X0 - 1 .. X0 + 8, zero outside the
-// image: loaded into registers (tc_load_patch, issued a tile ahead so that the loads are in flight
-// while the previous tile's epilogue runs), then split into its two TF32 parts in shared memory.
+// The tile's input patch, rows Y0 - 1 .. Y0 + 8 and columns X0 - 1 .. X0 + 30, zero outside the
+// image: loaded into registers (tc_load_patch, issued a tile ahead), then split into its two TF32
+// parts in shared memory.
 template <int C>
 struct TcPatch {
   static constexpr int N = kPatchPx * (C / 4), IT = (N + kTcThreads - 1) / kTcThreads;
@@ -756,39 +765,39 @@ __device__ __forceinline__ void tc_load_patch(TcPatch<C>& r, const float* __rest
       r.v[q] = __ldg(reinterpret_cast<const float4*>(in + ((size_t)Y * W + X) * C) + cg);
   }
 }
-template <int C>
+template <int C, int NO>
 __device__ __forceinline__ void tc_store_patch(unsigned char* sA, const TcPatch<C>& r) {
-  using S = TcShape<C>;
+  using S = TcShape<C, NO>;
 #pragma unroll
   for (int q = 0; q < TcPatch<C>::IT; ++q) {
     const int i = threadIdx.x + kTcThreads * q;
     if (i >= TcPatch<C>::N) continue;
     const int px = i / S::CG, cg = i % S::CG;
-    const uint32_t off = (uint32_t)cg * kPatchPlane + (uint32_t)px * 16;
+    const uint32_t off = (uint32_t)cg * S::Plane + (uint32_t)px * 16;
     const float4 h = split_hi(r.v[q]);
     *reinterpret_cast<float4*>(sA + off) = h;
     *reinterpret_cast<float4*>(sA + S::PartA + off) = split_lo(r.v[q], h);
   }
 }
 
-// The MMAs of one M-tile: 9 taps x C / 8 k-steps x 2 into the 32-column accumulator d.  The
-// descriptors of the patch buffer's and the weights' first core matrices are formed once; an
-// operand's offset only adds to the start-address field (16-byte units, no carry: shared
-// addresses stay below 2^18).
-template <int C>
+// The MMAs of one tile: two M-tiles x 3 tap rows x C / 8 k-steps x 2.  The descriptors of the patch
+// buffer's and the weights' first core matrices are formed once; an operand's offset only adds to the
+// start-address field (16-byte units, no carry: shared addresses stay below 2^18).
+template <int C, int NO>
 __device__ __forceinline__ void tc_issue(uint64_t a_hi, uint64_t b_desc, uint32_t d) {
-  using S = TcShape<C>;
-  constexpr uint32_t idesc32 = tc::idesc_tf32(128, 32), idesc16 = tc::idesc_tf32(128, 16);
+  using S = TcShape<C, NO>;
+  constexpr uint32_t idesc_hi = tc::idesc_tf32(128, 2 * S::N1), idesc_lo = tc::idesc_tf32(128, S::N2);
 #pragma unroll
-  for (int tap = 0; tap < 9; ++tap) {
+  for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int ks = 0; ks < C / 8; ++ks) {
-      const uint64_t ao = (2 * ks * kPatchPlane + (uint32_t)((tap / 3) * kPatchW + tap % 3) * 16) >> 4;
-      const uint64_t bo = (uint64_t)((tap * S::CG + 2 * ks) * 512) >> 4;
-      tc::mma_tf32(d, a_hi + ao, b_desc + bo, idesc32, tap + ks > 0);                    // A_hi [W_hi | W_lo]
-      tc::mma_tf32(d + 16, a_hi + ao + (S::PartA >> 4), b_desc + bo, idesc16, true);     // A_lo W_hi
-    }
-  }
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+      for (int ks = 0; ks < C / 8; ++ks) {
+        const uint64_t ao = (2 * ks * S::Plane + (uint32_t)(4 * mt + dy) * kPatchW * 16) >> 4;
+        const uint64_t bo = (uint64_t)((dy * S::CG + 2 * ks) * S::GroupB) >> 4;
+        tc::mma_tf32(d + mt * S::Acc, a_hi + ao, b_desc + bo, idesc_hi, dy + ks > 0);                       // A_hi [W_hi | W_lo]
+        tc::mma_tf32(d + mt * S::Acc + S::N1, a_hi + ao + (S::PartA >> 4), b_desc + bo, idesc_lo, true);    // A_lo W_hi
+      }
 }
 
 // Per-thread sums the epilogues carry across tiles.
@@ -797,17 +806,18 @@ struct TcSums {
   float db[16] = {};
 };
 
-// The epilogue's other inputs at the thread's pixel, loaded a tile ahead: Hh (kEpiMask) or I_r
-// and I (kEpiL1).
+// The epilogue's other inputs at the thread's pixel, loaded before the wait for the MMAs: Hh (kEpiMask)
+// or I_r and I (kEpiL1).
 struct TcEpiIn {
   float4 x[4];
 };
 
+// The thread's output pixel: row = warp, column = lane - 1 (lanes 0 and 31 only feed their neighbours).
 __device__ __forceinline__ bool tc_pixel(const TcArgs& a, int tile, int& Y, int& X) {
-  const int m = threadIdx.x;      // accumulator row = lane of tensor memory = this thread
-  Y = (tile / a.tiles_x) * kTcRows + (m >> 3);
-  X = (tile % a.tiles_x) * kTcCols + (m & 7);
-  return Y < a.H && X < a.W;
+  const int lane = threadIdx.x & 31;
+  Y = (tile / a.tiles_x) * kTcRows + (int)(threadIdx.x >> 5);
+  X = (tile % a.tiles_x) * kTcCols + lane - 1;
+  return lane >= 1 && lane <= kTcCols && Y < a.H && X < a.W;
 }
 
 template <int EPI>
@@ -825,20 +835,42 @@ __device__ __forceinline__ void tc_load_epi(const TcArgs& a, int tile, TcEpiIn& 
   }
 }
 
-// Epilogue of one M-tile: waits for its MMAs, reads the thread's accumulator row (row m = 32 warp +
-// lane = the thread index) and applies the layer's output step.  Returns false if the wait gave up.
-template <int EPI>
-__device__ __forceinline__ bool tc_epilogue(const TcArgs& a, int tile, uint32_t tm, uint64_t* mbar, uint32_t parity,
+// hi.hi + (hi.lo + lo.hi) of one tap column at the thread's accumulator row.
+__device__ __forceinline__ void tc_column(uint32_t tm, float (&v)[16], int n1) {
+  float w[16];
+  tc::ld16(tm, v);
+  tc::ld16(tm + n1, w);
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] += w[j];
+}
+__device__ __forceinline__ void tc_column(uint32_t tm, float (&v)[8], int n1) {
+  float w[8];
+  tc::ld8(tm, v);
+  tc::ld8(tm + n1, w);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] += w[j];
+}
+
+// Epilogue of one tile: waits for its MMAs, gathers the thread's pixel from the three tap columns and
+// applies the layer's output step.  Returns false if the wait gave up.
+template <int C, int NO, int EPI>
+__device__ __forceinline__ bool tc_epilogue(const TcArgs& a, int tile, uint32_t tmem, uint64_t* mbar, uint32_t parity,
                                             const TcEpiIn& e, TcSums& sums) {
+  using S = TcShape<C, NO>;
   const int warp = threadIdx.x >> 5;
   const bool ok = tc::mbar_wait(mbar, parity, kTcWaitNs);
   __syncwarp();
   tc::fence_after_sync();
-  float v[16], w[16];
-  tc::ld16(tm + ((uint32_t)(32 * warp) << 16), v);
-  tc::ld16(tm + ((uint32_t)(32 * warp) << 16) + 16u, w);
+  // row m of M-tile mt is lane m of tensor memory; a warp reads its quarter of the lanes
+  const uint32_t tm = tmem + (uint32_t)(warp >> 2) * S::Acc + ((uint32_t)(32 * (warp & 3)) << 16);
+  float v[NO], t[NO];
+  tc_column(tm + NO, v, S::N1);                     // dx = 1: the pixel's own column
+  tc_column(tm, t, S::N1);                          // dx = 0: from the column to the left
 #pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] += w[j];      // hi.hi + (hi.lo + lo.hi)
+  for (int j = 0; j < NO; ++j) v[j] += __shfl_up_sync(0xffffffffu, t[j], 1);
+  tc_column(tm + 2 * NO, t, S::N1);                 // dx = 2: from the column to the right
+#pragma unroll
+  for (int j = 0; j < NO; ++j) v[j] += __shfl_down_sync(0xffffffffu, t[j], 1);
   int Y, X;
   if (!tc_pixel(a, tile, Y, X) || !ok) return ok;
   const size_t pix = (size_t)Y * a.W + X;
@@ -890,88 +922,105 @@ __device__ __forceinline__ bool tc_epilogue(const TcArgs& a, int tile, uint32_t 
   return true;
 }
 
-template <int C, int EPI>
-__global__ void __launch_bounds__(kTcThreads) tc_conv_kernel(const TcArgs a) {
-  using S = TcShape<C>;
+template <int C, int NO, int EPI>
+__global__ void __launch_bounds__(kTcThreads, 2) tc_conv_kernel(const TcArgs a) {
+  using S = TcShape<C, NO>;
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   unsigned char* sA = tc_smem;                 // two patch buffers
   unsigned char* sB = tc_smem + 2 * S::BufA;   // the weights
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tslot;
   __shared__ double red[kTcThreads / 32];
+  __shared__ float s_db[kTcThreads / 32][16];
   const int tid = threadIdx.x, warp = tid >> 5;
-  if (warp == 0) tc::alloc(&tslot, 64);        // two 32-column accumulators
+  if (warp == 0) tc::alloc(&tslot, 2 * S::Acc);
   if (tid == 0) {
-    tc::mbar_init(&mbar[0], 1);
-    tc::mbar_init(&mbar[1], 1);
+    tc::mbar_init(&mbar, 1);
     tc::mbar_init_fence();
   }
+  auto load = [&](TcPatch<C>& p, int t) {
+    if (t < a.tiles) tc_load_patch<C>(p, a.in, (t / a.tiles_x) * kTcRows, (t % a.tiles_x) * kTcCols, a.H, a.W);
+  };
   TcPatch<C> pre;
-  TcEpiIn epi_next, epi_prev;
+  TcEpiIn epi;
   int tile = blockIdx.x;
-  if (tile < a.tiles) tc_load_patch<C>(pre, a.in, (tile / a.tiles_x) * kTcRows, (tile % a.tiles_x) * kTcCols, a.H, a.W);
-  tc_stage_weights<C>(sB, a);
+  load(pre, tile);
+  tc_stage_weights<C, NO>(sB, a);
+  if (tile < a.tiles) tc_store_patch<C, NO>(sA, pre);
+  load(pre, tile + gridDim.x);
+  tc::fence_smem_to_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tslot;
-  const uint64_t a_desc = tc::desc(smem_u32(sA), kPatchPlane, kPatchW * 16);
-  const uint64_t b_desc = tc::desc(smem_u32(sB), 512, 128);
+  const uint64_t a_desc = tc::desc(smem_u32(sA), S::Plane, 128);
+  const uint64_t b_desc = tc::desc(smem_u32(sB), S::GroupB, 128);
   TcSums sums;
   bool ok = true;
-  int k = 0, prev = -1;
-  // tile k is staged into buffer k & 1 and accumulated in columns 32 (k & 1); its epilogue runs
-  // in iteration k + 1, while the MMAs of tile k + 1 execute and the patch of tile k + 2 loads
+  int k = 0;
+  // Tile k's patch is in buffer k & 1.  While its MMAs run, tile k + 1's patch goes to the other buffer
+  // (its last reader's MMAs were waited for) and tile k + 2's loads start; the epilogue then overlaps
+  // the MMAs of the SM's other CTA.
   for (; tile < a.tiles; tile += gridDim.x, ++k) {
     const int b = k & 1;
-    tc_store_patch<C>(sA + b * S::BufA, pre);
-    tc::fence_smem_to_async();
-    tc::fence_before_sync();
-    __syncthreads();
     if (tid == 0) {
       tc::fence_after_sync();
-      tc_issue<C>(a_desc + ((b * S::BufA) >> 4), b_desc, tmem + 32u * b);
-      tc::commit(&mbar[b]);
+      tc_issue<C, NO>(a_desc + ((b * S::BufA) >> 4), b_desc, tmem);
+      tc::commit(&mbar);
     }
-    const int next = tile + gridDim.x;
-    if (next < a.tiles) tc_load_patch<C>(pre, a.in, (next / a.tiles_x) * kTcRows, (next % a.tiles_x) * kTcCols, a.H, a.W);
-    tc_load_epi<EPI>(a, tile, epi_next);
-    if (prev >= 0) ok &= tc_epilogue<EPI>(a, prev, tmem + 32u * (b ^ 1), &mbar[b ^ 1], ((k - 1) >> 1) & 1, epi_prev, sums);
-    epi_prev = epi_next;
-    prev = tile;
+    if (tile + gridDim.x < a.tiles) tc_store_patch<C, NO>(sA + (b ^ 1) * S::BufA, pre);
+    load(pre, tile + 2 * gridDim.x);
+    tc_load_epi<EPI>(a, tile, epi);
+    ok &= tc_epilogue<C, NO, EPI>(a, tile, tmem, &mbar, k & 1, epi, sums);
+    tc::fence_smem_to_async();
+    tc::fence_before_sync();
+    __syncthreads();             // accumulators read, the next patch written
   }
-  if (prev >= 0)
-    ok &= tc_epilogue<EPI>(a, prev, tmem + 32u * ((k - 1) & 1), &mbar[(k - 1) & 1], ((k - 1) >> 1) & 1, epi_prev, sums);
   if (!ok) {
     atomicOr(a.status, 1u);
-    // the last commit of each buffer, waited for again (bounded) before the memory is freed
-    for (int j = 1; j <= 2 && k - j >= 0; ++j) tc::mbar_wait(&mbar[(k - j) & 1], ((k - j) >> 1) & 1, kTcWaitNs);
+    tc::mbar_wait(&mbar, (k - 1) & 1, kTcWaitNs);     // the last commit, waited for again (bounded) before the memory is freed
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::dealloc(tmem, 64);
-  // the per-CTA sums of the epilogue
+  if (warp == 0) tc::dealloc(tmem, 2 * S::Acc);
+  // the CTA's sums of the epilogue, one row each (added up by sum_rows_kernel: additions of every warp
+  // to 16 words took 40 us of the 50 us pass at 330 x 200)
   const int lane = tid & 31;
   if constexpr (EPI == kEpiL1) {
     const float l = warp_sum(sums.l1);
     if (lane == 0) red[warp] = (double)l;
+  }
+  if constexpr (EPI == kEpiL1 || EPI == kEpiMask) {
+    constexpr int NB = EPI == kEpiL1 ? 3 : 16;
+#pragma unroll
+    for (int o = 0; o < NB; ++o) {
+      const float s = warp_sum(sums.db[o]);
+      if (lane == 0) s_db[warp][o] = s;
+    }
     __syncthreads();
-    if (tid == 0) {
+    if (EPI == kEpiL1 && tid == 0) {
       double s = 0;
       for (int w = 0; w < kTcThreads / 32; ++w) s += red[w];
       a.partials[blockIdx.x] = s;
     }
-  }
-  if constexpr (EPI == kEpiL1 || EPI == kEpiMask) {
-    if (a.dbias) {
-      constexpr int NB = EPI == kEpiL1 ? 3 : 16;
+    if (a.dbias && tid < NB) {
+      float s = 0.f;
 #pragma unroll
-      for (int o = 0; o < NB; ++o) {
-        const float s = warp_sum(sums.db[o]);
-        if (lane == 0) atomicAdd(a.dbias + o, a.cscale * s);
-      }
+      for (int w = 0; w < kTcThreads / 32; ++w) s += s_db[w][tid];
+      a.dbias[(size_t)blockIdx.x * 16 + tid] = s;
     }
   }
+}
+
+// db[o] = scale * the sum of column o of `rows` rows of 16: a warp a column.
+__global__ void __launch_bounds__(512) sum_rows_kernel(const float* __restrict__ part, int rows, int cols, float scale,
+                                                       float* __restrict__ db) {
+  const int o = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (o >= cols) return;
+  float s = 0.f;
+  for (int r = lane; r < rows; r += 32) s += __ldg(part + (size_t)r * 16 + o);
+  s = warp_sum(s);
+  if (lane == 0) db[o] = scale * s;
 }
 
 // Bilinear up-sampling from n_in to n_out samples: output y reads rows i0 and i1 with weight f
@@ -1247,12 +1296,12 @@ __global__ void __launch_bounds__(256) appearance_finalize(const double* __restr
 
 // Workspace regions (floats unless noted), for an H x W image with (h, w) = (H / 32, W / 32).
 struct AppLayout {
-  size_t E, G, P, gP, A[5], gA[5], U, Hh, gM, gZ, gU, gX, taps, packed, maps, ssim_part, head_part, status, total;
+  size_t E, G, P, gP, A[5], gA[5], U, Hh, gM, gZ, gU, gX, taps, packed, maps, ssim_part, head_part, db5, db6, status, total;
   int pack_off[kPackJobs];
   PackTable tab;
 };
 
-constexpr int kMaxHeadBlocks = 4096;
+constexpr int kMaxHeadBlocks = 1024;
 
 // Block k's channels: C_k = layer_c(k) inputs, O_k = layer_o(k) outputs; A_k at (2^k h, 2^k w).
 AppLayout make_app_layout(int W, int H) {
@@ -1305,6 +1354,8 @@ AppLayout make_app_layout(int W, int H) {
   L.maps = take(ssim_maps_floats(W, H) * 4);
   L.ssim_part = take((size_t)ssim_partials(W, H) * 2 * 8);
   L.head_part = take((size_t)kMaxHeadBlocks * 8);
+  L.db5 = take((size_t)kMaxHeadBlocks * 16 * 4);    // rows of bias-gradient sums of the two passes
+  L.db6 = take((size_t)kMaxHeadBlocks * 16 * 4);
   L.status = take(16);
   L.total = off;
   return L;
@@ -1356,18 +1407,16 @@ cudaError_t launch_wgrad(const float* Aprev, const float* gA, const float* A, fl
   return cudaGetLastError();
 }
 
-// One persistent pass of a head convolution: as many CTAs as the shared memory and the registers
-// of an SM hold (at most 6; their tensor memory, 64 columns each, stays within the 512 of an SM), at most one
-// per M-tile.
-template <int C, int EPI>
+// One persistent pass of a head convolution: two CTAs an SM (their tensor memory, at most 256 columns
+// each, fills the 512 of an SM), at most one per tile.
+template <int C, int NO, int EPI>
 cudaError_t launch_tc_conv(const TcArgs& a, int sms, cudaStream_t s, int* grid_out = nullptr) {
-  using S = TcShape<C>;
-  auto k = tc_conv_kernel<C, EPI>;
+  using S = TcShape<C, NO>;
+  auto k = tc_conv_kernel<C, NO, EPI>;
   cudaError_t e = set_smem(k, S::Smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
-  const int per_sm = resident_per_sm(k, kTcThreads, S::Smem, 6);
-  const int grid = std::max(1, std::min({a.tiles, per_sm * sms, kMaxHeadBlocks}));
+  const int grid = std::max(1, std::min({a.tiles, 2 * sms, kMaxHeadBlocks}));
   if (grid_out) *grid_out = grid;
   note_launches(1);
   k<<<grid, kTcThreads, S::Smem, s>>>(a);
@@ -1505,7 +1554,7 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
     c5.bias = params + b_off(5);
     c5.out = Hh;
     c5.wo = 16;
-    ok(launch_tc_conv<16, kEpiRelu>(c5, sms, s));
+    ok(launch_tc_conv<16, 16, kEpiRelu>(c5, sms, s));
     TcArgs c6 = ta;
     c6.in = Hh;
     c6.w = params + w_off(6);
@@ -1515,10 +1564,10 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
     c6.map = out_map;
     c6.gimg = grad_img;
     c6.out = bwd ? F(L.gM) : nullptr;
-    c6.dbias = bwd ? grad_params + b_off(6) : nullptr;
+    c6.dbias = bwd ? F(L.db6) : nullptr;
     c6.partials = head_part;
     c6.wo = 3;
-    ok(launch_tc_conv<16, kEpiL1>(c6, sms, s, &nhead));
+    ok(launch_tc_conv<16, 8, kEpiL1>(c6, sms, s, &nhead));
   }
   ok(link(E, side, s));      // the SSIM partials and maps
   appearance_finalize<<<1, 256, 0, s>>>(ssim_part, ssim_partials(W, H), head_part, nhead, inv, lambda, status, out_loss);
@@ -1532,11 +1581,15 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
     a6.w = params + w_off(6);
     a6.act = Hh;
     a6.out = F(L.gZ);
-    a6.dbias = gp + b_off(5);
+    a6.dbias = F(L.db5);
     a6.wo = 3;
     a6.adjoint = true;
-    ok(launch_tc_conv<8, kEpiMask>(a6, sms, s));
+    int n6 = 0;
+    ok(launch_tc_conv<8, 16, kEpiMask>(a6, sms, s, &n6));
     ok(link(E, s, sd[1]));
+    note_launches(2);
+    sum_rows_kernel<<<1, 512, 0, sd[1]>>>(F(L.db5), n6, 16, ta.cscale, gp + b_off(5));
+    sum_rows_kernel<<<1, 512, 0, sd[1]>>>(F(L.db6), nhead, 3, ta.cscale, gp + b_off(6));
     ok(launch_head_wgrad<16, 16, 4>(U, F(L.gZ), H, W, ta.cscale, gp + w_off(5), sms, sd[1]));
     ok(launch_head_wgrad<8, 3, 8>(Hh, F(L.gM), H, W, ta.cscale, gp + w_off(6), sms, sd[1]));
     TcArgs a5 = ta;
@@ -1545,7 +1598,7 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
     a5.out = F(L.gU);
     a5.wo = 16;
     a5.adjoint = true;
-    ok(launch_tc_conv<16, kEpiStore>(a5, sms, s));
+    ok(launch_tc_conv<16, 16, kEpiStore>(a5, sms, s));
     note_launches(2);
     const size_t n1 = (size_t)H * w4 * 4, n2 = (size_t)w4 * h4 * 4;
     upsample_adjoint_kernel<false><<<(unsigned)((n1 + 255) / 256), 256, 0, s>>>(
