@@ -279,37 +279,52 @@ __device__ __forceinline__ void stage_plain(float* dst, const float* __restrict_
   }
 }
 
-// One block computes MT rows x 16 columns of output pixels and all O channels.  The input tile
-// ((MT + 2) x 18 pixels x C channels, pitch C + 4 so that the 8 x 4 lanes of a fragment load hit
-// distinct banks) is staged once; the packed weights of one tap (C x O floats) at a time follow
-// it into shared memory with cp.async, double-buffered so that the next tap's copy overlaps the
-// current tap's MMAs.  Warps form WM x (8 / WM): each owns MT / WM pixel rows (m-tiles) and
-// O / 8 / (8 / WM) n-tiles.
+// One block computes MT rows x 16 columns of output pixels and OB of the O channels (blockIdx.z).  The
+// input tile ((MT + 2) x 18 pixels x C channels, pitch C + 4 so that the 8 x 4 lanes of a fragment load
+// hit distinct banks) is staged once; the packed weights follow it into shared memory with cp.async:
+// all nine taps at once where they fit (ALL: one wait and one barrier), else one tap (C x OB floats) at a
+// time, double-buffered.  Warps form WM x (8 / WM): each owns MT / WM pixel rows (m-tiles) and
+// OB / 8 / (8 / WM) n-tiles.
+//
+// Small images leave few tiles (2 x 3 for the first block of a 330 x 200 view): the channels are then split
+// over blocks as far as a warp keeps one n-tile, which shortens the serial chain of taps (first forward
+// convolution 31 -> 18 us, last input gradient 37 -> 20 us).  On large ones (8 x 17 tiles at 1080p) all
+// channels stay in one block, since every split loads and splits the activations again (33 against 49 us).
 //  forward (DGRAD false): input = shuffle(in) with in [Hr/2][Wr/2][4C]; output ReLU(acc + b) ->
 //    out [Hr][Wr][O].
 //  input gradient (DGRAD true): input = in [Hr][Wr][C], the output gradient of the block (times
 //    [act > 0] when MASK_IN; otherwise already masked); output = the gradient of the shuffled input
 //    (O channels), written in the previous layer's layout [Hr/2][Wr/2][4 O] and, when MASK_OUT,
 //    times [aout > 0] (that layer's ReLU).
-template <int C, int O, int MT, int WM, bool DGRAD, bool MASK_IN, bool MASK_OUT>
+template <int C, int OB>
+struct ConvShape {
+  static constexpr int TapF = C * OB;                               // packed weight floats of one tap
+  static constexpr bool All = 9 * TapF * sizeof(float) <= 75 * 1024;
+  static constexpr int Buffers = All ? 9 : 2;
+};
+template <int C, int O, int OB, int MT, int WM, bool DGRAD, bool MASK_IN, bool MASK_OUT>
 __global__ void __launch_bounds__(256) conv_mma_kernel(const float* __restrict__ in, const float* __restrict__ act,
                                                        const float* __restrict__ wpk, const float* __restrict__ bias,
                                                        const float* __restrict__ aout, float* __restrict__ out, int Hr,
                                                        int Wr) {
-  constexpr int NT = O / 8, WN = 8 / WM, NTW = NT / WN, MTW = MT / WM;
+  using W = ConvShape<C, OB>;
+  constexpr int NT = OB / 8, WN = 8 / WM, NTW = NT / WN, MTW = MT / WM;
   constexpr int PITCH = C + 4, SW = 18, SHT = MT + 2;
-  constexpr int TAPF = C * O;                      // packed weight floats of one tap
-  static_assert(NT % WN == 0 && MT % WM == 0 && C % 8 == 0, "tiling");
+  static_assert(O % OB == 0 && NT % WN == 0 && MT % WM == 0 && C % 8 == 0, "tiling");
   extern __shared__ __align__(16) float smem[];
-  float* wbuf = smem + SHT * SW * PITCH;           // [2][TAPF]
-  const int ox = blockIdx.x * 16, oy = blockIdx.y * MT;
-  auto fetch_tap = [&](int tap) {
-    float* dst = wbuf + (tap & 1) * TAPF;
-    const float* src = wpk + (size_t)tap * TAPF;
-    for (int i = threadIdx.x; i < TAPF / 4; i += 256) cp_async16(dst + 4 * i, src + 4 * i);
+  float* wbuf = smem + SHT * SW * PITCH;           // [Buffers][TapF]
+  const int ox = blockIdx.x * 16, oy = blockIdx.y * MT, n0 = blockIdx.z * NT;   // n0: the block's first n-tile
+  auto fetch_tap = [&](int tap) {                  // of each k-step (8 channels) the block's n-tiles
+    float* dst = wbuf + (W::All ? tap : tap & 1) * W::TapF;
+    const float* src = wpk + (size_t)tap * C * O;
+    for (int i = threadIdx.x; i < W::TapF / 4; i += 256) {
+      const int cb = i / (NT * 16), r = i % (NT * 16);
+      cp_async16(dst + 4 * i, src + ((size_t)cb * (O / 8) + n0) * 64 + 4 * r);
+    }
     cp_async_commit();
   };
-  fetch_tap(0);
+#pragma unroll 1
+  for (int tap = 0; tap < (W::All ? 9 : 1); ++tap) fetch_tap(tap);
   if constexpr (DGRAD)
     stage_plain<C, PITCH, MASK_IN>(smem, in, act, oy - 1, ox - 1, SHT, SW, Hr, Wr);
   else
@@ -326,14 +341,21 @@ __global__ void __launch_bounds__(256) conv_mma_kernel(const float* __restrict__
 #pragma unroll 1
   for (int tap = 0; tap < 9; ++tap) {
     const int dy = tap / 3, dx = tap % 3;
-    if (tap + 1 < 9) {
-      fetch_tap(tap + 1);
-      cp_async_wait<1>();
+    if constexpr (W::All) {
+      if (tap == 0) {
+        cp_async_wait<0>();
+        __syncthreads();                             // the weights and the input
+      }
     } else {
-      cp_async_wait<0>();
+      if (tap + 1 < 9) {
+        fetch_tap(tap + 1);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncthreads();                               // this tap's weights (and, first, the input)
     }
-    __syncthreads();                                 // this tap's weights (and, first, the input)
-    const float2* wt = reinterpret_cast<const float2*>(wbuf + (tap & 1) * TAPF);
+    const float2* wt = reinterpret_cast<const float2*>(wbuf + (W::All ? tap : tap & 1) * W::TapF);
 #pragma unroll
     for (int cb = 0; cb < C / 8; ++cb) {
       Split2 b[NTW];
@@ -350,7 +372,7 @@ __global__ void __launch_bounds__(256) conv_mma_kernel(const float* __restrict__
         for (int j = 0; j < NTW; ++j) mma8x3(acc[i][j], a, b[j]);
       }
     }
-    __syncthreads();                                 // the buffer is refilled two taps later
+    if constexpr (!W::All) __syncthreads();          // the buffer is refilled two taps later
   }
 #pragma unroll
   for (int i = 0; i < MTW; ++i) {
@@ -358,7 +380,7 @@ __global__ void __launch_bounds__(256) conv_mma_kernel(const float* __restrict__
     if (Y >= Hr) continue;
 #pragma unroll
     for (int j = 0; j < NTW; ++j) {
-      const int o = (wn * NTW + j) * 8 + 2 * t;
+      const int o = (n0 + wn * NTW + j) * 8 + 2 * t;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int X = ox + g + 8 * h;
@@ -1376,17 +1398,26 @@ int resident_per_sm(K kernel, int threads, size_t dyn_smem, int cap) {
   return std::max(1, std::min({cap, by_regs, by_smem}));
 }
 
-template <int C, int O, int MT, int WM, bool DGRAD, bool MASK_IN, bool MASK_OUT>
-cudaError_t launch_conv(const float* in, const float* act, const float* wpk, const float* bias, const float* aout,
-                        float* out, int Hr, int Wr, cudaStream_t s) {
-  const size_t smem = ((size_t)(MT + 2) * 18 * (C + 4) + 2 * (size_t)C * O) * sizeof(float);
-  auto k = conv_mma_kernel<C, O, MT, WM, DGRAD, MASK_IN, MASK_OUT>;
+template <int C, int O, int OB, int MT, int WM, bool DGRAD, bool MASK_IN, bool MASK_OUT>
+cudaError_t launch_conv_split(const float* in, const float* act, const float* wpk, const float* bias, const float* aout,
+                              float* out, int Hr, int Wr, cudaStream_t s) {
+  const size_t smem = ((size_t)(MT + 2) * 18 * (C + 4) + (size_t)ConvShape<C, OB>::Buffers * C * OB) * sizeof(float);
+  auto k = conv_mma_kernel<C, O, OB, MT, WM, DGRAD, MASK_IN, MASK_OUT>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  const dim3 grid((Wr + 15) / 16, (Hr + MT - 1) / MT);
+  const dim3 grid((Wr + 15) / 16, (Hr + MT - 1) / MT, O / OB);
   note_launches(1);
   k<<<grid, 256, smem, s>>>(in, act, wpk, bias, aout, out, Hr, Wr);
   return cudaGetLastError();
+}
+// The channels split into blocks of OB where even the split blocks do not fill the SMs twice over.
+template <int C, int O, int OB, int MT, int WM, bool DGRAD, bool MASK_IN, bool MASK_OUT>
+cudaError_t launch_conv(const float* in, const float* act, const float* wpk, const float* bias, const float* aout,
+                        float* out, int Hr, int Wr, int sms, cudaStream_t s) {
+  const int tiles = ((Wr + 15) / 16) * ((Hr + MT - 1) / MT);
+  return OB < O && tiles * (O / OB) <= 2 * sms
+             ? launch_conv_split<C, O, OB, MT, WM, DGRAD, MASK_IN, MASK_OUT>(in, act, wpk, bias, aout, out, Hr, Wr, s)
+             : launch_conv_split<C, O, O, MT, WM, DGRAD, MASK_IN, MASK_OUT>(in, act, wpk, bias, aout, out, Hr, Wr, s);
 }
 
 template <int C, int O, int TY, int MB, int WM, bool MASK_IN, int PF>
@@ -1523,10 +1554,10 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
   conv0_kernel<<<(ph * pw + kConv0FwdPx - 1) / kConv0FwdPx, 256, 0, s>>>(F(L.P), F(L.E), params, ph, pw, A[0]);
   ok(cudaGetLastError());
   const float* bias[5] = {nullptr, params + b_off(1), params + b_off(2), params + b_off(3), params + b_off(4)};
-  ok(launch_conv<64, 128, 4, 2, false, false, false>(A[0], nullptr, wf[1], bias[1], nullptr, A[1], ph << 1, pw << 1, s));
-  ok(launch_conv<32, 64, 8, 4, false, false, false>(A[1], nullptr, wf[2], bias[2], nullptr, A[2], ph << 2, pw << 2, s));
-  ok(launch_conv<16, 32, 16, 8, false, false, false>(A[2], nullptr, wf[3], bias[3], nullptr, A[3], ph << 3, pw << 3, s));
-  ok(launch_conv<8, 16, 16, 8, false, false, false>(A[3], nullptr, wf[4], bias[4], nullptr, A[4], ph << 4, pw << 4, s));
+  ok(launch_conv<64, 128, 32, 4, 2, false, false, false>(A[0], nullptr, wf[1], bias[1], nullptr, A[1], ph << 1, pw << 1, sms, s));
+  ok(launch_conv<32, 64, 32, 8, 4, false, false, false>(A[1], nullptr, wf[2], bias[2], nullptr, A[2], ph << 2, pw << 2, sms, s));
+  ok(launch_conv<16, 32, 16, 16, 8, false, false, false>(A[2], nullptr, wf[3], bias[3], nullptr, A[3], ph << 3, pw << 3, sms, s));
+  ok(launch_conv<8, 16, 16, 16, 8, false, false, false>(A[3], nullptr, wf[4], bias[4], nullptr, A[4], ph << 4, pw << 4, sms, s));
   // the head: up-sampling, conv5, conv6 with the L1 term (and, for the backward, gM')
   float* U = F(L.U);
   float* Hh = F(L.Hh);
@@ -1614,16 +1645,16 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
   // gradient); each weight gradient on a side stream once its output gradient exists
   ok(link(E, s, sd[1]));
   ok(launch_wgrad<8, 16, 16, 5, 4, true, 3>(A[3], gA[4], A[4], gp + w_off(4), gp + b_off(4), ph << 4, pw << 4, sms, sd[1]));
-  ok(launch_conv<16, 8, 16, 8, true, true, true>(gA[4], A[4], wd[4], nullptr, A[3], gA[3], ph << 4, pw << 4, s));
+  ok(launch_conv<16, 8, 8, 16, 8, true, true, true>(gA[4], A[4], wd[4], nullptr, A[3], gA[3], ph << 4, pw << 4, sms, s));
   ok(link(E, s, sd[2]));
   ok(launch_wgrad<16, 32, 16, 9, 4, false, 1>(A[2], gA[3], nullptr, gp + w_off(3), gp + b_off(3), ph << 3, pw << 3, sms, sd[2]));
-  ok(launch_conv<32, 16, 16, 8, true, false, true>(gA[3], nullptr, wd[3], nullptr, A[2], gA[2], ph << 3, pw << 3, s));
+  ok(launch_conv<32, 16, 8, 16, 8, true, false, true>(gA[3], nullptr, wd[3], nullptr, A[2], gA[2], ph << 3, pw << 3, sms, s));
   ok(link(E, s, sd[3]));
   ok(launch_wgrad<32, 64, 8, 9, 4, false, 0>(A[1], gA[2], nullptr, gp + w_off(2), gp + b_off(2), ph << 2, pw << 2, sms, sd[3]));
-  ok(launch_conv<64, 32, 8, 8, true, false, true>(gA[2], nullptr, wd[2], nullptr, A[1], gA[1], ph << 2, pw << 2, s));
+  ok(launch_conv<64, 32, 16, 8, 8, true, false, true>(gA[2], nullptr, wd[2], nullptr, A[1], gA[1], ph << 2, pw << 2, sms, s));
   ok(link(E, s, sd[2]));
   ok(launch_wgrad<64, 128, 4, 6, 2, false, 0>(A[0], gA[1], nullptr, gp + w_off(1), gp + b_off(1), ph << 1, pw << 1, sms, sd[2]));
-  ok(launch_conv<128, 64, 4, 4, true, false, false>(gA[1], nullptr, wd[1], nullptr, nullptr, gA[0], ph << 1, pw << 1, s));
+  ok(launch_conv<128, 64, 16, 4, 4, true, false, false>(gA[1], nullptr, wd[1], nullptr, nullptr, gA[0], ph << 1, pw << 1, sms, s));
   // conv0's adjoint: the input gradient on s, the weight and embedding gradients on a side stream;
   // then the block-mean term of dL/dI_r
   ok(link(E, s, sd[1]));
