@@ -561,7 +561,7 @@ __device__ __forceinline__ int find_cell(const MCell* cells, int n_cells, long l
 // the blocks that look back one after another.
 constexpr int kMergeItems = 4, kMergeTile = 256 * kMergeItems;
 template <int F>
-__global__ void __launch_bounds__(256) merge_kernel(const MCell* __restrict__ cells, int n_cells, long long total,
+__global__ void __launch_bounds__(256, 8) merge_kernel(const MCell* __restrict__ cells, int n_cells, long long total,
                                                     unsigned* ticket, unsigned long long* status, MergeOut out,
                                                     unsigned* timeout) {
   __shared__ unsigned s_blk, s_base;

@@ -232,17 +232,26 @@ __device__ __forceinline__ unsigned lookback(unsigned long long* status, unsigne
 // words (W a multiple of 4, rows on 16-byte boundaries).
 template <int W, bool VEC, typename Src, typename Skip>
 __device__ __forceinline__ void copy_rows(float* __restrict__ dst, int rows, Src src, Skip skip) {
-  constexpr int U = VEC ? W / 4 : W;
+  constexpr int U = VEC ? W / 4 : W, B = VEC ? 4 : 8;      // words in flight a thread
   using T = typename std::conditional<VEC, float4, float>::type;
   T* d = reinterpret_cast<T*>(dst);
-#pragma unroll 4
-  for (int i = threadIdx.x; i < rows * U; i += blockDim.x) {
-    const int r = i / U, c = i % U;
-    if (skip(r)) continue;
-    const float* s = src(r);
-    T v{};
-    if (s) v = __ldg(reinterpret_cast<const T*>(s) + c);
-    d[i] = v;
+  const int n = rows * U;
+  for (int i0 = threadIdx.x; i0 < n; i0 += B * blockDim.x) {
+    T v[B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {                          // every load before the first store
+      const int i = i0 + b * (int)blockDim.x;
+      v[b] = T{};
+      if (i < n) {
+        const float* s = src(i / U);
+        if (s) v[b] = __ldg(reinterpret_cast<const T*>(s) + i % U);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const int i = i0 + b * (int)blockDim.x;
+      if (i < n && !skip(i / U)) d[i] = v[b];
+    }
   }
 }
 
