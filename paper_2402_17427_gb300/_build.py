@@ -2,7 +2,8 @@
 
 Each .cu file is compiled in parallel with ``-gencode arch=compute_103a,code=sm_103a`` and the
 objects are linked into ``paper_2402_17427_gb300/libvgrast.so`` (CUDA runtime linked
-statically, so the library needs only the driver at run time).
+statically, so the library needs only the driver at run time).  Beside them the autograd nodes of the
+torch front end (``csrc/front.cpp``, host code against the installed torch) become ``_vgfront.so``.
 """
 from __future__ import annotations
 
@@ -18,6 +19,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libvgrast.so")
+FRONT_SRC = os.path.join(CSRC, "front.cpp")
+FRONT = os.path.join(PKG, "_vgfront.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "-I" + INCLUDE, "-I" + CSRC]
@@ -35,12 +38,31 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(FRONT)):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    t = min(os.path.getmtime(LIB), os.path.getmtime(FRONT))
+    deps = sources() + [FRONT_SRC] + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_front() -> None:
+    """Compiles the autograd nodes with the host compiler against the installed torch."""
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc())))
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"], INCLUDE]
+    tmp = FRONT + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f"-I{d}" for d in inc], FRONT_SRC,
+           "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{cmd[0]} failed on {FRONT_SRC}:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, FRONT)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -59,8 +81,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(r.stdout, r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 4)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(9, os.cpu_count() or 4)) as ex:
+        front = ex.submit(build_front)
         objs = list(ex.map(compile_one, sources()))
+        front.result()
     tmp = LIB + f".tmp{os.getpid()}"
     r = subprocess.run([cc, *ARCH, "-shared", "-o", tmp, *objs], capture_output=True, text=True)
     if r.returncode != 0:

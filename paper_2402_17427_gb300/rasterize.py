@@ -46,7 +46,10 @@ class RasterSettings:
         return o
 
 
-def camera_c(cam: Camera) -> B.vg_camera:
+def camera_c(cam) -> B.vg_camera:
+    """The C structure of a scenes.Camera (one that is that structure already comes back as it is)."""
+    if isinstance(cam, B.vg_camera):
+        return cam
     c = B.vg_camera()
     c.width, c.height = int(cam.width), int(cam.height)
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
@@ -68,7 +71,23 @@ def gaussians_c(means, log_scales, quats, logits, sh, degree: int) -> B.vg_gauss
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """Handle of the current device's current stream (without building a torch.cuda.Stream object)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+_front_module = None
+
+
+def _front():
+    """The autograd nodes in C++ (csrc/front.cpp), bound to the C ABI that the binding loaded."""
+    global _front_module
+    if _front_module is None:
+        from . import _vgfront
+        lib = B.lib()
+        _vgfront.init(ctypes.cast(lib.vg_rasterize_backward, ctypes.c_void_p).value,
+                      ctypes.cast(lib.vg_loss_l1_dssim_grad, ctypes.c_void_p).value)
+        _front_module = _vgfront
+    return _front_module
 
 
 class Workspace:
@@ -169,6 +188,8 @@ class Rasterizer:
 
 
 class _RasterizeFn(torch.autograd.Function):
+    """rasterize() through a Rasterizer subclass: its own forward and backward are called."""
+
     @staticmethod
     def forward(ctx, means, log_scales, quats, logits, sh, degree, cam, rasterizer):
         rgb, T, last = rasterizer.forward(means, log_scales, quats, logits, sh, degree, cam)
@@ -188,8 +209,13 @@ class _RasterizeFn(torch.autograd.Function):
 def rasterize(means, log_scales, quats, logits, sh, degree: int, cam: Camera, rasterizer: Rasterizer | None = None):
     """Differentiable render: returns the image [3,H,W]; gradients flow to the raw parameters."""
     r = rasterizer or Rasterizer()
-    rgb, _T, _last = _RasterizeFn.apply(means, log_scales, quats, logits, sh, degree, cam, r)
-    return rgb
+    if type(r) is not Rasterizer or "forward" in r.__dict__ or "backward" in r.__dict__:
+        rgb, _T, _last = _RasterizeFn.apply(means, log_scales, quats, logits, sh, degree, cam, r)
+        return rgb
+    camc = camera_c(cam)
+    rgb, T, last = r.forward(means, log_scales, quats, logits, sh, degree, camc)
+    return _front().attach_render(means, log_scales, quats, logits, sh, rgb, T, last, r.ws.buf, r.ws.capacity,
+                                  int(degree), bytes(camc), bytes(r.settings.c()))
 
 
 class LossL1DSSIM:
@@ -200,14 +226,19 @@ class LossL1DSSIM:
         self.buf = None
         self.loss = None
         self.grad = None
-        self.calls = 0          # forward calls on this workspace (the SSIM maps they leave behind)
+        self.uses = None        # forward calls on this workspace (the SSIM maps they leave behind)
+
+    @property
+    def calls(self) -> int:
+        return self.uses.value if self.uses is not None else 0
 
     def _workspace(self, img):
         _, H, W = img.shape
         need = B.vg_loss_workspace_bytes(W, H)
         if self.buf is None or self.buf.numel() < need:
             self.buf = torch.empty(need, dtype=torch.uint8, device=img.device)
-        self.calls += 1
+            self.uses = _front().Uses()
+        self.uses.bump()
         return W, H
 
     def __call__(self, img: torch.Tensor, target: torch.Tensor, reuse: bool = False):
@@ -240,8 +271,8 @@ class LossL1DSSIM:
 
 
 class _LossFn(torch.autograd.Function):
-    """Forward computes the loss only; backward runs the gradient pass scaled on the device by the
-    incoming gradient (no separate elementwise product)."""
+    """l1_dssim_loss() through a LossL1DSSIM subclass.  Forward computes the loss only; backward runs the
+    gradient pass scaled on the device by the incoming gradient (no separate elementwise product)."""
 
     @staticmethod
     def forward(ctx, img, target, lossobj):
@@ -262,7 +293,13 @@ class _LossFn(torch.autograd.Function):
 
 def l1_dssim_loss(img, target, lam: float = 0.2, lossobj: LossL1DSSIM | None = None):
     """Differentiable Eq. 1 loss ((1 - lam) L1 + lam D-SSIM) computed by the CUDA kernels."""
-    return _LossFn.apply(img, target, lossobj or LossL1DSSIM(lam))
+    f = lossobj or LossL1DSSIM(lam)
+    if type(f) is not LossL1DSSIM or "value" in f.__dict__ or "grad_scaled" in f.__dict__:
+        return _LossFn.apply(img, target, f)
+    with torch.no_grad():
+        x, y = img.contiguous(), target.contiguous()
+    loss = f.value(x, y)
+    return _front().attach_loss(img, x, y, loss, f.buf, f.uses, int(x.shape[2]), int(x.shape[1]), f.lam)
 
 
 def to_device(g, device="cuda"):
