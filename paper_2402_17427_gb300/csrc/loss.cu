@@ -2,8 +2,9 @@
 //
 // SSIM uses an 11x11 Gaussian window (sigma 1.5, separable, normalised) with zero padding and
 // C1 = 0.01^2, C2 = 0.03^2; both terms are means over 3 H W.  With the local moments
-// mx = w*x, exx = w*x^2, exy = w*(x y) (and my, eyy),
-//   S = (2 mx my + C1)(2 (exy - mx my) + C2) / ((mx^2 + my^2 + C1)(exx - mx^2 + eyy - my^2 + C2))
+// mx = w*x, my = w*y, ess = w*(x^2 + y^2), exy = w*(x y),
+//   S = (2 mx my + C1)(2 (exy - mx my) + C2) / ((mx^2 + my^2 + C1)(ess - mx^2 - my^2 + C2))
+// (the two second moments only enter as their sum, so four windows do instead of five),
 // and dL/dx(q) = l1' + (w * a)(q) + 2 x(q) (w * b)(q) + y(q) (w * c)(q), where a, b, c are
 // dL/dS times dS/dmx, dS/dexx, dS/dexy at every pixel (the window is symmetric, so correlation
 // with it is its own adjoint).  Two kernels: moments -> (a, b, c) maps + partial sums, then the
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
                                                                     double* __restrict__ partials) {
   pdl_enter();
   __shared__ __align__(16) float4 s4[NRP][QP];   // (x row 2p, x row 2p + 1, y row 2p, y row 2p + 1)
-  __shared__ __align__(16) float hs[5][LTH * LT];
+  __shared__ __align__(16) float hs[4][LTH * LT];
   __shared__ double red[kLossThreads / 32];
   const int c = blockIdx.z;
   const int ox = blockIdx.x * LT, oy = blockIdx.y * LT;
@@ -184,14 +185,14 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
   __syncthreads();
   if (threadIdx.x < NH) {
     const int p = threadIdx.x >> 2, g = threadIdx.x & 3;
-    float2 a[5][GH];
-    window_pairs<5, GH>(win, [&](int i, float2 (&v)[5]) {
+    float2 a[4][GH];
+    window_pairs<4, GH>(win, [&](int i, float2 (&v)[4]) {
       const float4 s = s4[p][qcol(GH * g + i)];
       const float2 xv = make_float2(s.x, s.y), yv = make_float2(s.z, s.w);
-      v[0] = xv; v[1] = yv; v[2] = __fmul2_rn(xv, xv); v[3] = __fmul2_rn(yv, yv); v[4] = __fmul2_rn(xv, yv);
+      v[0] = xv; v[1] = yv; v[2] = __ffma2_rn(xv, xv, __fmul2_rn(yv, yv)); v[3] = __fmul2_rn(xv, yv);
     }, a);
 #pragma unroll
-    for (int f = 0; f < 5; ++f)
+    for (int f = 0; f < 4; ++f)
 #pragma unroll
       for (int j = 0; j < GH; ++j) {
         hs[f][hs_at(2 * p, GH * g + j)] = a[f][j].x;
@@ -200,10 +201,10 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
   }
   __syncthreads();
   const int q = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * GV;   // column q, output rows r0 .. r0 + 7
-  float m[5][GV];
-  window_column<5>(win, [&](int i, float (&v)[5]) {
+  float m[4][GV];
+  window_column<4>(win, [&](int i, float (&v)[4]) {
 #pragma unroll
-    for (int f = 0; f < 5; ++f) v[f] = hs[f][hs_at(r0 + i, q)];
+    for (int f = 0; f < 4; ++f) v[f] = hs[f][hs_at(r0 + i, q)];
   }, m);
   // the per-pixel SSIM and its three partial derivatives for two rows at once (packed FP32; the
   // reciprocals approximate, within 1 ulp)
@@ -227,17 +228,16 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
       l1sum += fabsf(cell[sr & 1] - cell[2 + (sr & 1)]);
     }
     const float2 mx = make_float2(m[0][j], m[0][j + 1]), my = make_float2(m[1][j], m[1][j + 1]);
-    const float2 exx = make_float2(m[2][j], m[2][j + 1]), eyy = make_float2(m[3][j], m[3][j + 1]);
-    const float2 exy = make_float2(m[4][j], m[4][j + 1]);
-    const float2 mxx = __fmul2_rn(mx, mx), myy = __fmul2_rn(my, my), mxy = __fmul2_rn(mx, my);
-    const float2 sxx = __fadd2_rn(exx, neg(mxx)), syy = __fadd2_rn(eyy, neg(myy)), sxy = __fadd2_rn(exy, neg(mxy));
+    const float2 ess = make_float2(m[2][j], m[2][j + 1]), exy = make_float2(m[3][j], m[3][j + 1]);
+    const float2 mss = __ffma2_rn(mx, mx, __fmul2_rn(my, my)), mxy = __fmul2_rn(mx, my);
+    const float2 sss = __fadd2_rn(ess, neg(mss)), sxy = __fadd2_rn(exy, neg(mxy));
     const float2 N1 = __ffma2_rn(two, mxy, c1), N2 = __ffma2_rn(two, sxy, c2);
-    const float2 D1 = __fadd2_rn(__fadd2_rn(mxx, myy), c1), D2 = __fadd2_rn(__fadd2_rn(sxx, syy), c2);
+    const float2 D1 = __fadd2_rn(mss, c1), D2 = __fadd2_rn(sss, c2);
     const float2 iD1 = make_float2(rcp_approx(D1.x), rcp_approx(D1.y));
     const float2 iD2 = make_float2(rcp_approx(D2.x), rcp_approx(D2.y));
     const float2 iD = __fmul2_rn(iD1, iD2);
     const float2 S = __fmul2_rn(__fmul2_rn(N1, N2), iD);
-    // dS/dmx = 2 my (N2 - N1) iD - 2 mx S (iD1 - iD2), dS/dexx = -S iD2, dS/dexy = 2 N1 iD
+    // dS/dmx = 2 my (N2 - N1) iD - 2 mx S (iD1 - iD2), dS/dess = -S iD2, dS/dexy = 2 N1 iD
     const float2 t1 = __fmul2_rn(__fmul2_rn(__fmul2_rn(two, my), __fadd2_rn(N2, neg(N1))), iD);
     const float2 t2 = __fmul2_rn(__fmul2_rn(__fmul2_rn(two, mx), S), __fadd2_rn(iD1, neg(iD2)));
     const float2 g0 = __fmul2_rn(dl, __fadd2_rn(t1, neg(t2)));
