@@ -1,6 +1,6 @@
 // Evaluation with colour correction (paper Sec. 5.1, "Metrics"): a per-image least-squares
 // affine colour map fitted in centred form (channel means, then centred second moments; FP32
-// per thread, FP64 across threads and blocks, Cholesky in FP64), the corrected image clipped to
+// per thread, double-floats across threads and blocks, Cholesky in FP64), the corrected image clipped to
 // [0, 1], then PSNR (peak 1) and the loss's SSIM on the corrected image.
 //
 // Five launches.  Each streaming pass leaves one row of partial sums a block; the blocks of the next
@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "doublefloat.cuh"
 #include "internal.h"
 #include "vg_common.cuh"
 
@@ -31,37 +32,40 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// The block's sums of K per-thread values (FP32 inside a warp's first step, FP64 beyond): one row
-// of `part`.
+// The block's sums of K per-thread values: one row of `part`.  In double-floats: an FP64 addition holds the
+// SM's pipe for 16 clocks a warp, and 15 moments of 8 warps in FP64 took 20 us of the 44 us pass.
 template <int K>
-__device__ __forceinline__ void write_row(const float (&m)[K], double* __restrict__ part) {
-  __shared__ double sm[kEvalThreads / 32][K];
+__device__ __forceinline__ void write_row(const float (&m)[K], float2* __restrict__ part) {
+  __shared__ float2 sm[kEvalThreads / 32][K];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const double t = warp_sum_d((double)m[k]);
-    if (lane == 0) sm[w][k] = t;
+    const dd t = warp_sum_dd(dd(m[k]));
+    if (lane == 0) sm[w][k] = make_float2(t.h, t.l);
   }
   __syncthreads();
   if (threadIdx.x < K) {
-    double t = 0.0;
+    dd t(0.f);
 #pragma unroll
-    for (int j = 0; j < kEvalThreads / 32; ++j) t += sm[j][threadIdx.x];
-    part[(size_t)blockIdx.x * K + threadIdx.x] = t;
+    for (int j = 0; j < kEvalThreads / 32; ++j) t = t + dd(sm[j][threadIdx.x].x, sm[j][threadIdx.x].y);
+    part[(size_t)blockIdx.x * K + threadIdx.x] = make_float2(t.h, t.l);
   }
 }
 
 // tot[k] = sum over the nb rows of `part`, by every block that needs it: a warp takes columns
 // w, w + 8, ...  Ends with a block barrier.
 template <int K>
-__device__ __forceinline__ void sum_rows(const double* __restrict__ part, int nb, double* tot /*shared [K]*/) {
+__device__ __forceinline__ void sum_rows(const float2* __restrict__ part, int nb, double* tot /*shared [K]*/) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int k = w; k < K; k += kEvalThreads / 32) {
-    double t = 0.0;
+    dd t(0.f);
 #pragma unroll 5
-    for (int b = lane; b < nb; b += 32) t += part[(size_t)b * K + k];
-    t = warp_sum_d(t);
-    if (lane == 0) tot[k] = t;
+    for (int b = lane; b < nb; b += 32) {
+      const float2 v = part[(size_t)b * K + k];
+      t = t + dd(v.x, v.y);
+    }
+    t = warp_sum_dd(t);
+    if (lane == 0) tot[k] = (double)t.h + (double)t.l;
   }
   __syncthreads();
 }
@@ -98,7 +102,7 @@ __device__ __forceinline__ void each_quad(const float* __restrict__ img, const f
 // pass 1: channel sums of the rendering and the target
 template <bool WIDE>
 __global__ void __launch_bounds__(kEvalThreads) cc_sums(const float* __restrict__ img, const float* __restrict__ tgt,
-                                                        long long npx, double* __restrict__ part) {
+                                                        long long npx, float2* __restrict__ part) {
   pdl_enter();
   float m[kMeans] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   each_quad<WIDE>(img, tgt, npx, [&](const float (&x)[3][4], const float (&y)[3][4], long long, int) {
@@ -115,8 +119,8 @@ __global__ void __launch_bounds__(kEvalThreads) cc_sums(const float* __restrict_
 // the means for the fit.
 template <bool WIDE>
 __global__ void __launch_bounds__(kEvalThreads) cc_moments(const float* __restrict__ img, const float* __restrict__ tgt,
-                                                           long long npx, const double* __restrict__ sums, int nb,
-                                                           double* __restrict__ mean, double* __restrict__ part) {
+                                                           long long npx, const float2* __restrict__ sums, int nb,
+                                                           double* __restrict__ mean, float2* __restrict__ part) {
   pdl_enter();
   __shared__ double tot[kMeans];
   sum_rows<kMeans>(sums, nb, tot);
@@ -204,9 +208,9 @@ __device__ void cc_solve(const double* tot, const double* mean, double* coef) {
 // corrected image and its squared error.
 template <bool WIDE>
 __global__ void __launch_bounds__(kEvalThreads) cc_apply(const float* __restrict__ img, const float* __restrict__ tgt,
-                                                         long long npx, const double* __restrict__ mom, int nb,
+                                                         long long npx, const float2* __restrict__ mom, int nb,
                                                          const double* __restrict__ mean, float* __restrict__ corr,
-                                                         double* __restrict__ part, float* __restrict__ out) {
+                                                         float2* __restrict__ part, float* __restrict__ out) {
   pdl_enter();
   __shared__ double tot[kMoments], coef[12];
   sum_rows<kMoments>(mom, nb, tot);
@@ -244,12 +248,12 @@ __global__ void __launch_bounds__(kEvalThreads) cc_apply(const float* __restrict
 }
 
 // PSNR from the squared-error rows, SSIM from the moment pass's partial sums (sum S, sum |x - y|).
-__global__ void __launch_bounds__(1024) cc_finish(const double* __restrict__ sq, int nb, const double* __restrict__ ssim,
+__global__ void __launch_bounds__(1024) cc_finish(const float2* __restrict__ sq, int nb, const double* __restrict__ ssim,
                                                   int ns, long long n, float* __restrict__ out) {
   pdl_enter();
   __shared__ double sm[2][32];
   double e = 0.0, t = 0.0;
-  for (int b = threadIdx.x; b < nb; b += 1024) e += sq[b];
+  for (int b = threadIdx.x; b < nb; b += 1024) e += (double)sq[b].x + (double)sq[b].y;
 #pragma unroll 4
   for (int b = threadIdx.x; b < ns; b += 1024) t += ssim[2 * (size_t)b];
   e = warp_sum_d(e);
@@ -278,10 +282,10 @@ EvalLayout eval_layout(int W, int H) {
   auto take = [&](size_t b) { size_t at = o; o = align_up(o + b); return at; };
   const size_t px = (size_t)W * H;
   L.corr = take(3 * px * sizeof(float));
-  L.sums = take((size_t)kEvalBlocks * kMeans * sizeof(double));
+  L.sums = take((size_t)kEvalBlocks * kMeans * sizeof(float2));
   L.mean = take(kMeans * sizeof(double));
-  L.mom = take((size_t)kEvalBlocks * kMoments * sizeof(double));
-  L.sq = take((size_t)kEvalBlocks * sizeof(double));
+  L.mom = take((size_t)kEvalBlocks * kMoments * sizeof(float2));
+  L.sq = take((size_t)kEvalBlocks * sizeof(float2));
   L.ssim = take((size_t)ssim_partials(W, H) * 2 * sizeof(double));
   L.total = o;
   return L;
@@ -293,14 +297,15 @@ cudaError_t launch_eval(const float* img, const float* target, int W, int H, con
   const long long npx = (long long)W * H;
   const int nb = (int)std::min<long long>(kEvalBlocks, (npx + 4 * kEvalThreads - 1) / (4 * kEvalThreads));
   auto D = [&](size_t off) { return reinterpret_cast<double*>(ws + off); };
+  auto P = [&](size_t off) { return reinterpret_cast<float2*>(ws + off); };
   float* corr = reinterpret_cast<float*>(ws + L.corr);
   note_launches(4);
-  cc_sums<WIDE><<<nb, kEvalThreads, 0, s>>>(img, target, npx, D(L.sums));
-  launch_pdl(cc_moments<WIDE>, nb, kEvalThreads, 0, s, img, target, npx, D(L.sums), nb, D(L.mean), D(L.mom));
-  launch_pdl(cc_apply<WIDE>, nb, kEvalThreads, 0, s, img, target, npx, D(L.mom), nb, D(L.mean), corr, D(L.sq), out);
+  cc_sums<WIDE><<<nb, kEvalThreads, 0, s>>>(img, target, npx, P(L.sums));
+  launch_pdl(cc_moments<WIDE>, nb, kEvalThreads, 0, s, img, target, npx, P(L.sums), nb, D(L.mean), P(L.mom));
+  launch_pdl(cc_apply<WIDE>, nb, kEvalThreads, 0, s, img, target, npx, P(L.mom), nb, D(L.mean), corr, P(L.sq), out);
   const cudaError_t e = launch_ssim_value(corr, target, W, H, D(L.ssim), s);
   if (e != cudaSuccess) return e;
-  launch_pdl(cc_finish, 1, 1024, 0, s, D(L.sq), nb, D(L.ssim), ssim_partials(W, H), 3 * npx, out);
+  launch_pdl(cc_finish, 1, 1024, 0, s, P(L.sq), nb, D(L.ssim), ssim_partials(W, H), 3 * npx, out);
   return cudaGetLastError();
 }
 
