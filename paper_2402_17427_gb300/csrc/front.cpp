@@ -76,6 +76,13 @@ struct RenderNode : Function<RenderNode> {
     const variable_list s = ctx->get_saved_variables();
     const auto call = c10::static_intrusive_pointer_cast<RenderCall>(ctx->saved_data["call"].toCapsule());
     const at::Tensor dL = grad_outputs[0].contiguous();
+    // what saved-tensor hooks hand back may be anything
+    for (int k = 0; k < 5; ++k)
+      TORCH_CHECK_VALUE(s[k].is_cuda() && s[k].scalar_type() == at::kFloat && s[k].is_contiguous(),
+                        "Gaussian parameters must be contiguous float32 CUDA tensors");
+    for (int k = 5; k < 7; ++k)
+      TORCH_CHECK_VALUE(s[k].is_cuda() && s[k].is_contiguous() && s[k].element_size() == 4,
+                        "the saved transmittance and last indices must be contiguous CUDA tensors of 4-byte entries");
     variable_list g(6);                                    // the call itself has no gradient
     for (int k = 0; k < 5; ++k) g[k] = at::empty_like(s[k]);
     auto ptr = [](const at::Tensor& t) { return static_cast<float*>(t.data_ptr()); };
@@ -126,7 +133,9 @@ struct LossCall : torch::CustomClassHolder {
 };
 
 struct LossNode : Function<LossNode> {
-  static at::Tensor forward(AutogradContext* ctx, const at::Tensor& /*img: the graph's input*/,
+  // img and target are the graph's inputs; the call holds what the pass read (contiguous copies where
+  // they were not).  The target gets no gradient, as with a node that returns None for it.
+  static at::Tensor forward(AutogradContext* ctx, const at::Tensor& /*img*/, const at::Tensor& /*target*/,
                             c10::intrusive_ptr<LossCall> call) {
     ctx->save_for_backward({call->img, call->target});
     at::Tensor loss = std::move(call->loss);
@@ -141,6 +150,9 @@ struct LossNode : Function<LossNode> {
     const auto call = c10::static_intrusive_pointer_cast<LossCall>(ctx->saved_data["call"].toCapsule());
     if (*call->uses != call->use)
       throw std::runtime_error("the loss workspace was used by another forward before this backward");
+    for (const at::Tensor& t : s)
+      TORCH_CHECK_VALUE(t.is_cuda() && t.scalar_type() == at::kFloat && t.is_contiguous(),
+                        "the saved images must be contiguous float32 CUDA tensors");
     const at::Tensor scale = grad_outputs[0].detach().to(at::kFloat).contiguous();
     at::Tensor grad = at::empty_like(s[0]);
     const vg_status status = g_loss_grad(
@@ -148,11 +160,11 @@ struct LossNode : Function<LossNode> {
         call->height, call->lambda, call->workspace.data_ptr(), static_cast<size_t>(call->workspace.numel()),
         static_cast<const float*>(scale.data_ptr()), static_cast<float*>(grad.data_ptr()), current_stream(s[0]));
     if (status != VG_OK) raise_status(status, "vg_loss_l1_dssim_grad");
-    return {grad, at::Tensor()};
+    return {grad, at::Tensor(), at::Tensor()};
   }
 };
 
-at::Tensor attach_loss(const at::Tensor& img, const at::Tensor& img_c, const at::Tensor& target_c,
+at::Tensor attach_loss(const at::Tensor& img, const at::Tensor& target, const at::Tensor& img_c, const at::Tensor& target_c,
                        const at::Tensor& loss, const at::Tensor& workspace, const Uses& uses, int32_t width,
                        int32_t height, double lambda) {
   auto call = c10::make_intrusive<LossCall>();
@@ -165,7 +177,7 @@ at::Tensor attach_loss(const at::Tensor& img, const at::Tensor& img_c, const at:
   call->workspace = workspace;
   call->uses = uses.n;
   call->use = *uses.n;
-  return LossNode::apply(img, std::move(call));
+  return LossNode::apply(img, target, std::move(call));
 }
 
 }  // namespace
@@ -177,6 +189,12 @@ PYBIND11_MODULE(_vgfront, m) {
   });
   pybind11::class_<Uses>(m, "Uses")
       .def(pybind11::init<>())
+      .def(pybind11::pickle([](const Uses& u) { return *u.n; },        // a copy of a loss object counts by itself
+                            [](int64_t n) {
+                              Uses u;
+                              *u.n = n;
+                              return u;
+                            }))
       .def("bump", [](Uses& u) { ++*u.n; })
       .def_property_readonly("value", [](const Uses& u) { return *u.n; });
   m.def("attach_render", &attach_render);

@@ -299,7 +299,7 @@ def l1_dssim_loss(img, target, lam: float = 0.2, lossobj: LossL1DSSIM | None = N
     with torch.no_grad():
         x, y = img.contiguous(), target.contiguous()
     loss = f.value(x, y)
-    return _front().attach_loss(img, x, y, loss, f.buf, f.uses, int(x.shape[2]), int(x.shape[1]), f.lam)
+    return _front().attach_loss(img, target, x, y, loss, f.buf, f.uses, int(x.shape[2]), int(x.shape[1]), f.lam)
 
 
 def to_device(g, device="cuda"):

@@ -119,3 +119,41 @@ def test_backward_error_is_the_bindings():
     with pytest.raises(B.VGError) as e:
         img.sum().backward()
     assert e.value.status == B.VG_ERR_CAPACITY
+
+
+@pytest.mark.parametrize("unpack", [lambda t: t, lambda t: t.cuda().half(), lambda t: torch.stack([t.cuda()] * 2, -1)[..., 0]],
+                         ids=["cpu", "half", "strided"])
+def test_what_hooks_hand_back_is_checked(unpack):
+    """Saved tensors that come back off the device, in another type or strided are refused on the host."""
+    p, deg, cam, target = _scene()
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: t.cpu(), unpack):
+        img = R.rasterize(*p, deg, cam)
+    with pytest.raises(ValueError):
+        torch.autograd.grad(img.sum(), p)
+    x = torch.rand(3, 20, 24, device="cuda", requires_grad=True)
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: t.cpu(), lambda t: t):
+        loss = R.l1_dssim_loss(x, torch.rand(3, 20, 24, device="cuda"))
+    with pytest.raises(ValueError):
+        loss.backward()
+
+
+def test_target_that_requires_a_gradient_gets_none():
+    x, y = (torch.rand(3, 20, 24, device="cuda") for _ in range(2))
+    y.requires_grad_(True)
+    loss = R.l1_dssim_loss(x, y)
+    assert loss.requires_grad
+    loss.backward()
+    assert y.grad is None
+
+
+def test_loss_objects_copy():
+    import copy
+    f = R.LossL1DSSIM(0.2)
+    x, y = torch.rand(3, 20, 24, device="cuda", requires_grad=True), torch.rand(3, 20, 24, device="cuda")
+    loss = R.l1_dssim_loss(x, y, 0.2, f)
+    other = copy.deepcopy(f)
+    assert other.calls == 1
+    R.l1_dssim_loss(x, y, 0.2, other)          # another workspace and count: the first one's state stands
+    assert (f.calls, other.calls) == (1, 2)
+    loss.backward()
+    assert torch.isfinite(x.grad).all()
