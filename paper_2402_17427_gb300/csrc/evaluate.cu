@@ -34,20 +34,23 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 
 // The block's sums of K per-thread values: one row of `part`.  In double-floats: an FP64 addition holds the
 // SM's pipe for 16 clocks a warp, and 15 moments of 8 warps in FP64 took 20 us of the 44 us pass.
+// Scaled by 2^-17, since fewer than 2^17 threads add up: no sum of finite values leaves FP32's range.
+constexpr float kSumScale = 1.f / 131072.f;
+static_assert(kEvalBlocks * kEvalThreads <= 131072, "the scale covers every thread");
 template <int K>
 __device__ __forceinline__ void write_row(const float (&m)[K], float2* __restrict__ part) {
   __shared__ float2 sm[kEvalThreads / 32][K];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const dd t = warp_sum_dd(dd(m[k]));
+    const dd t = warp_sum_dd(dd(m[k] * kSumScale));
     if (lane == 0) sm[w][k] = make_float2(t.h, t.l);
   }
   __syncthreads();
   if (threadIdx.x < K) {
     dd t(0.f);
 #pragma unroll
-    for (int j = 0; j < kEvalThreads / 32; ++j) t = t + dd(sm[j][threadIdx.x].x, sm[j][threadIdx.x].y);
+    for (int j = 0; j < kEvalThreads / 32; ++j) t = dd_accumulate(t, dd(sm[j][threadIdx.x].x, sm[j][threadIdx.x].y));
     part[(size_t)blockIdx.x * K + threadIdx.x] = make_float2(t.h, t.l);
   }
 }
@@ -62,10 +65,10 @@ __device__ __forceinline__ void sum_rows(const float2* __restrict__ part, int nb
 #pragma unroll 5
     for (int b = lane; b < nb; b += 32) {
       const float2 v = part[(size_t)b * K + k];
-      t = t + dd(v.x, v.y);
+      t = dd_accumulate(t, dd(v.x, v.y));
     }
     t = warp_sum_dd(t);
-    if (lane == 0) tot[k] = (double)t.h + (double)t.l;
+    if (lane == 0) tot[k] = ((double)t.h + (double)t.l) / (double)kSumScale;
   }
   __syncthreads();
 }
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(1024) cc_finish(const float2* __restrict__ sq,
   e = warp_sum_d(sm[0][threadIdx.x]);
   t = warp_sum_d(sm[1][threadIdx.x]);
   if (threadIdx.x != 0) return;
-  const double mse = e / (double)n;
+  const double mse = e / (double)kSumScale / (double)n;
   out[0] = mse > 0.0 ? (float)(-10.0 * log10(mse)) : INFINITY;
   out[1] = (float)(t / (double)n);
 }

@@ -38,3 +38,25 @@ def test_metrics_at_any_size_and_alignment(H, W, offset):
     assert abs(out[1] - oracle.ssim(c, y)) <= 2e-5
     assert np.allclose(out[2:11].reshape(3, 3), A, rtol=1e-4, atol=1e-5)
     assert np.allclose(out[11:14], b, rtol=1e-4, atol=1e-5)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3e18])
+def test_infinite_and_huge_targets(value):
+    """One target pixel that is infinite, NaN or so large that the sums pass FP32's range: what plain FP64 sums of the
+    same fit give (a NaN fit is clipped to 0, and the squared error follows)."""
+    x = torch.rand(3, 65, 260, device="cuda")
+    y = torch.rand(3, 65, 260, device="cuda")
+    y[1] = y[1] if not np.isfinite(value) else value * (0.5 + 0.5 * y[1])
+    if not np.isfinite(value):
+        y[1, 7, 9] = value
+    out = R.color_corrected_metrics(x, y).cpu().numpy().astype(np.float64)
+    if np.isnan(value):
+        assert out[0] == np.inf and np.isnan(out[12])     # a squared error that is no positive number
+    elif np.isinf(value):
+        assert np.isnan(out[12]) and out[0] == -np.inf
+    else:
+        d = y[1].double() - 1.0           # the fit is far above 1 everywhere, so it is clipped to 1
+        rest = sum(float((y[c].double() - y[c].double().mean()).square().sum()) for c in (0, 2))
+        mse = (float(d.square().sum()) + rest) / y.numel()
+        assert abs(out[0] + 10.0 * np.log10(mse)) <= 1e-3
+        assert np.isfinite(out).all()
