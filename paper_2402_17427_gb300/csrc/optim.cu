@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(256) accumulate_kernel(const float* __restrict
                                                          const uint32_t* d0, const uint32_t* d1,
                                                          const uint32_t* __restrict__ vis_ids, float hw, float hh,
                                                          float* __restrict__ accum, int* __restrict__ count) {
+  if (render_dead(hdr)) return;     // the depth order may hold unwritten slots
   const uint32_t* __restrict__ dorder = depth_order(hdr, d0, d1);
   const unsigned V = hdr->visible;
   for (unsigned s = blockIdx.x * blockDim.x + threadIdx.x; s < V; s += gridDim.x * blockDim.x) {
