@@ -176,10 +176,16 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
   const int c = blockIdx.z;
   const int ox = blockIdx.x * LT, oy = blockIdx.y * LT;
   const size_t plane = (size_t)W * H;
+  // Every value of the tile, its zero padding too, is taken relative to the rendering at the tile's middle:
+  // variances and covariance do not change, and their cancellation (mean of squares less square of
+  // mean) is of small numbers where the image is smooth.  The sum of both second moments alone made the
+  // gradient's error 1.12 times that of two (photograph-like images: 3.4e-6 against 3.0e-6).
+  float base = __ldg(x + c * plane + (size_t)min(oy + LT / 2, H - 1) * W + min(ox + LT / 2, W - 1));
+  base = fabsf(base) <= 1024.f ? base : 0.f;     // 0 for a NaN
   {
     const float* const src[2] = {x + c * plane, y + c * plane};
     stage_pairs<2>(src, W, H, ox, oy, [&](int p, int q, const float2 (&v)[2]) {
-      s4[p][q] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+      s4[p][q] = make_float4(v[0].x - base, v[0].y - base, v[1].x - base, v[1].y - base);
     });
   }
   __syncthreads();
@@ -227,10 +233,12 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
       const float* cell = sf + ((sr >> 1) * QP + qcol(q + HALO)) * 4;
       l1sum += fabsf(cell[sr & 1] - cell[2 + (sr & 1)]);
     }
-    const float2 mx = make_float2(m[0][j], m[0][j + 1]), my = make_float2(m[1][j], m[1][j + 1]);
+    const float2 dx = make_float2(m[0][j], m[0][j + 1]), dy = make_float2(m[1][j], m[1][j + 1]);
     const float2 ess = make_float2(m[2][j], m[2][j + 1]), exy = make_float2(m[3][j], m[3][j + 1]);
+    const float2 sss = __fadd2_rn(ess, neg(__ffma2_rn(dx, dx, __fmul2_rn(dy, dy))));
+    const float2 sxy = __fadd2_rn(exy, neg(__fmul2_rn(dx, dy)));
+    const float2 b2 = make_float2(base, base), mx = __fadd2_rn(dx, b2), my = __fadd2_rn(dy, b2);
     const float2 mss = __ffma2_rn(mx, mx, __fmul2_rn(my, my)), mxy = __fmul2_rn(mx, my);
-    const float2 sss = __fadd2_rn(ess, neg(mss)), sxy = __fadd2_rn(exy, neg(mxy));
     const float2 N1 = __ffma2_rn(two, mxy, c1), N2 = __ffma2_rn(two, sxy, c2);
     const float2 D1 = __fadd2_rn(mss, c1), D2 = __fadd2_rn(sss, c2);
     const float2 iD1 = make_float2(rcp_approx(D1.x), rcp_approx(D1.y));
