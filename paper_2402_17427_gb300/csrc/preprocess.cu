@@ -161,13 +161,13 @@ struct Proj {
   bool valid;
 };
 
-// Projection of Gaussian i.  The key-defining values (depth, u, v) follow the exact FP32
-// operation order stated for the sort keys; the rest is ordinary FP32.
-__device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const KOpts& op, int i, Proj& P) {
+// Projection of Gaussian i, whose mean the caller has put into P.m; log_scale(k) gives its k-th log-scale.
+// The key-defining values (depth, u, v) follow the exact FP32 operation order stated for the sort keys;
+// the rest is ordinary FP32.
+template <typename LogScale>
+__device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const KOpts& op, int i, LogScale log_scale,
+                                        Proj& P) {
   P.valid = false;
-  P.m[0] = __ldg(g.means + 3 * i);
-  P.m[1] = __ldg(g.means + 3 * i + 1);
-  P.m[2] = __ldg(g.means + 3 * i + 2);
 #pragma unroll
   for (int r = 0; r < 3; ++r)
     P.p[r] = __fmaf_rn(cm.R[3 * r], P.m[0], __fmaf_rn(cm.R[3 * r + 1], P.m[1], __fmaf_rn(cm.R[3 * r + 2], P.m[2], cm.t[r])));
@@ -188,7 +188,7 @@ __device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const K
   P.Rq[3] = 2.f * (x * y + w * zq);        P.Rq[4] = 1.f - 2.f * (x * x + zq * zq); P.Rq[5] = 2.f * (y * zq - w * x);
   P.Rq[6] = 2.f * (x * zq - w * y);        P.Rq[7] = 2.f * (y * zq + w * x);        P.Rq[8] = 1.f - 2.f * (x * x + y * y);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) P.s[k] = expf(__ldg(g.log_scales + 3 * i + k));
+  for (int k = 0; k < 3; ++k) P.s[k] = expf(log_scale(k));
   float M[9];
 #pragma unroll
   for (int r = 0; r < 3; ++r)
@@ -240,32 +240,38 @@ __device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const K
   P.valid = true;
 }
 
-// Whether Gaussian i may touch the image, from its mean and its largest scale alone: false only if
+__device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const KOpts& op, int i, Proj& P) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) P.m[k] = __ldg(g.means + 3 * i + k);
+  project(g, cm, op, i, [&](int k) { return __ldg(g.log_scales + 3 * i + k); }, P);
+}
+
+// Whether a Gaussian may touch the image, from its mean and its log-scales alone: false only if
 // project() and the rectangle rule would cull it.  lambda_max(T Sigma T^T) <= |T|_F^2 max(s)^2 bounds the
-// radius; the margins (1e-3 relative, 0.01 px + 1e-6 |u|) are far above the rounding of either side.
-// Comparisons are written so that a NaN or an infinity passes on to project().
-__device__ __forceinline__ bool may_touch(const KGauss& g, const KCam& cm, const KOpts& op, int i, const float* m) {
+// radius; the margins (1e-3 relative, 0.01 px + 1e-6 (|u| + |cx|)) are far above the rounding of either side
+// and above the errors of the approximate reciprocal, root and exponential (a few 1e-7; the exponential's
+// grow with the exponent, to 1e-5 at scales of e^88).  Comparisons are written so that a NaN or an
+// infinity passes on to project().
+__device__ __forceinline__ bool may_touch(const KCam& cm, const KOpts& op, const float* m, const float* ls) {
   float p[3];
 #pragma unroll
   for (int r = 0; r < 3; ++r)
     p[r] = __fmaf_rn(cm.R[3 * r], m[0], __fmaf_rn(cm.R[3 * r + 1], m[1], __fmaf_rn(cm.R[3 * r + 2], m[2], cm.t[r])));
   const float z = p[2];
   if (!(z > cm.near_plane)) return false;
-  const float smax = expf(fmaxf(fmaxf(__ldg(g.log_scales + 3 * i), __ldg(g.log_scales + 3 * i + 1)),
-                                __ldg(g.log_scales + 3 * i + 2)));
-  const float xz = __fdiv_rn(p[0], z), yz = __fdiv_rn(p[1], z);
-  const float u = __fmaf_rn(cm.fx, xz, cm.cx), v = __fmaf_rn(cm.fy, yz, cm.cy);
+  const float smax = __expf(fmaxf(fmaxf(ls[0], ls[1]), ls[2]));
+  const float iz = rcp_approx(z), xz = p[0] * iz, yz = p[1] * iz;
+  const float u = fmaf(cm.fx, xz, cm.cx), v = fmaf(cm.fy, yz, cm.cy);
   const float xzc = fminf(cm.limx, fmaxf(-cm.limx, xz)), yzc = fminf(cm.limy, fmaxf(-cm.limy, yz));
-  const float iz = 1.f / z;
-  const float j00 = cm.fx * iz, j02 = -cm.fx * xzc * iz, j11 = cm.fy * iz, j12 = -cm.fy * yzc * iz;
+  const float j00 = cm.fx * iz, j02 = -j00 * xzc, j11 = cm.fy * iz, j12 = -j11 * yzc;
   float f2 = 0.f;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const float a = j00 * cm.R[c] + j02 * cm.R[6 + c], b = j11 * cm.R[3 + c] + j12 * cm.R[6 + c];
     f2 = fmaf(a, a, fmaf(b, b, f2));
   }
-  const float rb = 3.003f * sqrtf(fmaf(1.001f * f2, smax * smax, op.dilation)) + 0.01f;
-  const float ru = fmaf(1e-6f, fabsf(u), rb), rv = fmaf(1e-6f, fabsf(v), rb);
+  const float rb = 3.003f * sqrt_approx(fmaf(1.001f * f2, smax * smax, op.dilation)) + 0.01f;
+  const float ru = fmaf(1e-6f, fabsf(u) + fabsf(cm.cx), rb), rv = fmaf(1e-6f, fabsf(v) + fabsf(cm.cy), rb);
   return !(u + ru < 0.f || u - ru > (float)(cm.W - 1) || v + rv < 0.f || v - rv > (float)(cm.H - 1));
 }
 
@@ -273,103 +279,142 @@ __device__ __forceinline__ bool may_touch(const KGauss& g, const KCam& cm, const
 // entry (depth key, Gaussian, tile rectangle) in the run's own part of `entries`, and their number.
 //
 // Only ~1 in 5 Gaussians is visible (1 in 25 in the 20M-Gaussian city), in no order, so may_touch()
-// first thins them out on 24 bytes a Gaussian, four a thread with their loads in flight together; the
-// candidates are packed densely in shared memory, and whole warps of them go through project().  No
-// block waits for another: compact_kernel closes the gaps between the runs.  In one kernel with a
-// look-back over the runs (and the spherical harmonics, which now follow in record_kernel) a block
-// spent most of its ~19 us waiting: 963 us for the 20M Gaussians of the city and 58 us for 1M; with
-// the harmonics moved out 550 and 44 us.
-constexpr int kCullThreads = 128, kCullItems = 4, kCullWarps = kCullThreads / 32;
+// first thins them out on 24 bytes a Gaussian; the candidates are packed densely in shared memory, and
+// whole warps of them go through project().  No block waits for another: compact_kernel closes the gaps
+// between the runs.  In one kernel with a look-back over the runs (and the spherical harmonics, which now
+// follow in record_kernel) a block spent most of its ~19 us waiting: 963 us for the 20M Gaussians of the
+// city and 58 us for 1M; with the harmonics moved out 550 and 44 us, without the look-back 283 and 22.
+// What bounded it then was the latency of each block's loads (means, then scales, then the candidates'
+// rows): the blocks are persistent now, and copy the next run's means and log-scales into shared memory
+// (cp.async, 16 bytes where the run lies in one segment on a 16-byte boundary) while they work on this one.
+constexpr int kCullThreads = 128, kCullItems = 4, kCullWarps = kCullThreads / 32, kCullBlocks = 8;
 static_assert(kCullThreads * kCullItems == kCullRun, "a block takes one run");
-__global__ void __launch_bounds__(kCullThreads, 9) cull_kernel(const DevTables* __restrict__ tab, int total_n,
-                                                               uint4* __restrict__ entries,
-                                                               unsigned* __restrict__ counts,
-                                                               uint32_t* __restrict__ touched,
-                                                               float4* __restrict__ key_inputs) {
+__global__ void __launch_bounds__(kCullThreads, kCullBlocks) cull_kernel(const DevTables* __restrict__ tab,
+                                                                         int total_n, int runs,
+                                                                         uint4* __restrict__ entries,
+                                                                         unsigned* __restrict__ counts,
+                                                                         uint32_t* __restrict__ touched,
+                                                                         float4* __restrict__ key_inputs) {
   pdl_enter();
-  __shared__ unsigned s_wc[2][kCullItems * kCullWarps];  // counts a warp (and item) leaves for the others
+  __shared__ __align__(16) float s_in[2][2][3 * kCullRun];   // [buffer][means, log-scales]
+  __shared__ unsigned s_wc[2][kCullItems * kCullWarps];      // counts a warp (and item) leaves for the others
   __shared__ uint16_t s_cand[kCullRun];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int base = (int)blockIdx.x * kCullRun, last = min(total_n - 1, base + (kCullRun - 1));
-  const int seg0 = find_seg(tab, base);
-  const bool one = seg0 == tab->h.n_segs - 1 || tseg(tab, seg0 + 1).offset > last;   // one segment in this run
-  // 1. candidates: a mean each, all four requested together, then the largest scales
-  float m[kCullItems][3];
+  // segment of a run's first Gaussian; complemented if the run reaches into the next one
+  auto fetch = [&](int run, int buf) {
+    const int base = run * kCullRun, last = min(total_n - 1, base + (kCullRun - 1));
+    const int seg = find_seg(tab, base);
+    const bool one = seg == tab->h.n_segs - 1 || tseg(tab, seg + 1).offset > last;
+    const KSeg& sg = tseg(tab, seg);
+    const float* m = sg.g.means + 3 * (size_t)(base - sg.offset);
+    const float* ls = sg.g.log_scales + 3 * (size_t)(base - sg.offset);
+    if (one && last - base == kCullRun - 1 &&
+        ((reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(ls)) & 15u) == 0) {
 #pragma unroll
-  for (int j = 0; j < kCullItems; ++j) {
-    const int i = base + j * kCullThreads + tid;
-    if (i <= last) {
-      const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
-      const float* q = sg.g.means + 3 * (size_t)(i - sg.offset);
-      m[j][0] = __ldg(q); m[j][1] = __ldg(q + 1); m[j][2] = __ldg(q + 2);
-    }
-  }
-  unsigned votes[kCullItems];
-#pragma unroll
-  for (int j = 0; j < kCullItems; ++j) {
-    const int i = base + j * kCullThreads + tid;
-    bool c = false;
-    if (i <= last) {
-      const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
-      const KView& vw = tview(tab, sg.view);
-      c = key_inputs != nullptr || may_touch(sg.g, vw.cam, vw.op, i - sg.offset, m[j]);
-      if (!c) touched[i] = 0;
-    }
-    votes[j] = __ballot_sync(0xffffffffu, c);
-    if (lane == 0) s_wc[0][j * kCullWarps + warp] = __popc(votes[j]);
-  }
-  __syncthreads();
-  const uint32_t lt = lanemask_lt();
-  int ncand = 0;
-#pragma unroll
-  for (int k = 0; k < kCullItems * kCullWarps; ++k) {      // counts in index order: item, then warp
-    const int j = k / kCullWarps;
-    if (k % kCullWarps == warp && (votes[j] >> lane & 1u))
-      s_cand[ncand + __popc(votes[j] & lt)] = (uint16_t)(j * kCullThreads + tid);
-    ncand += (int)s_wc[0][k];
-  }
-  __syncthreads();
-  // 2. projection, tile rectangle and visibility of the candidates, the visible ones written in order
-  unsigned tot = 0;
-  for (int r = 0, odd = 1; r < ncand; r += kCullThreads, odd ^= 1) {
-    bool vis = false;
-    uint4 e = make_uint4(0u, 0u, 0u, 0u);
-    if (r + tid < ncand) {
-      const int i = base + s_cand[r + tid];
-      const KSeg& sg = tseg(tab, one ? seg0 : find_seg(tab, i));
-      const KView& vw = tview(tab, sg.view);
-      Proj P;
-      project(sg.g, vw.cam, vw.op, i - sg.offset, P);
-      uint32_t cnt = 0;
-      if (P.valid) {
-        const int T = vw.op.tile;
-        const int xlo = rect_lo(P.u, P.r, vw.cam.W), xhi = rect_hi(P.u, P.r, vw.cam.W);
-        const int ylo = rect_lo(P.v, P.r, vw.cam.H), yhi = rect_hi(P.v, P.r, vw.cam.H);
-        if (xlo <= xhi && ylo <= yhi) {
-          const int tx0 = xlo / T, tx1 = xhi / T, ty0 = ylo / T, ty1 = yhi / T;
-          cnt = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
-          vis = true;
-          e = make_uint4(__float_as_uint(P.depth), (uint32_t)i, (uint32_t)tx0 | ((uint32_t)tx1 << 16),
-                         (uint32_t)ty0 | ((uint32_t)ty1 << 16));
-        }
+      for (int k = 4 * tid; k < 3 * kCullRun; k += 4 * kCullThreads) {
+        cp_async16(&s_in[buf][0][k], m + k);
+        cp_async16(&s_in[buf][1][k], ls + k);
       }
-      touched[i] = cnt;
-      if (key_inputs)
-        key_inputs[i] = P.valid ? make_float4(P.u, P.v, P.r, P.depth) : make_float4(0.f, 0.f, -1.f, 0.f);
+    } else {
+      for (int k = tid; k < 3 * (last - base + 1); k += kCullThreads) {
+        const float *pm = m + k, *pl = ls + k;
+        if (!one) {
+          const int i = base + k / 3;
+          const KSeg& si = tseg(tab, find_seg(tab, i));
+          const size_t o = 3 * (size_t)(i - si.offset) + k % 3;
+          pm = si.g.means + o;
+          pl = si.g.log_scales + o;
+        }
+        cp_async4_zfill(&s_in[buf][0][k], pm, true);
+        cp_async4_zfill(&s_in[buf][1][k], pl, true);
+      }
     }
-    const unsigned vote = __ballot_sync(0xffffffffu, vis);
-    if (lane == 0) s_wc[odd][warp] = __popc(vote);
-    __syncthreads();                      // the other buffer is written in the next round
-    unsigned at = tot + __popc(vote & lt);
+    return one ? seg : ~seg;
+  };
+  int seg_next = 0;
+  if ((int)blockIdx.x < runs) seg_next = fetch(blockIdx.x, 0);
+  cp_async_commit();
+  int buf = 0;
+  for (int run = blockIdx.x; run < runs; run += gridDim.x, buf ^= 1) {
+    const int seg = seg_next;
+    if (run + (int)gridDim.x < runs) seg_next = fetch(run + gridDim.x, buf ^ 1);
+    cp_async_commit();
+    cp_async_wait<1>();
+    __syncthreads();
+    const float* const s_m = s_in[buf][0];
+    const float* const s_ls = s_in[buf][1];
+    const int base = run * kCullRun, last = min(total_n - 1, base + (kCullRun - 1));
+    auto seg_of = [&](int i) -> const KSeg& { return tseg(tab, seg >= 0 ? seg : find_seg(tab, i)); };
+    // 1. candidates
+    unsigned votes[kCullItems];
 #pragma unroll
-    for (int w = 0; w < kCullWarps; ++w) {
-      const unsigned c = s_wc[odd][w];
-      if (w < warp) at += c;
-      tot += c;
+    for (int j = 0; j < kCullItems; ++j) {
+      const int k = j * kCullThreads + tid, i = base + k;
+      bool c = false;
+      if (i <= last) {
+        const KView& vw = tview(tab, seg_of(i).view);
+        c = key_inputs != nullptr || may_touch(vw.cam, vw.op, s_m + 3 * k, s_ls + 3 * k);
+        if (!c) touched[i] = 0;
+      }
+      votes[j] = __ballot_sync(0xffffffffu, c);
+      if (lane == 0) s_wc[0][j * kCullWarps + warp] = __popc(votes[j]);
     }
-    if (vis) entries[(size_t)base + at] = e;
+    __syncthreads();
+    const uint32_t lt = lanemask_lt();
+    int ncand = 0;
+#pragma unroll
+    for (int k = 0; k < kCullItems * kCullWarps; ++k) {      // counts in index order: item, then warp
+      const int j = k / kCullWarps;
+      if (k % kCullWarps == warp && (votes[j] >> lane & 1u))
+        s_cand[ncand + __popc(votes[j] & lt)] = (uint16_t)(j * kCullThreads + tid);
+      ncand += (int)s_wc[0][k];
+    }
+    __syncthreads();
+    // 2. projection, tile rectangle and visibility of the candidates, the visible ones written in order
+    unsigned tot = 0;
+    for (int r = 0, odd = 1; r < ncand; r += kCullThreads, odd ^= 1) {
+      bool vis = false;
+      uint4 e = make_uint4(0u, 0u, 0u, 0u);
+      if (r + tid < ncand) {
+        const int k = s_cand[r + tid], i = base + k;
+        const KSeg& sg = seg_of(i);
+        const KView& vw = tview(tab, sg.view);
+        Proj P;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) P.m[a] = s_m[3 * k + a];
+        project(sg.g, vw.cam, vw.op, i - sg.offset, [&](int a) { return s_ls[3 * k + a]; }, P);
+        uint32_t cnt = 0;
+        if (P.valid) {
+          const int T = vw.op.tile;
+          const int xlo = rect_lo(P.u, P.r, vw.cam.W), xhi = rect_hi(P.u, P.r, vw.cam.W);
+          const int ylo = rect_lo(P.v, P.r, vw.cam.H), yhi = rect_hi(P.v, P.r, vw.cam.H);
+          if (xlo <= xhi && ylo <= yhi) {
+            const int tx0 = xlo / T, tx1 = xhi / T, ty0 = ylo / T, ty1 = yhi / T;
+            cnt = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
+            vis = true;
+            e = make_uint4(__float_as_uint(P.depth), (uint32_t)i, (uint32_t)tx0 | ((uint32_t)tx1 << 16),
+                           (uint32_t)ty0 | ((uint32_t)ty1 << 16));
+          }
+        }
+        touched[i] = cnt;
+        if (key_inputs)
+          key_inputs[i] = P.valid ? make_float4(P.u, P.v, P.r, P.depth) : make_float4(0.f, 0.f, -1.f, 0.f);
+      }
+      const unsigned vote = __ballot_sync(0xffffffffu, vis);
+      if (lane == 0) s_wc[odd][warp] = __popc(vote);
+      __syncthreads();                      // the other buffer is written in the next round
+      unsigned at = tot + __popc(vote & lt);
+#pragma unroll
+      for (int w = 0; w < kCullWarps; ++w) {
+        const unsigned c = s_wc[odd][w];
+        if (w < warp) at += c;
+        tot += c;
+      }
+      if (vis) entries[(size_t)base + at] = e;
+    }
+    if (tid == 0) counts[run] = tot;
+    __syncthreads();                        // the buffers are free for the next run
   }
-  if (tid == 0) counts[blockIdx.x] = tot;
 }
 
 // Projection, second part: the runs' entries moved together in index order (slot = position among all
@@ -858,7 +903,8 @@ cudaError_t launch_preprocess(const DevTables* tab, int total_n, uint2* rects, u
   if (total_n == 0) return cudaSuccess;
   note_launches(2);
   const int runs = (total_n - 1) / kCullRun + 1;
-  launch_pdl(cull_kernel, runs, kCullThreads, 0, s, tab, total_n, cp.entries, cp.counts, touched, cp.key_inputs);
+  launch_pdl(cull_kernel, std::min(runs, kCullBlocks * sort_blocks() / 2), kCullThreads, 0, s, tab, total_n, runs, cp.entries,
+             cp.counts, touched, cp.key_inputs);
   // a warp a run on small scenes, up to 4 blocks an SM (2 an SM left a block of a merged scene, whose
   // visible Gaussians sit in few runs, with a long tail: 41 us for four views; more add up more counts)
   const int blocks = std::max(1, std::min((runs + kCompactThreads / 32 - 1) / (kCompactThreads / 32), 2 * sort_blocks()));

@@ -64,6 +64,12 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // The adjoint compositing accumulates, per splat, six moments of g = alpha dL/dalpha over the
 // pixels it reaches (dx = px - u, dy = py - v; FP32 sums):
 //   m = (sum dx g, sum dy g, sum dx^2 g, sum dx dy g, sum dy^2 g, sum g).
