@@ -3,8 +3,6 @@
 
 #include <cuda_runtime.h>
 
-#include <cmath>
-
 namespace vg {
 
 // Double-float: a value as an unevaluated sum of two FP32 numbers (48 bits), by the classical
@@ -38,18 +36,11 @@ __device__ __forceinline__ dd operator/(dd a, dd b) {
 __device__ __forceinline__ bool operator<(dd a, dd b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
 __device__ __forceinline__ bool operator==(dd a, dd b) { return a.h == b.h && a.l == b.l; }
 
-// a + b for sums of any values: an infinity or a NaN comes out as FP32 addition leaves it (the error terms of
-// operator+ would make a NaN of every infinity).
-__device__ __forceinline__ dd dd_accumulate(dd a, dd b) {
-  const float s = __fadd_rn(a.h, b.h);
-  return fabsf(s) < INFINITY ? a + b : dd(s);
-}
-
 // Sum over a warp's lanes (every lane).
 __device__ __forceinline__ dd warp_sum_dd(dd v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
-    v = dd_accumulate(v, dd(__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)));
+    v = v + dd(__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o));
   return v;
 }
 

@@ -32,6 +32,17 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
+// A warp's sum of any values: where double-floats give no finite one (their error terms make a NaN of
+// every infinity), what FP32 additions leave.
+__device__ __forceinline__ dd warp_sum_any(dd v) {
+  const dd t = warp_sum_dd(v);
+  if (__all_sync(0xffffffffu, fabsf(t.h) < INFINITY)) return t;
+  float s = v.h;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return dd(s);
+}
+
 // The block's sums of K per-thread values: one row of `part`.  In double-floats: an FP64 addition holds the
 // SM's pipe for 16 clocks a warp, and 15 moments of 8 warps in FP64 took 20 us of the 44 us pass.
 // Scaled by 2^-17, since fewer than 2^17 threads add up: no sum of finite values leaves FP32's range.
@@ -43,14 +54,18 @@ __device__ __forceinline__ void write_row(const float (&m)[K], float2* __restric
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const dd t = warp_sum_dd(dd(m[k] * kSumScale));
+    const dd t = warp_sum_any(dd(m[k] * kSumScale));
     if (lane == 0) sm[w][k] = make_float2(t.h, t.l);
   }
   __syncthreads();
   if (threadIdx.x < K) {
     dd t(0.f);
 #pragma unroll
-    for (int j = 0; j < kEvalThreads / 32; ++j) t = dd_accumulate(t, dd(sm[j][threadIdx.x].x, sm[j][threadIdx.x].y));
+    for (int j = 0; j < kEvalThreads / 32; ++j) t = t + dd(sm[j][threadIdx.x].x, sm[j][threadIdx.x].y);
+    if (!(fabsf(t.h) < INFINITY)) {
+      t = dd(0.f);
+      for (int j = 0; j < kEvalThreads / 32; ++j) t.h += sm[j][threadIdx.x].x;
+    }
     part[(size_t)blockIdx.x * K + threadIdx.x] = make_float2(t.h, t.l);
   }
 }
@@ -65,9 +80,13 @@ __device__ __forceinline__ void sum_rows(const float2* __restrict__ part, int nb
 #pragma unroll 5
     for (int b = lane; b < nb; b += 32) {
       const float2 v = part[(size_t)b * K + k];
-      t = dd_accumulate(t, dd(v.x, v.y));
+      t = t + dd(v.x, v.y);
     }
-    t = warp_sum_dd(t);
+    if (!(fabsf(t.h) < INFINITY)) {
+      t = dd(0.f);
+      for (int b = lane; b < nb; b += 32) t.h += part[(size_t)b * K + k].x;
+    }
+    t = warp_sum_any(t);
     if (lane == 0) tot[k] = ((double)t.h + (double)t.l) / (double)kSumScale;
   }
   __syncthreads();
