@@ -1151,8 +1151,10 @@ __device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, boo
 // tile's copies are in flight while this one computes).  X's pixels are 80 bytes apart in shared
 // memory (16 channels + 4 of padding), so that 8 consecutive pixels fall on 8 different bank
 // quads.  The sums are updated by packed FP32 FMAs.
-//  * NO = 16: a thread owns 4 output x 8 input channels of one tap (32 sums) and a phase of the
+//  * NO = 16: a thread owns 8 output x 8 input channels of one tap (64 sums) and a phase of the
 //    pixels; within a warp the output-channel groups vary fastest, so the Z loads are broadcasts.
+//    Every 16-byte shared load of a warp holds the pipe 4 clocks, so 4 x 8 sums a thread (3 loads for
+//    16 packed FMAs) were bound by the loads (269 us at 1080p); 8 x 8 take 4 loads for 32.
 //  * NO = 3: warp w owns tap w, lane l the pixels of column l; a thread keeps 4 (3 used) x 16
 //    sums, and the warp adds its lanes' sums before the atomic additions.
 constexpr int kWgThreads = 288, kWgCols = 32, kWgPitch = 5;      // pitch: float4s per staged X pixel
@@ -1163,7 +1165,7 @@ struct WgShape {
   static constexpr size_t Smem = 2 * (size_t)(XF4 + ZF4) * 16;
 };
 template <int ZC, int NO, int ROWS>
-__global__ void __launch_bounds__(kWgThreads, NO > 4 ? 3 : 2) head_wgrad_kernel(const float* __restrict__ X, const float* __restrict__ Z,
+__global__ void __launch_bounds__(kWgThreads, 2) head_wgrad_kernel(const float* __restrict__ X, const float* __restrict__ Z,
                                                                 int H, int W, int tiles_x, int tiles, float scale,
                                                                 float* __restrict__ dW) {
   constexpr int NOG = (NO + 3) / 4;
@@ -1185,16 +1187,17 @@ __global__ void __launch_bounds__(kWgThreads, NO > 4 ? 3 : 2) head_wgrad_kernel(
     }
   };
   constexpr bool WIDE = NO > 4;                       // the two thread layouts above
-  constexpr int GROUPS = WIDE ? NOG * 2 * 9 : 9, PHASES = kWgThreads / GROUPS;
+  constexpr int NI = WIDE ? 8 : 4, NIG = WIDE ? NO / NI : 1;   // output channels a thread owns, and their groups
+  constexpr int GROUPS = WIDE ? NIG * 2 * 9 : 9, PHASES = kWgThreads / GROUPS;
   static_assert(kWgThreads % GROUPS == 0 && S::NPX % PHASES == 0 && (WIDE || kWgThreads == 9 * 32), "thread layout");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = WIDE ? threadIdx.x % GROUPS : warp, phase = WIDE ? threadIdx.x / GROUPS : lane;
-  const int og = WIDE ? grp % NOG : 0, ch = WIDE ? (grp / NOG) % 2 : 0, tap = WIDE ? grp / (2 * NOG) : warp;
+  const int og = WIDE ? grp % NIG : 0, ch = WIDE ? (grp / NIG) % 2 : 0, tap = WIDE ? grp / (2 * NIG) : warp;
   constexpr int NJ = WIDE ? 4 : 8;                    // float2 pairs of input channels a thread owns
   const int dy = tap / 3, dx = tap % 3;
-  float2 acc[4][NJ];
+  float2 acc[NI][NJ];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < NI; ++i)
 #pragma unroll
     for (int j = 0; j < NJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
   if (blockIdx.x < tiles) stage(0, blockIdx.x);
@@ -1208,10 +1211,15 @@ __global__ void __launch_bounds__(kWgThreads, NO > 4 ? 3 : 2) head_wgrad_kernel(
     __syncthreads();                                 // ... and everyone's
     const float4* sX = wg_smem + (k & 1) * (S::XF4 + S::ZF4);
     const float4* sZ = sX + S::XF4;
-#pragma unroll 4
+#pragma unroll (WIDE ? 1 : 4)
     for (int p = phase; p < S::NPX; p += PHASES) {
       const int r = p / kWgCols, c = p % kWgCols;
-      const float4 z = sZ[p * NOG + og];
+      float zz[NI];
+#pragma unroll
+      for (int q = 0; q < NI / 4; ++q) {
+        const float4 z = sZ[p * NOG + og * (NI / 4) + q];
+        zz[4 * q] = z.x; zz[4 * q + 1] = z.y; zz[4 * q + 2] = z.z; zz[4 * q + 3] = z.w;
+      }
       const float4* xp = sX + ((r + dy) * S::XW + c + dx) * kWgPitch + 2 * ch;
       float2 xx[NJ];
 #pragma unroll
@@ -1220,9 +1228,8 @@ __global__ void __launch_bounds__(kWgThreads, NO > 4 ? 3 : 2) head_wgrad_kernel(
         xx[2 * q] = make_float2(xv.x, xv.y);
         xx[2 * q + 1] = make_float2(xv.z, xv.w);
       }
-      const float zz[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < NI; ++i)
 #pragma unroll
         for (int j = 0; j < NJ; ++j) acc[i][j] = __ffma2_rn(make_float2(zz[i], zz[i]), xx[j], acc[i][j]);
     }
@@ -1231,29 +1238,34 @@ __global__ void __launch_bounds__(kWgThreads, NO > 4 ? 3 : 2) head_wgrad_kernel(
   cp_async_wait<0>();
   if constexpr (WIDE) {
     // the phases of one group add their sums in shared memory (the staging buffers are free), so
-    // that one thread a group makes the atomic additions
-    static_assert((size_t)kWgThreads * 32 * 4 <= S::Smem, "the reduction fits the staging buffers");
+    // that one thread a group makes the atomic additions; a quarter of the sums at a time
+    static_assert((size_t)kWgThreads * 16 * 4 <= S::Smem, "a quarter of the sums fits the staging buffers");
     float2* red = reinterpret_cast<float2*>(wg_smem);
-    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i0 = 0; i0 < NI; i0 += 2) {
+      __syncthreads();
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) red[(i * NJ + j) * kWgThreads + threadIdx.x] = acc[i][j];
-    __syncthreads();
+      for (int i = i0; i < i0 + 2; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) red[((i - i0) * NJ + j) * kWgThreads + threadIdx.x] = acc[i][j];
+      __syncthreads();
+      if (phase == 0) {
+#pragma unroll
+        for (int i = i0; i < i0 + 2; ++i)
+#pragma unroll
+          for (int j = 0; j < NJ; ++j)
+            for (int q = 1; q < PHASES; ++q) {
+              const float2 v = red[((i - i0) * NJ + j) * kWgThreads + threadIdx.x + q * GROUPS];
+              acc[i][j].x += v.x;
+              acc[i][j].y += v.y;
+            }
+      }
+    }
     if (phase != 0) return;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < NJ; ++j)
-        for (int q = 1; q < PHASES; ++q) {
-          const float2 v = red[(i * NJ + j) * kWgThreads + threadIdx.x + q * GROUPS];
-          acc[i][j].x += v.x;
-          acc[i][j].y += v.y;
-        }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int o = 4 * og + i;
+  for (int i = 0; i < NI; ++i) {
+    const int o = NI * og + i;
     if (o >= NO) continue;
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
@@ -1621,7 +1633,7 @@ extern "C" vg_status vg_appearance_loss(const float* img, const float* target, i
     note_launches(2);
     sum_rows_kernel<<<1, 512, 0, sd[1]>>>(F(L.db5), n6, 16, ta.cscale, gp + b_off(5));
     sum_rows_kernel<<<1, 512, 0, sd[1]>>>(F(L.db6), nhead, 3, ta.cscale, gp + b_off(6));
-    ok(launch_head_wgrad<16, 16, 4>(U, F(L.gZ), H, W, ta.cscale, gp + w_off(5), sms, sd[1]));
+    ok(launch_head_wgrad<16, 16, 8>(U, F(L.gZ), H, W, ta.cscale, gp + w_off(5), sms, sd[1]));
     ok(launch_head_wgrad<8, 3, 8>(Hh, F(L.gM), H, W, ta.cscale, gp + w_off(6), sms, sd[1]));
     TcArgs a5 = ta;
     a5.in = F(L.gZ);
