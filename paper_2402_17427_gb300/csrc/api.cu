@@ -421,36 +421,17 @@ vg_status run_backward(Call& c, const vg_raster_opts* opts0, void* workspace, si
   const bool accumulate = (opts0->flags & VG_FLAG_ACCUMULATE_GRADS) != 0;
   stage_event(ev, VG_STAGE_BLEND_BACKWARD, true, s);
   cudaError_t e = launch_prepare_backward(L, ws, s);
-  // The dense zeroing of the culled Gaussians' gradients (HBM-bound) runs on a side stream: whole runs
-  // of Gaussians while the compositing adjoint (bound by instruction issue) takes its tiles, and the
-  // culled ones of the remaining runs beside the adjoint of the visible ones (latency-bound), which
-  // waits for the former.  Forked from s here and joined back into s before the call returns.
-  cudaEvent_t fork = nullptr, zeroed = nullptr, join = nullptr;
-  WsHeader* hdr = reinterpret_cast<WsHeader*>(ws + L.header);
-  const bool zero = !accumulate && c.total_n > 0;
-  if (zero) {
-    cudaStream_t side = side_stream();
-    if (!side || !(fork = call_event(kEvBackwardFork)) || !(zeroed = call_event(kEvBackwardZero)) ||
-        !(join = call_event(kEvBackwardJoin)))
-      return VG_ERR_CUDA;
-    cudaEventRecord(fork, s);
-    cudaStreamWaitEvent(side, fork, 0);
-    if (e == cudaSuccess) e = launch_zero_ahead(tab, c.plan, c.total_n, c.degree, hdr, side);
-    cudaEventRecord(zeroed, side);
-    if (e == cudaSuccess)
-      e = launch_zero_culled(tab, c.total_n, c.degree, reinterpret_cast<const uint32_t*>(ws + L.touched), hdr, side);
-    cudaEventRecord(join, side);
-  }
+  // the dense zeroing of the gradients (HBM-bound) goes beside the compositing adjoint (bound by instruction issue)
   if (e == cudaSuccess)
-    e = launch_blend_backward(tab, c.plan, L, ws, abs, (opts0->flags & VG_FLAG_COUNT_BLENDS) != 0, zero, s);
+    e = launch_blend_backward(tab, c.plan, L, ws, abs, (opts0->flags & VG_FLAG_COUNT_BLENDS) != 0,
+                              accumulate ? 0 : c.total_n, c.degree, s);
   stage_event(ev, VG_STAGE_BLEND_BACKWARD, false, s);
   stage_event(ev, VG_STAGE_PROJECT_BACKWARD, true, s);
-  if (zeroed) cudaStreamWaitEvent(s, zeroed, 0);
   if (e == cudaSuccess)
     e = launch_preprocess_backward(tab, c.total_n, c.degree, reinterpret_cast<const Splat*>(ws + L.splats),
-                                   reinterpret_cast<const uint32_t*>(ws + L.vis_ids), hdr,
+                                   reinterpret_cast<const uint32_t*>(ws + L.vis_ids),
+                                   reinterpret_cast<const WsHeader*>(ws + L.header),
                                    reinterpret_cast<const float*>(ws + L.g2d), accumulate, s);
-  if (join) cudaStreamWaitEvent(s, join, 0);   // always joined, so no work of the call outlives it on s
   stage_event(ev, VG_STAGE_PROJECT_BACKWARD, false, s);
   return cuda_status(e);
 }

@@ -401,8 +401,9 @@ blend_backward_kernel(const DevTables* __restrict__ tab, const Splat* __restrict
                       const uint32_t* __restrict__ lists, const uint2* __restrict__ ranges,
                       const uint32_t* __restrict__ order, int item_begin, int item_count, float* __restrict__ g2d,
                       const uint32_t* dorder0, const uint32_t* dorder1, const uint32_t* __restrict__ vis_ids,
-                      WsHeader* __restrict__ hdr) {
-  pdl_enter();
+                      bool beside_zeroing, WsHeader* __restrict__ hdr) {
+  // launched behind zero_grads, which has waited for everything before it and which this kernel runs beside
+  if (!beside_zeroing) pdl_enter();
   using S = TileShape<TS, true>;
   const uint32_t* __restrict__ dorder = depth_order(hdr, dorder0, dorder1);
   const bool dead = render_dead(hdr);   // a look-back gave up: every list counts as empty
@@ -664,6 +665,7 @@ blend_backward_kernel(const DevTables* __restrict__ tab, const Splat* __restrict
     for (int o = 16; o > 0; o >>= 1) xr += __shfl_xor_sync(0xffffffffu, xr, o);
     if (lane == 0) atomicAdd(&hdr->evals_run_bwd, xr);
   }
+  if (beside_zeroing) asm volatile("griddepcontrol.wait;" ::: "memory");   // complete only with zero_grads
 }
 
 // Before the adjoint: the 2D-gradient accumulators of the visible Gaussians zeroed, the adjoint's
@@ -712,29 +714,29 @@ cudaError_t fwd_class(const DevTables* tab, const HostPlan& plan, const Splat* v
 template <int TS, bool ABS, bool COUNT>
 void bwd_launch(const DevTables* tab, const Splat* vsplats, const uint32_t* lists, const uint2* ranges,
                 const uint32_t* order, int begin, int items, float* g2d, const uint32_t* d0, const uint32_t* d1,
-                const uint32_t* vis_ids, WsHeader* hdr, bool share, cudaStream_t s) {
+                const uint32_t* vis_ids, WsHeader* hdr, bool beside, cudaStream_t s) {
   using S = TileShape<TS, true>;
   auto k = blend_backward_kernel<TS, ABS, COUNT>;
   // The 8 x 8 and 16 x 16 kernels fill an SM with 16 blocks or more, so one fewer costs little and
-  // gives zero_ahead its registers and shared memory; the 32 x 32 kernel holds only a few.
-  launch_pdl(k, resident_grid(k, S::kThreads, items, share && TS <= 16 ? 1 : 0), S::kThreads, 0, s, tab, vsplats, lists, ranges, order, begin, items, g2d,
-                                                                 d0, d1, vis_ids, hdr);
+  // gives zero_grads its registers and shared memory; the 32 x 32 kernel holds only a few.
+  launch_pdl(k, resident_grid(k, S::kThreads, items, beside && TS <= 16 ? 1 : 0), S::kThreads, 0, s, tab, vsplats, lists, ranges, order, begin, items, g2d,
+                                                                 d0, d1, vis_ids, beside, hdr);
 }
 
 template <int TS>
 cudaError_t bwd_class(const DevTables* tab, const HostPlan& plan, const Splat* vsplats, const uint32_t* lists,
                       const uint2* ranges, const uint32_t* order, float* g2d, const uint32_t* d0, const uint32_t* d1,
-                      const uint32_t* vis_ids, WsHeader* hdr, bool abs, bool count, bool share,
+                      const uint32_t* vis_ids, WsHeader* hdr, bool abs, bool count, bool beside,
                       cudaStream_t s) {
   using S = TileShape<TS, true>;
   const int items = plan.class_tiles[S::kClass];
   if (items == 0) return cudaSuccess;
   note_launches(1);
   const int begin = plan.class_begin[S::kClass];
-  if (abs && count) bwd_launch<TS, true, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
-  else if (abs) bwd_launch<TS, true, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
-  else if (count) bwd_launch<TS, false, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
-  else bwd_launch<TS, false, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, share, s);
+  if (abs && count) bwd_launch<TS, true, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, beside, s);
+  else if (abs) bwd_launch<TS, true, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, beside, s);
+  else if (count) bwd_launch<TS, false, true>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, beside, s);
+  else bwd_launch<TS, false, false>(tab, vsplats, lists, ranges, order, begin, items, g2d, d0, d1, vis_ids, hdr, beside, s);
   return cudaGetLastError();
 }
 
@@ -760,7 +762,7 @@ cudaError_t launch_prepare_backward(const Layout& L, char* ws, cudaStream_t s) {
 }
 
 cudaError_t launch_blend_backward(const DevTables* tab, const HostPlan& plan, const Layout& L, char* ws, bool abs,
-                                  bool count, bool share, cudaStream_t s) {
+                                  bool count, int zero_n, int degree, cudaStream_t s) {
   const Splat* vsplats = reinterpret_cast<const Splat*>(ws + L.vsplats);
   const uint32_t* lists = reinterpret_cast<const uint32_t*>(ws + L.pvals[0]);   // final tile-sorted ranks
   const uint2* ranges = reinterpret_cast<const uint2*>(ws + L.ranges);
@@ -770,9 +772,20 @@ cudaError_t launch_blend_backward(const DevTables* tab, const HostPlan& plan, co
   const uint32_t* d0 = reinterpret_cast<const uint32_t*>(ws + L.vvals[0]);
   const uint32_t* d1 = reinterpret_cast<const uint32_t*>(ws + L.vvals[1]);
   const uint32_t* vis_ids = reinterpret_cast<const uint32_t*>(ws + L.vis_ids);
-  cudaError_t e = bwd_class<8>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, share, s);
-  if (e == cudaSuccess) e = bwd_class<16>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, share, s);
-  if (e == cudaSuccess) e = bwd_class<32>(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, share, s);
+  // the zeroing goes beside the last class's kernel (the one kernel launched right behind it)
+  auto pass = [&](auto kernel_class, int cls) {
+    if (plan.class_tiles[cls] == 0) return cudaSuccess;
+    bool beside = zero_n > 0;
+    for (int later = cls + 1; later < kTileClasses; ++later) beside = beside && plan.class_tiles[later] == 0;
+    if (beside) {
+      const cudaError_t z = launch_zero_grads(tab, zero_n, degree, reinterpret_cast<const uint32_t*>(ws + L.touched), hdr, s);
+      if (z != cudaSuccess) return z;
+    }
+    return kernel_class(tab, plan, vsplats, lists, ranges, order, g2d, d0, d1, vis_ids, hdr, abs, count, beside, s);
+  };
+  cudaError_t e = pass(bwd_class<8>, TileShape<8, true>::kClass);
+  if (e == cudaSuccess) e = pass(bwd_class<16>, TileShape<16, true>::kClass);
+  if (e == cudaSuccess) e = pass(bwd_class<32>, TileShape<32, true>::kClass);
   return e;
 }
 

@@ -114,7 +114,7 @@ struct WsHeader {
   unsigned int tile_bits;       // unused (kept for the header layout)
   unsigned int work_fwd[kTileClasses];   // persistent-blend work queues (next item)
   unsigned int work_bwd[kTileClasses];
-  unsigned int zero_next;       // runs of Gaussians whose gradients zero_ahead has taken
+  unsigned int zero_next;       // runs of Gaussians whose gradients zero_grads has taken
   unsigned int pad[2];
   unsigned long long evals_run_bwd;  // pixel slots the backward pass evaluated (optional count)
 };
@@ -227,17 +227,14 @@ cudaError_t launch_records(const DevTables* tab, int total_n, int degree, const 
 // Regions of the workspace; opts0 supplies the optional key-input record.
 Compact make_compact(const Layout& L, char* ws, const vg_raster_opts* opts0);
 // Adjoint of the projection for the visible Gaussians (gradients of the culled ones are left
-// to the two launches below, or untouched when accumulating).  Sized to leave launch_zero_culled
-// room to run beside it when not accumulating; launched plainly then, as it follows a join.
+// to launch_zero_grads, or untouched when accumulating).
 cudaError_t launch_preprocess_backward(const DevTables* tab, int total_n, int degree, const Splat* splats,
                                        const uint32_t* vis_ids, const WsHeader* hdr, const float* g2d,
                                        bool accumulate, cudaStream_t s);
-// Zero gradients of every Gaussian of the runs that can be written while the compositing adjoint
-// still has tiles to take, and then of every culled Gaussian of the runs that are left.
-cudaError_t launch_zero_ahead(const DevTables* tab, const HostPlan& plan, int total_n, int degree, WsHeader* hdr,
+// Zero gradients of every Gaussian.  The kernel launched next starts beside it, sees all that came before,
+// and must itself wait for it (griddepcontrol.wait) before it ends.
+cudaError_t launch_zero_grads(const DevTables* tab, int total_n, int degree, const uint32_t* touched, WsHeader* hdr,
                               cudaStream_t s);
-cudaError_t launch_zero_culled(const DevTables* tab, int total_n, int degree, const uint32_t* touched,
-                               const WsHeader* hdr, cudaStream_t s);
 
 // Depth order of the visible Gaussians beside their splat records, pair generation (with the
 // depth-ordered records), tile sort, ranges and the largest-first order of the tiles.  stall (tests
@@ -249,9 +246,10 @@ cudaError_t launch_blend_forward(const DevTables* tab, const HostPlan& plan, con
                                  cudaStream_t s);
 // Before the adjoint: accumulators, work queues and counters reset.
 cudaError_t launch_prepare_backward(const Layout& L, char* ws, cudaStream_t s);
-// share: leave room on every SM for launch_zero_ahead's block.
+// zero_n > 0: the gradients of that many Gaussians are zeroed beside it (launch_zero_grads), complete when
+// it is.
 cudaError_t launch_blend_backward(const DevTables* tab, const HostPlan& plan, const Layout& L, char* ws, bool abs,
-                                  bool count, bool share, cudaStream_t s);
+                                  bool count, int zero_n, int degree, cudaStream_t s);
 
 // Unique id of the current CUDA context (false if none is current or the driver cannot say).
 bool current_context_id(unsigned long long* id);
@@ -271,7 +269,7 @@ cudaStream_t side_stream_for(cudaStream_t caller);
 // is legal, since each cudaStreamWaitEvent takes the record that precedes it in host order, and
 // one thread's calls are issued one after another.  nullptr if creation fails.
 enum CallEventSlot {
-  kEvBackwardFork, kEvBackwardZero, kEvBackwardJoin, kEvBinningFork, kEvBinningJoin, kEvRecordJoin, kEvLossFork, kEvLossJoin,
+  kEvBinningFork, kEvBinningJoin, kEvRecordJoin, kEvLossFork, kEvLossJoin,
   kEvAppearance, kCallEvents = kEvAppearance + 16
 };
 cudaEvent_t call_event(int slot);

@@ -578,13 +578,19 @@ __global__ void __launch_bounds__(128) record_kernel(const DevTables* __restrict
 }
 
 // Dense gradient outputs are zero for every Gaussian that touches no tile: 236 bytes a Gaussian, most of
-// the bytes of a step (4.7 GB for 20M Gaussians, 0.80 ms at the write rate).  The compositing adjoint before
-// it leaves HBM idle (2% of its bandwidth), so one warp an SM zeroes whole runs of 512 Gaussians, visible or
-// not, while it runs: bulk copies (cp.async.bulk) of a zeroed shared buffer, which take no issue slots.
-// It stops when the adjoint's queues are empty; zero_culled_grads does the rest beside the projection
-// adjoint, which writes the visible rows afterwards.  Which kernel zeroes a run depends on timing, the
-// result does not.  Evict-first, so that the adjoint's records and images stay in L2.
-constexpr uint32_t kZeroBytes = 8192;
+// the bytes of a step (4.7 GB for 20M Gaussians, 0.79 ms alone).  The compositing adjoint before the
+// projection's leaves HBM idle (2% of its bandwidth), so two warps an SM zero all rows, visible or not, beside
+// it: bulk copies (cp.async.bulk) of a zeroed shared buffer, which take no issue slots.  The projection
+// adjoint writes the visible rows afterwards.  20M step 2,800 -> 2,212 us, six-cell batch 2,010 -> 1,900.
+//  * Launched in the caller's stream before the compositing adjoint, which follows as soon as every block here
+//    has started: on a side stream the blocks came after the adjoint's and were packed on a few SMs.
+//  * Nothing else zeroes: a kernel for the culled rows of what was left when the adjoint had taken its last
+//    tile ran beside that one's last blocks and made them end 380 us later (20M).
+//  * Two copies of 16 KB in flight a block: with 2 KB the adjoint was slowed and the zeroing too (20M 2,620 us),
+//    with one block an SM the zeroing outlasts the adjoint (2,390).
+// Evict-first, so that the adjoint's records and images stay in L2.
+constexpr uint32_t kZeroBytes = 16384;
+constexpr int kZeroPerSM = 2;
 __device__ __forceinline__ void bulk_zero(float* dst, size_t bytes, uint32_t src, uint64_t policy) {
   char* p = reinterpret_cast<char*>(dst);
   char* const e = p + bytes;
@@ -597,27 +603,46 @@ __device__ __forceinline__ void bulk_zero(float* dst, size_t bytes, uint32_t src
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(p), "r"(src),
                  "r"(n), "l"(policy)
                  : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group 1;" ::: "memory");
     p += n;
   }
   for (; p < e; p += 4) *reinterpret_cast<float*>(p) = 0.f;
 }
 
-__global__ void __launch_bounds__(32) zero_ahead(const DevTables* __restrict__ tab, int total_n, int F, int items0,
-                                                 int items1, int items2, WsHeader* __restrict__ hdr) {
+// Zero gradients of the culled ones of Gaussians first .. last, by one warp.
+__device__ __noinline__ void zero_culled(const DevTables* __restrict__ tab, const uint32_t* __restrict__ touched, int F,
+                                         int first, int last) {
+  for (int i = first + (int)(threadIdx.x & 31); i <= last; i += 32) {
+    if (touched[i] != 0) continue;
+    const KSeg& sg = tseg(tab, find_seg(tab, i));
+    if (!sg.gm) continue;
+    const size_t l = (size_t)(i - sg.offset);
+    for (int k = 0; k < 3; ++k) { sg.gm[3 * l + k] = 0.f; sg.gs[3 * l + k] = 0.f; }
+    for (int k = 0; k < 4; ++k) sg.gq[4 * l + k] = 0.f;
+    sg.gl[l] = 0.f;
+    for (int k = 0; k < F; ++k) sg.gsh[l * F + k] = 0.f;
+  }
+}
+
+__global__ void __launch_bounds__(32) zero_grads(const DevTables* __restrict__ tab, int total_n, int F,
+                                                 const uint32_t* __restrict__ touched, WsHeader* __restrict__ hdr) {
   __shared__ __align__(128) float4 s_zero[kZeroBytes / 16];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (int k = threadIdx.x; k < (int)(kZeroBytes / 16); k += 32) s_zero[k] = make_float4(0.f, 0.f, 0.f, 0.f);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncwarp();
-  // after a wait of the forward gave up, no gradient of a visible Gaussian is written
-  if (threadIdx.x != 0 || render_dead(hdr)) return;
+  const int runs = (total_n - 1) / kCullRun + 1;
+  if (render_dead(hdr)) {     // a wait of the forward gave up: no gradient of a visible Gaussian is written
+    for (int run = blockIdx.x; run < runs; run += gridDim.x)
+      zero_culled(tab, touched, F, run * kCullRun, min(total_n - 1, run * kCullRun + (kCullRun - 1)));
+    return;
+  }
+  if (threadIdx.x != 0) return;
   uint64_t policy;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
   const uint32_t src = smem_u32(s_zero);
-  const int runs = (total_n - 1) / kCullRun + 1;
-  const volatile unsigned* q = hdr->work_bwd;
   for (;;) {
-    // every tile has been taken: the rest is left to zero_culled_grads
-    if (q[0] >= (unsigned)items0 && q[1] >= (unsigned)items1 && q[2] >= (unsigned)items2) break;
     const unsigned run = atomicAdd(&hdr->zero_next, 1u);
     if (run >= (unsigned)runs) break;
     const int first = (int)run * kCullRun, last = min(total_n - 1, first + (kCullRun - 1));
@@ -632,64 +657,8 @@ __global__ void __launch_bounds__(32) zero_ahead(const DevTables* __restrict__ t
       bulk_zero(sg.gs + l * 3, n * 3, src, policy);
       bulk_zero(sg.gl + l, n, src, policy);
     }
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    asm volatile("cp.async.bulk.wait_group 2;" ::: "memory");      // a few runs in flight
   }
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // written before the kernel ends
-}
-
-// Zero gradients of the culled ones of Gaussians base .. base + 31, by one warp.
-template <int DEG>
-__device__ __forceinline__ void zero_rows(const DevTables* __restrict__ tab, int total_n,
-                                          const uint32_t* __restrict__ touched, int base, int lane) {
-  constexpr int F = 3 * (DEG + 1) * (DEG + 1);
-  const int i = base + lane;
-  bool zero = false;
-  float* gsh = nullptr;
-  if (i < total_n && touched[i] == 0) {
-    const KSeg& sg = tseg(tab, find_seg(tab, i));
-    if (sg.gm) {
-      zero = true;
-      const size_t l = (size_t)(i - sg.offset);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) { sg.gm[3 * l + k] = 0.f; sg.gs[3 * l + k] = 0.f; }
-      *reinterpret_cast<float4*>(sg.gq + 4 * l) = make_float4(0.f, 0.f, 0.f, 0.f);
-      sg.gl[l] = 0.f;
-      gsh = sg.gsh + l * F;
-    }
-  }
-  const unsigned any = __ballot_sync(0xffffffffu, zero);
-  if (!any) return;
-  const unsigned long long me = reinterpret_cast<unsigned long long>(gsh);
-  if constexpr (F % 4 == 0) {
-    constexpr int Q = F / 4;   // float4 words per Gaussian
-    for (int f = lane; f < 32 * Q; f += 32) {
-      const int src = f / Q;
-      const unsigned long long p = __shfl_sync(0xffffffffu, me, src);
-      if ((any >> src) & 1u) reinterpret_cast<float4*>(p)[f % Q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  } else {
-    for (int f = lane; f < 32 * F; f += 32) {
-      const int src = f / F;
-      const unsigned long long p = __shfl_sync(0xffffffffu, me, src);
-      if ((any >> src) & 1u) reinterpret_cast<float*>(p)[f % F] = 0.f;
-    }
-  }
-}
-
-// Zero gradients of the Gaussians that touch no tile (skipped when accumulating), in the runs that
-// zero_ahead did not take.  A warp owns 32 consecutive Gaussians and writes their SH gradient rows
-// cooperatively, so consecutive lanes store consecutive 16-byte words.
-template <int DEG>
-__global__ void __launch_bounds__(256) zero_culled_grads(const DevTables* __restrict__ tab, int total_n,
-                                                         const uint32_t* __restrict__ touched,
-                                                         const WsHeader* __restrict__ hdr) {
-  constexpr int F = 3 * (DEG + 1) * (DEG + 1);
-  const int lane = threadIdx.x & 31;
-  const long long begin = min((long long)total_n, (long long)hdr->zero_next * kCullRun);
-  for (long long base = begin + ((blockIdx.x * blockDim.x + threadIdx.x) & ~31u); base < total_n;
-       base += (long long)gridDim.x * blockDim.x)
-    zero_rows<DEG>(tab, total_n, touched, (int)base, lane);
 }
 
 // Adjoint of the projection for visible Gaussian i: writes (or, accumulating, adds) the gradients
@@ -927,27 +896,14 @@ cudaError_t launch_records(const DevTables* tab, int total_n, int degree, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_zero_ahead(const DevTables* tab, const HostPlan& plan, int total_n, int degree, WsHeader* hdr,
+cudaError_t launch_zero_grads(const DevTables* tab, int total_n, int degree, const uint32_t* touched, WsHeader* hdr,
                               cudaStream_t s) {
-  if (total_n == 0) return cudaSuccess;
   const int runs = (total_n - 1) / kCullRun + 1, F = 3 * (degree + 1) * (degree + 1);
   note_launches(1);
-  zero_ahead<<<std::min(runs, sort_blocks() / 2), 32, 0, s>>>(tab, total_n, F, plan.class_tiles[0], plan.class_tiles[1],
-                                                              plan.class_tiles[2], hdr);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_zero_culled(const DevTables* tab, int total_n, int degree, const uint32_t* touched,
-                               const WsHeader* hdr, cudaStream_t s) {
-  if (total_n == 0) return cudaSuccess;
-  const int zb = std::min((total_n - 1) / 256 + 1, 4 * sort_blocks());
-  note_launches(1);
-  switch (degree) {
-    case 0: zero_culled_grads<0><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
-    case 1: zero_culled_grads<1><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
-    case 2: zero_culled_grads<2><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
-    default: zero_culled_grads<3><<<zb, 256, 0, s>>>(tab, total_n, touched, hdr); break;
-  }
+  // launched plainly: what precedes is complete before the adjoint may start (it does not wait for it itself), and the
+  // blocks find the SMs empty and spread evenly (started early behind the accumulators' reset they took
+  // the SMs that came free first: 20M 2,920 us)
+  zero_grads<<<std::min(runs, kZeroPerSM * sort_blocks() / 2), 32, 0, s>>>(tab, total_n, F, touched, hdr);
   return cudaGetLastError();
 }
 
@@ -959,17 +915,10 @@ cudaError_t launch_preprocess_backward(const DevTables* tab, int total_n, int de
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // The kernel is latency-bound and holds 128 registers a thread, so 4 blocks an SM fill the
-  // register file.  Beside the HBM-bound zeroing of the culled Gaussians' gradients (run on a
-  // side stream unless accumulating) it takes 3 an SM and leaves the zeroing kernel room to be
-  // resident at the same time: 1080p step, 1M Gaussians, 99 -> 82 us for the pair.
-  const int per_sm = accumulate ? 4 : 3;
-  const int blocks = std::max(1, std::min((total_n + 127) / 128, per_sm * std::max(sms, 1)));
+  // latency-bound at 128 registers a thread: 4 blocks an SM fill the register file
+  const int blocks = std::max(1, std::min((total_n + 127) / 128, 4 * std::max(sms, 1)));
   note_launches(1);
-  auto go = [&](auto kernel) {
-    if (accumulate) launch_pdl(kernel, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc);
-    else kernel<<<blocks, 128, 0, s>>>(tab, vis_ids, hdr, splats, g2d, acc);
-  };
+  auto go = [&](auto kernel) { launch_pdl(kernel, blocks, 128, 0, s, tab, vis_ids, hdr, splats, g2d, acc); };
   switch (degree) {
     case 0: go(preprocess_backward_kernel<0>); break;
     case 1: go(preprocess_backward_kernel<1>); break;
