@@ -45,16 +45,16 @@ OPS_EVAL, OPS_BLEND_FWD, OPS_BLEND_BWD = 11, 7, 37
 TRAFFIC_SOURCES = ("paper_2402_17427_gb300/csrc/blend.cu", "paper_2402_17427_gb300/csrc/vg_common.cuh",
                    "paper_2402_17427_gb300/csrc/internal.h")
 PROFILED_TRAFFIC = {
-    "sources_sha256": "41622bed1adda167cb60d63ef8b9ece17d6e7f7cf8280c257725cd320cd9aed1",
-    "blend": 18660864 + 1536768,
-    "blend_backward": 67457536 + 1475328,
+    "sources_sha256": "045fdd8d1d7be9bdb9a1cf070434eaf029129e0c8d21e081908cd592ccaabf3e",
+    "blend": 18678784 + 508416,
+    "blend_backward": 67458304 + 86784,
 }
 # Warp instructions issued per launch (smsp__inst_executed.sum) of the compositing kernels on this
 # workload, from the same captures; held to the same source hash.
 PROFILED_INSTRUCTIONS = {
-    "sources_sha256": "41622bed1adda167cb60d63ef8b9ece17d6e7f7cf8280c257725cd320cd9aed1",
+    "sources_sha256": "045fdd8d1d7be9bdb9a1cf070434eaf029129e0c8d21e081908cd592ccaabf3e",
     "blend": 259017717,
-    "blend_backward": 357429896,
+    "blend_backward": 357442664,
 }
 
 
