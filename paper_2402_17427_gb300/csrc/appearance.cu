@@ -685,42 +685,52 @@ __global__ void __launch_bounds__(256) conv0_embed_grad_kernel(const float* __re
 // with hi = tf32(x) and lo = tf32(x - hi), and each product is formed as lo.hi + hi.lo + hi.hi, so the
 // products are FP32-accurate (relative error about 2^-21; the dropped lo.lo term is below FP32 rounding).
 //
-// What bounds them is the shared-memory traffic of the activation operand, so one read of it serves as
-// many products as possible: M = 128 input pixels (4 rows of 32), K = the 3 rows of taps x the input's
-// channels, and N holds all three columns of taps, 3 x NO outputs, hi and lo weights side by side:
-//   D[p][dx][o] = sum over dy, c of X(y + dy - 1, x)[c] W[o][c][dy][dx],
-// one MMA with A_hi against [W_hi | W_lo] and one with A_lo against W_hi into the second half.  The
-// epilogue adds the halves and gathers the taps, out(y, x) = sum over dx of D[(y, x + dx - 1)][dx]: lanes are
-// consecutive pixels of a row, so the neighbours' parts come by one shuffle each and 30 of a row's
-// 32 pixels are outputs.  With the nine taps one after another (N = 32, the activations read 18 times
-// instead of 6 for 16 channels) a pass at 1080p took 119 us.
+// What bounds them is the shared-memory traffic of the activation operand.  M = 128 pixels (4 rows of 32), hi
+// and lo weights are side by side in N, and a k-step takes one MMA with A_hi against [W_hi | W_lo] and
+// one with A_lo against W_hi into the second half; the epilogue adds the halves.  The taps go two ways:
+//  * Adjoint passes (linear in what follows): one read of the activations serves as many products as
+//    possible.  K = the 3 rows of taps x the input's channels, and N holds all three columns of taps:
+//      D[p][dx][o] = sum over dy, c of X(y + dy - 1, x)[c] W[o][c][dy][dx].
+//    The epilogue gathers the taps, out(y, x) = sum over dx of D[(y, x + dx - 1)][dx]: lanes are consecutive
+//    pixels of a row, so the neighbours' parts come by one shuffle each.
+//  * Forward passes (kSeq): the nine taps one after another in K, (dy, dx) = (0, 0), (0, 1), ... (2, 2), N = one
+//    set of outputs.  Conv5's sums gate the gradient by their sign and conv6's set that of the L1 term, so
+//    an output whose sum is within rounding of zero changes the gradients by far more than rounding when
+//    the order of its additions changes (on a small image one crossing moves the embedding's by some 1e-5
+//    of its norm).  This order is therefore part of what the passes compute.
+// Either way 30 of a row's 32 pixels are outputs.
 //
 // Shared-memory operands use the no-swizzle K-major layout: a core matrix is 8 rows of 16 bytes
 // (4 channels).  The patch (10 rows x 32 pixels for 8 rows of outputs) is stored [part][channel
 // group][10][32][4 floats]: core matrices follow one another along M, the next channel group is one
-// plane further, a tap row dy moves the start address by 512 bytes.  Planes are 128 / groups bytes
-// longer than their data, so that the groups of the pixels that eight lanes write fall on distinct banks.
-// Weights are [dy][group][part][dx][o][4 channels].
+// plane further, a tap row dy moves the start address by 512 bytes and (kSeq) a tap column dx by 16.  Planes
+// are 128 / groups bytes longer than their data, so that the groups of the pixels that eight lanes write
+// fall on distinct banks.  Weights are [dy][group][part][dx][o][4 channels], kSeq: [dy][dx][group][part][o][4].
 
 constexpr int kTcThreads = 256;                      // eight warps, an output row each; one thread issues
 constexpr int kTcRows = 8, kTcCols = 30;             // outputs of a tile (two M-tiles of 4 rows x 32 pixels)
 constexpr int kPatchH = kTcRows + 2, kPatchW = 32, kPatchPx = kPatchH * kPatchW;
 constexpr uint64_t kTcWaitNs = 1000000000ull;        // bounded wait for the MMAs of one tile (1 s)
 enum : int { kEpiRelu = 0, kEpiL1 = 1, kEpiMask = 2, kEpiStore = 3 };
+template <int EPI>
+constexpr bool kTcForward = EPI == kEpiRelu || EPI == kEpiL1;
 
-template <int C, int NO>
+template <int C, int NO, bool kSeq>
 struct TcShape {
   static constexpr int CG = C / 4;                           // channel groups (K = 8 per MMA: 2 groups)
-  static constexpr int N1 = 3 * NO;                          // outputs of the three tap columns
+  static constexpr int NX = kSeq ? 1 : 3, KT = 9 / NX;       // tap columns side by side in N, taps in K
+  static constexpr int N1 = NX * NO;                         // outputs side by side
   static constexpr int N2 = (N1 + 15) / 16 * 16;             // N of the A_lo MMA (past N1: columns nobody reads)
   static constexpr uint32_t Plane = kPatchPx * 16 + 128 / CG;   // one channel group of a patch part
   static constexpr uint32_t PartA = CG * Plane;
   static constexpr uint32_t BufA = 2 * PartA;                // hi and lo parts of one patch
-  static constexpr uint32_t GroupB = 2 * N1 * 16;            // one tap row and channel group, both parts
-  static constexpr uint32_t SizeB = 3 * CG * GroupB;
+  static constexpr uint32_t GroupB = 2 * N1 * 16;            // one K tap and channel group, both parts
+  static constexpr uint32_t SizeB = KT * CG * GroupB;
   static constexpr uint32_t Smem = 2 * BufA + SizeB;         // two patch buffers + weights
-  static constexpr uint32_t Acc = N1 + N2 <= 64 ? 64 : 128;  // tensor-memory columns of an M-tile
+  static constexpr uint32_t Acc = N1 + N2 <= 32 ? 32 : N1 + N2 <= 64 ? 64 : 128;   // tensor-memory columns of an M-tile
   static_assert(2 * N1 % 16 == 0 && N1 + N2 <= Acc, "accumulator layout");
+  // the last pixels of a shifted M-tile lie past the patch: within the plane's padding, and never outputs
+  static_assert(!kSeq || Plane >= (kPatchPx + 2) * 16, "a shifted operand stays in its plane");
 };
 
 struct TcArgs {
@@ -746,9 +756,9 @@ __device__ __forceinline__ float4 split_lo(float4 v, float4 h) {
 
 // B[n][tap][k]: forward W[n][k][tap]; adjoint W[k][n][8 - tap] (n = the layer's input channel).
 // Entries past the layer's channels are zero.
-template <int C, int NO>
+template <int C, int NO, bool kSeq>
 __device__ void tc_stage_weights(unsigned char* sB, const TcArgs& a) {
-  using S = TcShape<C, NO>;
+  using S = TcShape<C, NO, kSeq>;
   for (int i = threadIdx.x; i < 9 * S::CG * NO; i += kTcThreads) {
     const int n = i % NO, cg = (i / NO) % S::CG, tap = i / (NO * S::CG);
     float v[4];
@@ -759,7 +769,7 @@ __device__ void tc_stage_weights(unsigned char* sB, const TcArgs& a) {
       else v[j] = (k < a.wo && n < a.wc) ? __ldg(a.w + ((size_t)k * a.wc + n) * 9 + (8 - tap)) : 0.f;
     }
     const float4 x = make_float4(v[0], v[1], v[2], v[3]), h = split_hi(x);
-    const uint32_t off = (uint32_t)((tap / 3) * S::CG + cg) * S::GroupB + (uint32_t)((tap % 3) * NO + n) * 16;
+    const uint32_t off = (uint32_t)((tap / S::NX) * S::CG + cg) * S::GroupB + (uint32_t)((tap % S::NX) * NO + n) * 16;
     *reinterpret_cast<float4*>(sB + off) = h;
     *reinterpret_cast<float4*>(sB + off + S::N1 * 16) = split_lo(x, h);
   }
@@ -787,9 +797,8 @@ __device__ __forceinline__ void tc_load_patch(TcPatch<C>& r, const float* __rest
       r.v[q] = __ldg(reinterpret_cast<const float4*>(in + ((size_t)Y * W + X) * C) + cg);
   }
 }
-template <int C, int NO>
+template <int C, typename S>
 __device__ __forceinline__ void tc_store_patch(unsigned char* sA, const TcPatch<C>& r) {
-  using S = TcShape<C, NO>;
 #pragma unroll
   for (int q = 0; q < TcPatch<C>::IT; ++q) {
     const int i = threadIdx.x + kTcThreads * q;
@@ -802,22 +811,22 @@ __device__ __forceinline__ void tc_store_patch(unsigned char* sA, const TcPatch<
   }
 }
 
-// The MMAs of one tile: two M-tiles x 3 tap rows x C / 8 k-steps x 2.  The descriptors of the patch
+// The MMAs of one tile: two M-tiles x the taps in K x C / 8 k-steps x 2.  The descriptors of the patch
 // buffer's and the weights' first core matrices are formed once; an operand's offset only adds to the
 // start-address field (16-byte units, no carry: shared addresses stay below 2^18).
-template <int C, int NO>
+template <int C, typename S>
 __device__ __forceinline__ void tc_issue(uint64_t a_hi, uint64_t b_desc, uint32_t d) {
-  using S = TcShape<C, NO>;
   constexpr uint32_t idesc_hi = tc::idesc_tf32(128, 2 * S::N1), idesc_lo = tc::idesc_tf32(128, S::N2);
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int dy = 0; dy < 3; ++dy)
+    for (int t = 0; t < S::KT; ++t)
 #pragma unroll
       for (int ks = 0; ks < C / 8; ++ks) {
-        const uint64_t ao = (2 * ks * S::Plane + (uint32_t)(4 * mt + dy) * kPatchW * 16) >> 4;
-        const uint64_t bo = (uint64_t)((dy * S::CG + 2 * ks) * S::GroupB) >> 4;
-        tc::mma_tf32(d + mt * S::Acc, a_hi + ao, b_desc + bo, idesc_hi, dy + ks > 0);                       // A_hi [W_hi | W_lo]
+        const int dy = S::NX == 1 ? t / 3 : t, dx = S::NX == 1 ? t % 3 : 0;
+        const uint64_t ao = (2 * ks * S::Plane + (uint32_t)((4 * mt + dy) * kPatchW + dx) * 16) >> 4;
+        const uint64_t bo = (uint64_t)((t * S::CG + 2 * ks) * S::GroupB) >> 4;
+        tc::mma_tf32(d + mt * S::Acc, a_hi + ao, b_desc + bo, idesc_hi, t + ks > 0);                        // A_hi [W_hi | W_lo]
         tc::mma_tf32(d + mt * S::Acc + S::N1, a_hi + ao + (S::PartA >> 4), b_desc + bo, idesc_lo, true);    // A_lo W_hi
       }
 }
@@ -834,18 +843,20 @@ struct TcEpiIn {
   float4 x[4];
 };
 
-// The thread's output pixel: row = warp, column = lane - 1 (lanes 0 and 31 only feed their neighbours).
+// The thread's output pixel: row = warp, column = lane - 1 (lanes 0 and 31 only feed their neighbours),
+// kSeq: column = lane (lanes 30 and 31 have none).
+template <bool kSeq>
 __device__ __forceinline__ bool tc_pixel(const TcArgs& a, int tile, int& Y, int& X) {
-  const int lane = threadIdx.x & 31;
+  const int col = (int)(threadIdx.x & 31) - (kSeq ? 0 : 1);
   Y = (tile / a.tiles_x) * kTcRows + (int)(threadIdx.x >> 5);
-  X = (tile % a.tiles_x) * kTcCols + lane - 1;
-  return lane >= 1 && lane <= kTcCols && Y < a.H && X < a.W;
+  X = (tile % a.tiles_x) * kTcCols + col;
+  return col >= 0 && col < kTcCols && Y < a.H && X < a.W;
 }
 
-template <int EPI>
+template <int EPI, bool kSeq>
 __device__ __forceinline__ void tc_load_epi(const TcArgs& a, int tile, TcEpiIn& e) {
   int Y, X;
-  if (!tc_pixel(a, tile, Y, X)) return;
+  if (!tc_pixel<kSeq>(a, tile, Y, X)) return;
   const size_t pix = (size_t)Y * a.W + X;
   if constexpr (EPI == kEpiMask) {
 #pragma unroll
@@ -873,28 +884,33 @@ __device__ __forceinline__ void tc_column(uint32_t tm, float (&v)[8], int n1) {
   for (int j = 0; j < 8; ++j) v[j] += w[j];
 }
 
-// Epilogue of one tile: waits for its MMAs, gathers the thread's pixel from the three tap columns and
-// applies the layer's output step.  Returns false if the wait gave up.
-template <int C, int NO, int EPI>
+// Epilogue of one tile: waits for its MMAs, takes the thread's pixel (gathered from the three tap columns
+// unless kSeq) and applies the layer's output step.  Returns false if the wait gave up.
+template <int C, int NO, int EPI, bool kSeq>
 __device__ __forceinline__ bool tc_epilogue(const TcArgs& a, int tile, uint32_t tmem, uint64_t* mbar, uint32_t parity,
                                             const TcEpiIn& e, TcSums& sums) {
-  using S = TcShape<C, NO>;
+  using S = TcShape<C, NO, kSeq>;
   const int warp = threadIdx.x >> 5;
   const bool ok = tc::mbar_wait(mbar, parity, kTcWaitNs);
   __syncwarp();
   tc::fence_after_sync();
   // row m of M-tile mt is lane m of tensor memory; a warp reads its quarter of the lanes
   const uint32_t tm = tmem + (uint32_t)(warp >> 2) * S::Acc + ((uint32_t)(32 * (warp & 3)) << 16);
-  float v[NO], t[NO];
-  tc_column(tm + NO, v, S::N1);                     // dx = 1: the pixel's own column
-  tc_column(tm, t, S::N1);                          // dx = 0: from the column to the left
+  float v[NO];
+  if constexpr (kSeq) {
+    tc_column(tm, v, S::N1);
+  } else {
+    float t[NO];
+    tc_column(tm + NO, v, S::N1);                   // dx = 1: the pixel's own column
+    tc_column(tm, t, S::N1);                        // dx = 0: from the column to the left
 #pragma unroll
-  for (int j = 0; j < NO; ++j) v[j] += __shfl_up_sync(0xffffffffu, t[j], 1);
-  tc_column(tm + 2 * NO, t, S::N1);                 // dx = 2: from the column to the right
+    for (int j = 0; j < NO; ++j) v[j] += __shfl_up_sync(0xffffffffu, t[j], 1);
+    tc_column(tm + 2 * NO, t, S::N1);               // dx = 2: from the column to the right
 #pragma unroll
-  for (int j = 0; j < NO; ++j) v[j] += __shfl_down_sync(0xffffffffu, t[j], 1);
+    for (int j = 0; j < NO; ++j) v[j] += __shfl_down_sync(0xffffffffu, t[j], 1);
+  }
   int Y, X;
-  if (!tc_pixel(a, tile, Y, X) || !ok) return ok;
+  if (!tc_pixel<kSeq>(a, tile, Y, X) || !ok) return ok;
   const size_t pix = (size_t)Y * a.W + X;
   if constexpr (EPI == kEpiRelu) {
     float4* o = reinterpret_cast<float4*>(a.out + pix * 16);
@@ -946,7 +962,8 @@ __device__ __forceinline__ bool tc_epilogue(const TcArgs& a, int tile, uint32_t 
 
 template <int C, int NO, int EPI>
 __global__ void __launch_bounds__(kTcThreads, 2) tc_conv_kernel(const TcArgs a) {
-  using S = TcShape<C, NO>;
+  constexpr bool kSeq = kTcForward<EPI>;
+  using S = TcShape<C, NO, kSeq>;
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   unsigned char* sA = tc_smem;                 // two patch buffers
   unsigned char* sB = tc_smem + 2 * S::BufA;   // the weights
@@ -967,8 +984,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_conv_kernel(const TcArgs a) 
   TcEpiIn epi;
   int tile = blockIdx.x;
   load(pre, tile);
-  tc_stage_weights<C, NO>(sB, a);
-  if (tile < a.tiles) tc_store_patch<C, NO>(sA, pre);
+  tc_stage_weights<C, NO, kSeq>(sB, a);
+  if (tile < a.tiles) tc_store_patch<C, S>(sA, pre);
   load(pre, tile + gridDim.x);
   tc::fence_smem_to_async();
   tc::fence_before_sync();
@@ -987,13 +1004,13 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_conv_kernel(const TcArgs a) 
     const int b = k & 1;
     if (tid == 0) {
       tc::fence_after_sync();
-      tc_issue<C, NO>(a_desc + ((b * S::BufA) >> 4), b_desc, tmem);
+      tc_issue<C, S>(a_desc + ((b * S::BufA) >> 4), b_desc, tmem);
       tc::commit(&mbar);
     }
-    if (tile + gridDim.x < a.tiles) tc_store_patch<C, NO>(sA + (b ^ 1) * S::BufA, pre);
+    if (tile + gridDim.x < a.tiles) tc_store_patch<C, S>(sA + (b ^ 1) * S::BufA, pre);
     load(pre, tile + 2 * gridDim.x);
-    tc_load_epi<EPI>(a, tile, epi);
-    ok &= tc_epilogue<C, NO, EPI>(a, tile, tmem, &mbar, k & 1, epi, sums);
+    tc_load_epi<EPI, kSeq>(a, tile, epi);
+    ok &= tc_epilogue<C, NO, EPI, kSeq>(a, tile, tmem, &mbar, k & 1, epi, sums);
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();             // accumulators read, the next patch written
@@ -1454,7 +1471,7 @@ cudaError_t launch_wgrad(const float* Aprev, const float* gA, const float* A, fl
 // each, fills the 512 of an SM), at most one per tile.
 template <int C, int NO, int EPI>
 cudaError_t launch_tc_conv(const TcArgs& a, int sms, cudaStream_t s, int* grid_out = nullptr) {
-  using S = TcShape<C, NO>;
+  using S = TcShape<C, NO, kTcForward<EPI>>;
   auto k = tc_conv_kernel<C, NO, EPI>;
   cudaError_t e = set_smem(k, S::Smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
