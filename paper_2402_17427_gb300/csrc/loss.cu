@@ -2,9 +2,8 @@
 //
 // SSIM uses an 11x11 Gaussian window (sigma 1.5, separable, normalised) with zero padding and
 // C1 = 0.01^2, C2 = 0.03^2; both terms are means over 3 H W.  With the local moments
-// mx = w*x, my = w*y, ess = w*(x^2 + y^2), exy = w*(x y),
-//   S = (2 mx my + C1)(2 (exy - mx my) + C2) / ((mx^2 + my^2 + C1)(ess - mx^2 - my^2 + C2))
-// (the two second moments only enter as their sum, so four windows do instead of five),
+// mx = w*x, exx = w*x^2, exy = w*(x y) (and my, eyy),
+//   S = (2 mx my + C1)(2 (exy - mx my) + C2) / ((mx^2 + my^2 + C1)(exx - mx^2 + eyy - my^2 + C2))
 // and dL/dx(q) = l1' + (w * a)(q) + 2 x(q) (w * b)(q) + y(q) (w * c)(q), where a, b, c are
 // dL/dS times dS/dmx, dS/dexx, dS/dexy at every pixel (the window is symmetric, so correlation
 // with it is its own adjoint).  Two kernels: moments -> (a, b, c) maps + partial sums, then the
@@ -56,7 +55,7 @@ __device__ __forceinline__ int qcol(int q) { return q + (q >> 3); }
 __device__ __forceinline__ int hs_at(int r, int c) { return r * LT + 2 * ((c >> 1) ^ ((r >> 1) & 3)) + (c & 1); }
 
 // Rows 2p and 2p + 1, columns c .. c + GH - 1 of F quantities, two columns a store: the moment pass is bound
-// by the shared-memory pipe, and single columns took twice its clocks (51.5 -> 47.6 us at 1080p).
+// by the shared-memory pipe, and single columns take twice its clocks for these stores (53.4 -> 51.9 us at 1080p).
 template <int F>
 __device__ __forceinline__ void store_rows(const float2 (&a)[F][GH], float (*hs)[LTH * LT], int p, int c) {
 #pragma unroll
@@ -174,7 +173,10 @@ __device__ __forceinline__ void stage_pairs(const float* const (&plane)[F], int 
 
 // Moments of a 32x32 output tile: x, y staged with a 5-pixel zero-padded halo as row pairs.  The
 // horizontal pass (21 row pairs x 4 groups of 8 columns) slides the window along a row for two
-// rows at once; the vertical pass (32 columns x 4 groups of 8 rows) slides it down a column.
+// rows at once; the vertical pass (32 columns x 4 groups of 8 rows) slides it down a column.  The
+// values enter as they are: relative to one pixel of the tile (which halves the rounding of smooth images)
+// a pixel unlike its surroundings cost the whole tile its digits, and with x^2 + y^2 in one window instead
+// of two (four windows: 47 us instead of 52) the gradient's error was 1.12 times as large.
 // kMaps: the derivative maps for the gradient pass are written; without it the pass leaves the
 // partial sums alone (the evaluation needs no gradient).
 template <bool kMaps>
@@ -184,40 +186,34 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
                                                                     double* __restrict__ partials) {
   pdl_enter();
   __shared__ __align__(16) float4 s4[NRP][QP];   // (x row 2p, x row 2p + 1, y row 2p, y row 2p + 1)
-  __shared__ __align__(16) float hs[4][LTH * LT];
+  __shared__ __align__(16) float hs[5][LTH * LT];
   __shared__ double red[kLossThreads / 32];
   const int c = blockIdx.z;
   const int ox = blockIdx.x * LT, oy = blockIdx.y * LT;
   const size_t plane = (size_t)W * H;
-  // Every value of the tile, its zero padding too, is taken relative to the rendering at the tile's middle:
-  // variances and covariance do not change, and their cancellation (mean of squares less square of
-  // mean) is of small numbers where the image is smooth.  The sum of both second moments alone made the
-  // gradient's error 1.12 times that of two (photograph-like images: 3.4e-6 against 3.0e-6).
-  float base = __ldg(x + c * plane + (size_t)min(oy + LT / 2, H - 1) * W + min(ox + LT / 2, W - 1));
-  base = fabsf(base) <= 1024.f ? base : 0.f;     // 0 for a NaN
   {
     const float* const src[2] = {x + c * plane, y + c * plane};
     stage_pairs<2>(src, W, H, ox, oy, [&](int p, int q, const float2 (&v)[2]) {
-      s4[p][q] = make_float4(v[0].x - base, v[0].y - base, v[1].x - base, v[1].y - base);
+      s4[p][q] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
     });
   }
   __syncthreads();
   if (threadIdx.x < NH) {
     const int p = threadIdx.x >> 2, g = threadIdx.x & 3;
-    float2 a[4][GH];
-    window_pairs<4, GH>(win, [&](int i, float2 (&v)[4]) {
+    float2 a[5][GH];
+    window_pairs<5, GH>(win, [&](int i, float2 (&v)[5]) {
       const float4 s = s4[p][qcol(GH * g + i)];
       const float2 xv = make_float2(s.x, s.y), yv = make_float2(s.z, s.w);
-      v[0] = xv; v[1] = yv; v[2] = __ffma2_rn(xv, xv, __fmul2_rn(yv, yv)); v[3] = __fmul2_rn(xv, yv);
+      v[0] = xv; v[1] = yv; v[2] = __fmul2_rn(xv, xv); v[3] = __fmul2_rn(yv, yv); v[4] = __fmul2_rn(xv, yv);
     }, a);
     store_rows(a, hs, p, GH * g);
   }
   __syncthreads();
   const int q = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * GV;   // column q, output rows r0 .. r0 + 7
-  float m[4][GV];
-  window_column<4>(win, [&](int i, float (&v)[4]) {
+  float m[5][GV];
+  window_column<5>(win, [&](int i, float (&v)[5]) {
 #pragma unroll
-    for (int f = 0; f < 4; ++f) v[f] = hs[f][hs_at(r0 + i, q)];
+    for (int f = 0; f < 5; ++f) v[f] = hs[f][hs_at(r0 + i, q)];
   }, m);
   // the per-pixel SSIM and its three partial derivatives for two rows at once (packed FP32; the
   // reciprocals approximate, within 1 ulp)
@@ -240,19 +236,18 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
       const float* cell = sf + ((sr >> 1) * QP + qcol(q + HALO)) * 4;
       l1sum += fabsf(cell[sr & 1] - cell[2 + (sr & 1)]);
     }
-    const float2 dx = make_float2(m[0][j], m[0][j + 1]), dy = make_float2(m[1][j], m[1][j + 1]);
-    const float2 ess = make_float2(m[2][j], m[2][j + 1]), exy = make_float2(m[3][j], m[3][j + 1]);
-    const float2 sss = __fadd2_rn(ess, neg(__ffma2_rn(dx, dx, __fmul2_rn(dy, dy))));
-    const float2 sxy = __fadd2_rn(exy, neg(__fmul2_rn(dx, dy)));
-    const float2 b2 = make_float2(base, base), mx = __fadd2_rn(dx, b2), my = __fadd2_rn(dy, b2);
-    const float2 mss = __ffma2_rn(mx, mx, __fmul2_rn(my, my)), mxy = __fmul2_rn(mx, my);
+    const float2 mx = make_float2(m[0][j], m[0][j + 1]), my = make_float2(m[1][j], m[1][j + 1]);
+    const float2 exx = make_float2(m[2][j], m[2][j + 1]), eyy = make_float2(m[3][j], m[3][j + 1]);
+    const float2 exy = make_float2(m[4][j], m[4][j + 1]);
+    const float2 mxx = __fmul2_rn(mx, mx), myy = __fmul2_rn(my, my), mxy = __fmul2_rn(mx, my);
+    const float2 sxx = __fadd2_rn(exx, neg(mxx)), syy = __fadd2_rn(eyy, neg(myy)), sxy = __fadd2_rn(exy, neg(mxy));
     const float2 N1 = __ffma2_rn(two, mxy, c1), N2 = __ffma2_rn(two, sxy, c2);
-    const float2 D1 = __fadd2_rn(mss, c1), D2 = __fadd2_rn(sss, c2);
+    const float2 D1 = __fadd2_rn(__fadd2_rn(mxx, myy), c1), D2 = __fadd2_rn(__fadd2_rn(sxx, syy), c2);
     const float2 iD1 = make_float2(rcp_approx(D1.x), rcp_approx(D1.y));
     const float2 iD2 = make_float2(rcp_approx(D2.x), rcp_approx(D2.y));
     const float2 iD = __fmul2_rn(iD1, iD2);
     const float2 S = __fmul2_rn(__fmul2_rn(N1, N2), iD);
-    // dS/dmx = 2 my (N2 - N1) iD - 2 mx S (iD1 - iD2), dS/dess = -S iD2, dS/dexy = 2 N1 iD
+    // dS/dmx = 2 my (N2 - N1) iD - 2 mx S (iD1 - iD2), dS/dexx = -S iD2, dS/dexy = 2 N1 iD
     const float2 t1 = __fmul2_rn(__fmul2_rn(__fmul2_rn(two, my), __fadd2_rn(N2, neg(N1))), iD);
     const float2 t2 = __fmul2_rn(__fmul2_rn(__fmul2_rn(two, mx), S), __fadd2_rn(iD1, neg(iD2)));
     const float2 g0 = __fmul2_rn(dl, __fadd2_rn(t1, neg(t2)));
