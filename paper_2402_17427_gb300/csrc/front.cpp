@@ -25,6 +25,7 @@ using torch::autograd::AutogradContext;
 using torch::autograd::Function;
 using torch::autograd::variable_list;
 
+decltype(&vg_rasterize_forward) g_rasterize_forward = nullptr;
 decltype(&vg_rasterize_backward) g_rasterize_backward = nullptr;
 decltype(&vg_loss_l1_dssim_grad) g_loss_grad = nullptr;
 
@@ -51,6 +52,11 @@ T from_bytes(const std::string& s) {
   return v;
 }
 
+// Forward calls made on one workspace, shared by its owner and the nodes that read the workspace later.
+struct Uses {
+  std::shared_ptr<int64_t> n = std::make_shared<int64_t>(0);
+};
+
 // What a render's backward needs besides the saved tensors.
 struct RenderCall : torch::CustomClassHolder {
   vg_camera cam;
@@ -58,6 +64,8 @@ struct RenderCall : torch::CustomClassHolder {
   int32_t degree = 0;
   int64_t capacity = 0;
   at::Tensor rgb, T, last, workspace;
+  std::shared_ptr<int64_t> uses;      // null: the workspace is this render's alone
+  int64_t use = 0;
 };
 
 struct RenderNode : Function<RenderNode> {
@@ -94,8 +102,22 @@ struct RenderNode : Function<RenderNode> {
     p.sh = ptr(s[4]);
     p.n = s[0].size(0);
     p.sh_degree = call->degree;
+    at::Tensor workspace = call->workspace;
+    if (call->uses && *call->uses != call->use) {
+      // Another forward has overwritten the workspace (two renders of one Rasterizer before the first one's
+      // backward): its lists are another render's, perhaps in another layout.  This one's are made again, in a
+      // workspace of their own, since the later render's backward still needs the shared one.
+      workspace = at::empty_like(call->workspace);
+      const at::Tensor T = at::empty_like(s[5]), last = at::empty_like(s[6]);
+      const at::Tensor rgb = at::empty_like(dL), counters = at::empty({VG_CNT_LEN}, dL.options().dtype(at::kLong));
+      const vg_status again = g_rasterize_forward(
+          &p, &call->cam, &call->opts, workspace.data_ptr(), static_cast<size_t>(workspace.numel()), call->capacity,
+          ptr(rgb), ptr(T), static_cast<uint32_t*>(last.data_ptr()), static_cast<int64_t*>(counters.data_ptr()),
+          current_stream(dL));
+      if (again != VG_OK) raise_status(again, "vg_rasterize_forward");
+    }
     const vg_status status = g_rasterize_backward(
-        &p, &call->cam, &call->opts, call->workspace.data_ptr(), static_cast<size_t>(call->workspace.numel()),
+        &p, &call->cam, &call->opts, workspace.data_ptr(), static_cast<size_t>(workspace.numel()),
         call->capacity, ptr(s[5]), static_cast<const uint32_t*>(s[6].data_ptr()), ptr(dL), ptr(g[0]), ptr(g[1]),
         ptr(g[2]), ptr(g[3]), ptr(g[4]), nullptr, current_stream(dL));
     if (status != VG_OK) raise_status(status, "vg_rasterize_backward");
@@ -106,7 +128,7 @@ struct RenderNode : Function<RenderNode> {
 at::Tensor attach_render(const at::Tensor& means, const at::Tensor& log_scales, const at::Tensor& quats,
                          const at::Tensor& logits, const at::Tensor& sh, const at::Tensor& rgb, const at::Tensor& T,
                          const at::Tensor& last, const at::Tensor& workspace, int64_t capacity, int32_t degree,
-                         const pybind11::bytes& cam, const pybind11::bytes& opts) {
+                         const pybind11::bytes& cam, const pybind11::bytes& opts, const Uses* uses) {
   auto call = c10::make_intrusive<RenderCall>();
   call->cam = from_bytes<vg_camera>(cam);
   call->opts = from_bytes<vg_raster_opts>(opts);
@@ -116,13 +138,12 @@ at::Tensor attach_render(const at::Tensor& means, const at::Tensor& log_scales, 
   call->T = T;
   call->last = last;
   call->workspace = workspace;
+  if (uses) {
+    call->uses = uses->n;
+    call->use = *uses->n;
+  }
   return RenderNode::apply(means, log_scales, quats, logits, sh, std::move(call));
 }
-
-// Forward calls made on one loss workspace.
-struct Uses {
-  std::shared_ptr<int64_t> n = std::make_shared<int64_t>(0);
-};
 
 struct LossCall : torch::CustomClassHolder {
   int32_t width = 0, height = 0;
@@ -183,13 +204,14 @@ at::Tensor attach_loss(const at::Tensor& img, const at::Tensor& target, const at
 }  // namespace
 
 PYBIND11_MODULE(_vgfront, m) {
-  m.def("init", [](uintptr_t rasterize_backward, uintptr_t loss_grad) {
+  m.def("init", [](uintptr_t rasterize_forward, uintptr_t rasterize_backward, uintptr_t loss_grad) {
+    g_rasterize_forward = reinterpret_cast<decltype(g_rasterize_forward)>(rasterize_forward);
     g_rasterize_backward = reinterpret_cast<decltype(g_rasterize_backward)>(rasterize_backward);
     g_loss_grad = reinterpret_cast<decltype(g_loss_grad)>(loss_grad);
   });
   pybind11::class_<Uses>(m, "Uses")
       .def(pybind11::init<>())
-      .def(pybind11::pickle([](const Uses& u) { return *u.n; },        // a copy of a loss object counts by itself
+      .def(pybind11::pickle([](const Uses& u) { return *u.n; },        // a copy of a workspace counts by itself
                             [](int64_t n) {
                               Uses u;
                               *u.n = n;
@@ -197,6 +219,9 @@ PYBIND11_MODULE(_vgfront, m) {
                             }))
       .def("bump", [](Uses& u) { ++*u.n; })
       .def_property_readonly("value", [](const Uses& u) { return *u.n; });
-  m.def("attach_render", &attach_render);
+  using pybind11::arg;
+  m.def("attach_render", &attach_render, arg("means"), arg("log_scales"), arg("quats"), arg("logits"), arg("sh"),
+        arg("rgb"), arg("T"), arg("last"), arg("workspace"), arg("capacity"), arg("degree"), arg("cam"), arg("opts"),
+        arg("uses") = nullptr);
   m.def("attach_loss", &attach_loss);
 }

@@ -84,14 +84,17 @@ def _front():
     if _front_module is None:
         from . import _vgfront
         lib = B.lib()
-        _vgfront.init(ctypes.cast(lib.vg_rasterize_backward, ctypes.c_void_p).value,
-                      ctypes.cast(lib.vg_loss_l1_dssim_grad, ctypes.c_void_p).value)
+        _vgfront.init(*(ctypes.cast(f, ctypes.c_void_p).value for f in
+                        (lib.vg_rasterize_forward, lib.vg_rasterize_backward, lib.vg_loss_l1_dssim_grad)))
         _front_module = _vgfront
     return _front_module
 
 
 class Workspace:
     """Caller-owned device workspace of one view, grown when a render needs more pairs."""
+
+    calls = 0          # renders made on the buffer
+    uses = None        # their number as the autograd nodes see it (made with the first node on the buffer)
 
     def __init__(self, device=None, pair_capacity: int | None = None):
         self.device = torch.device(device or "cuda")
@@ -109,6 +112,10 @@ class Workspace:
             raise ValueError("invalid rasteriser sizes")
         if self.buf is None or self.buf.numel() < need:
             self.buf = torch.empty(need, dtype=torch.uint8, device=self.device)
+            self.uses = None
+        self.calls += 1
+        if self.uses is not None:
+            self.uses.bump()
         self.key = (n, width, height, cap, opts.tile_size)
         return self.buf, need
 
@@ -191,16 +198,23 @@ class _RasterizeFn(torch.autograd.Function):
     """rasterize() through a Rasterizer subclass: its own forward and backward are called."""
 
     @staticmethod
+    def use(rasterizer):
+        """The render that the rasteriser's workspace holds (None for one without such a workspace)."""
+        return getattr(getattr(rasterizer, "ws", None), "calls", None)
+
+    @staticmethod
     def forward(ctx, means, log_scales, quats, logits, sh, degree, cam, rasterizer):
         rgb, T, last = rasterizer.forward(means, log_scales, quats, logits, sh, degree, cam)
         ctx.save_for_backward(means, log_scales, quats, logits, sh, T, last)
-        ctx.degree, ctx.cam, ctx.rasterizer = degree, cam, rasterizer
+        ctx.degree, ctx.cam, ctx.rasterizer, ctx.use = degree, cam, rasterizer, _RasterizeFn.use(rasterizer)
         ctx.mark_non_differentiable(T, last)
         return rgb, T, last
 
     @staticmethod
     def backward(ctx, dL_drgb, _dT, _dlast):
         means, log_scales, quats, logits, sh, T, last = ctx.saved_tensors
+        if _RasterizeFn.use(ctx.rasterizer) != ctx.use:      # another render has overwritten the workspace: made again
+            ctx.rasterizer.forward(means, log_scales, quats, logits, sh, ctx.degree, ctx.cam)
         grads = ctx.rasterizer.backward(means, log_scales, quats, logits, sh, ctx.degree, ctx.cam, T, last,
                                         dL_drgb)
         return (*grads, None, None, None)
@@ -214,8 +228,11 @@ def rasterize(means, log_scales, quats, logits, sh, degree: int, cam: Camera, ra
         return rgb
     camc = camera_c(cam)
     rgb, T, last = r.forward(means, log_scales, quats, logits, sh, degree, camc)
-    return _front().attach_render(means, log_scales, quats, logits, sh, rgb, T, last, r.ws.buf, r.ws.capacity,
-                                  int(degree), bytes(camc), bytes(r.settings.c()))
+    front = _front()
+    if getattr(r.ws, "uses", None) is None:
+        r.ws.uses = front.Uses()
+    return front.attach_render(means, log_scales, quats, logits, sh, rgb, T, last, r.ws.buf, r.ws.capacity,
+                               int(degree), bytes(camc), bytes(r.settings.c()), r.ws.uses)
 
 
 class LossL1DSSIM:
