@@ -19,6 +19,9 @@
 
 #include "vgrast.h"
 
+// What this file was compiled against: the build compares it with what is installed.
+__attribute__((used)) extern const char vg_front_key[] = VG_FRONT_KEY;
+
 namespace {
 
 using torch::autograd::AutogradContext;

@@ -12,6 +12,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import os
 
 import numpy as np
 import torch
@@ -79,9 +80,16 @@ _front_module = None
 
 
 def _front():
-    """The autograd nodes in C++ (csrc/front.cpp), bound to the C ABI that the binding loaded."""
+    """The autograd nodes in C++ (csrc/front.cpp), bound to the C ABI that the binding loaded; None where they were
+    not built (no torch headers), and the nodes written in Python serve."""
     global _front_module
     if _front_module is None:
+        from . import _build
+        if not os.path.exists(_build.FRONT):
+            return None
+        if not _build.front_matches(torch):
+            raise RuntimeError(f"{_build.FRONT} was compiled against another torch: build it with "
+                               "paper_2402_17427_gb300._build.build()")
         from . import _vgfront
         lib = B.lib()
         _vgfront.init(*(ctypes.cast(f, ctypes.c_void_p).value for f in
@@ -223,12 +231,12 @@ class _RasterizeFn(torch.autograd.Function):
 def rasterize(means, log_scales, quats, logits, sh, degree: int, cam: Camera, rasterizer: Rasterizer | None = None):
     """Differentiable render: returns the image [3,H,W]; gradients flow to the raw parameters."""
     r = rasterizer or Rasterizer()
-    if type(r) is not Rasterizer or "forward" in r.__dict__ or "backward" in r.__dict__:
+    front = _front()
+    if front is None or type(r) is not Rasterizer or "forward" in r.__dict__ or "backward" in r.__dict__:
         rgb, _T, _last = _RasterizeFn.apply(means, log_scales, quats, logits, sh, degree, cam, r)
         return rgb
     camc = camera_c(cam)
     rgb, T, last = r.forward(means, log_scales, quats, logits, sh, degree, camc)
-    front = _front()
     if getattr(r.ws, "uses", None) is None:
         r.ws.uses = front.Uses()
     return front.attach_render(means, log_scales, quats, logits, sh, rgb, T, last, r.ws.buf, r.ws.capacity,
@@ -243,19 +251,19 @@ class LossL1DSSIM:
         self.buf = None
         self.loss = None
         self.grad = None
-        self.uses = None        # forward calls on this workspace (the SSIM maps they leave behind)
+        self.calls = 0          # forward calls on this workspace (the SSIM maps they leave behind)
 
-    @property
-    def calls(self) -> int:
-        return self.uses.value if self.uses is not None else 0
+    uses = None        # their number as the autograd nodes see it (made with the first node on the buffer)
 
     def _workspace(self, img):
         _, H, W = img.shape
         need = B.vg_loss_workspace_bytes(W, H)
         if self.buf is None or self.buf.numel() < need:
             self.buf = torch.empty(need, dtype=torch.uint8, device=img.device)
-            self.uses = _front().Uses()
-        self.uses.bump()
+            self.uses = None
+        self.calls += 1
+        if self.uses is not None:
+            self.uses.bump()
         return W, H
 
     def __call__(self, img: torch.Tensor, target: torch.Tensor, reuse: bool = False):
@@ -311,12 +319,15 @@ class _LossFn(torch.autograd.Function):
 def l1_dssim_loss(img, target, lam: float = 0.2, lossobj: LossL1DSSIM | None = None):
     """Differentiable Eq. 1 loss ((1 - lam) L1 + lam D-SSIM) computed by the CUDA kernels."""
     f = lossobj or LossL1DSSIM(lam)
-    if type(f) is not LossL1DSSIM or "value" in f.__dict__ or "grad_scaled" in f.__dict__:
+    front = _front()
+    if front is None or type(f) is not LossL1DSSIM or "value" in f.__dict__ or "grad_scaled" in f.__dict__:
         return _LossFn.apply(img, target, f)
     with torch.no_grad():
         x, y = img.contiguous(), target.contiguous()
     loss = f.value(x, y)
-    return _front().attach_loss(img, target, x, y, loss, f.buf, f.uses, int(x.shape[2]), int(x.shape[1]), f.lam)
+    if f.uses is None:
+        f.uses = front.Uses()
+    return front.attach_loss(img, target, x, y, loss, f.buf, f.uses, int(x.shape[2]), int(x.shape[1]), f.lam)
 
 
 def to_device(g, device="cuda"):
