@@ -225,7 +225,10 @@ __device__ __forceinline__ void project(const KGauss& g, const KCam& cm, const K
   P.A = TS[0][0] * P.T[0] + TS[0][1] * P.T[1] + TS[0][2] * P.T[2] + op.dilation;
   P.B = TS[0][0] * P.T[3] + TS[0][1] * P.T[4] + TS[0][2] * P.T[5];
   P.C = TS[1][0] * P.T[3] + TS[1][1] * P.T[4] + TS[1][2] * P.T[5] + op.dilation;
-  const float det = P.A * P.C - P.B * P.B;
+  // The fused form by name: visibility hangs on its sign, which must not depend on what else a kernel takes from
+  // the determinant (where only the sign was used, the compiler compared the two rounded products, and needles
+  // whose products round to the same value were culled).
+  const float det = __fmaf_rn(P.A, P.C, -__fmul_rn(P.B, P.B));
   if (!(det > 0.f)) return;
   const float idet = 1.f / det;
   P.ca = P.C * idet;
