@@ -282,14 +282,17 @@ __device__ __forceinline__ dd dd_clamp(dd v, float lo, float hi) {
   return v < dd(lo) ? dd(lo) : dd(hi) < v ? dd(hi) : v;
 }
 
-// Signed area between the image of the edge p -> n (camera coordinates, both in front) and the y axis,
-// with x clamped to [-1/2, W - 1/2] and y to [-1/2, H - 1/2]: the integral of clamp(x(y)) dy over the
-// edge.  Summed over a closed polygon's edges it is the signed area of its intersection with that
-// rectangle.  The bounds of y are met in space, where they are linear, not on the image, where the end
-// of an edge beside the camera lies a million pixels off and takes the digits with it.
-__device__ __forceinline__ dd edge_area(const dd* p, const dd* n, const vg_camera& cam) {
-  const float xh = (float)cam.width - 0.5f, yh = (float)cam.height - 0.5f;
-  const dd fx(cam.fx), fy(cam.fy), cx(cam.cx), cy(cam.cy), below = cy + dd(0.5f), above = dd(yh) - cy;
+// Signed area between the image of the edge p -> n (camera coordinates, both in front) and the image's left
+// side, with x clamped to [-1/2, W - 1/2] and y to [-1/2, H - 1/2]: the integral of clamp(x(y)) + 1/2 over
+// the edge's y.  Summed over a closed polygon's edges it is the signed area of its intersection with that
+// rectangle, and exactly 0 for a polygon beside the image: above and below no edge has a y in range, on the
+// left every x is clamped to 0, and on the right (where the dy would only cancel up to rounding) no edge
+// sets `within`, which says that some of it has an x left of the right side.  The bounds of y are met in
+// space, where they are linear, not on the image, where the end of an edge beside the camera lies a
+// million pixels off and takes the digits with it.
+__device__ __forceinline__ dd edge_area(const dd* p, const dd* n, const vg_camera& cam, bool& within) {
+  const float width = (float)cam.width, yh = (float)cam.height - 0.5f;
+  const dd fx(cam.fx), fy(cam.fy), cx = dd(cam.cx) + dd(0.5f), cy(cam.cy), below = cy + dd(0.5f), above = dd(yh) - cy;
   const dd ph = fy * p[1], nh = fy * n[1];
   const dd lo0 = ph + below * p[2], lo1 = nh + below * n[2];       // >= 0: at or above the lower bound
   const dd hi0 = above * p[2] - ph, hi1 = above * n[2] - nh;       // >= 0: at or below the upper bound
@@ -308,7 +311,8 @@ __device__ __forceinline__ dd edge_area(const dd* p, const dd* n, const vg_camer
   dd xa, ya, xb, yb;
   at(p, ph, lo0, hi0, xa, ya);
   at(n, nh, lo1, hi1, xb, yb);
-  const dd dy = yb - ya, ca = dd_clamp(xa, -0.5f, xh), cb = dd_clamp(xb, -0.5f, xh);
+  const dd dy = yb - ya, ca = dd_clamp(xa, 0.f, width), cb = dd_clamp(xb, 0.f, width);
+  within = within || !(ca == dd(width) && cb == dd(width));
   if (ca == cb) return dy * ca;
   const dd mean = dd(0.5f) * (ca + cb);
   if (ca == xa && cb == xb) return dy * mean;
@@ -323,18 +327,21 @@ __device__ __forceinline__ dd edge_area(const dd* p, const dd* n, const vg_camer
 struct CamBox {
   dd c0[3], e[3][3];
   int away;
+  bool thin;        // a line or a point
 };
 constexpr float kFarBox = 1e9f, kNearest = 1e-6f, kLongest = 1e7f;   // metres, metres, pixels
 __device__ __forceinline__ CamBox cam_box(const float* __restrict__ box, const vg_camera& cam) {
   CamBox q;
   dd lo[3], len[3];
   float R[3][3], top = 0.f;
+  int flat = 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const float u = fminf(box[a], box[a + 3]), v = fmaxf(box[a], box[a + 3]);
     lo[a] = dd(u);
     len[a] = dd(v) - dd(u);
     top = fmaxf(top, fmaxf(fabsf(u), fabsf(v)));
+    flat += u == v ? 1 : 0;
   }
   bool ok = top < kFarBox && cam.near_plane > kNearest && cam.fx < kLongest && cam.fy < kLongest &&
             fabsf(cam.cx) < kLongest && fabsf(cam.cy) < kLongest;
@@ -356,6 +363,7 @@ __device__ __forceinline__ CamBox cam_box(const float* __restrict__ box, const v
   // the camera (the origin) against the planes of each axis's two faces, normal R_b x R_c (so that a
   // flat box has two faces too, one of them turned away)
   q.away = 0;
+  q.thin = flat >= 2;
   dd det(0.f);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -393,7 +401,7 @@ __device__ dd face_area(const CamBox& q, int face, const vg_camera& cam) {
   // corners in the order b, c: counter-clockwise from outside on the upper face, clockwise on the lower
   const int around[4] = {base, base | b, base | b | c, base | c};
   dd p[3], area(0.f), out[3], in[3];
-  bool cuts = false;
+  bool cuts = false, within = false;
   cam_corner(q, around[3], p);
 #pragma unroll 1
   for (int k = 0; k < 4; ++k) {
@@ -412,13 +420,13 @@ __device__ dd face_area(const CamBox& q, int face, const vg_camera& cam) {
           else u[r] = in[r] = w[r];
         }
       }
-      area = area + edge_area(u, v, cam);
+      area = area + edge_area(u, v, cam, within);
     }
 #pragma unroll
     for (int r = 0; r < 3; ++r) p[r] = n[r];
   }
-  if (cuts) area = area + edge_area(out, in, cam);       // along the near plane
-  return (face & 1) ? area : -area;
+  if (cuts) area = area + edge_area(out, in, cam, within);       // along the near plane
+  return !within ? dd(0.f) : (face & 1) ? area : -area;
 }
 
 // Bound by instruction issue.  A box wholly in front of the near plane (most) takes no arrays, sorts or
@@ -461,10 +469,11 @@ __global__ void __launch_bounds__(kVisThreads) visibility_kernel(const float* __
     const int edges = c_silhouette.n[q.away];
     if (q.away == 0) {
       put(idx, box_visibility(box, cam));
-    } else if (in == 0) {
+    } else if (in == 0 || q.thin) {      // thin: no area, and its edges' would cancel only up to rounding
       put(idx, 0.0);
     } else if (in == 8 && edges > 0) {
       dd area(0.f);
+      bool within = false;
 #pragma unroll 1
       for (int k = 0; k < edges; ++k) {
         const int w = c_silhouette.edge[q.away][k];
@@ -475,9 +484,9 @@ __global__ void __launch_bounds__(kVisThreads) visibility_kernel(const float* __
           p[r] = dd(a.x, a.y);
           n[r] = dd(b.x, b.y);
         }
-        area = area + edge_area(p, n, cam);
+        area = area + edge_area(p, n, cam, within);
       }
-      put(idx, share(area, cam));
+      put(idx, within ? share(area, cam) : 0.0);
     } else {
       s_cut[atomicAdd(&s_ncut, 1)] = threadIdx.x;
     }
