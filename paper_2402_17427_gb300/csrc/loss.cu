@@ -2,10 +2,12 @@
 //
 // SSIM uses an 11x11 Gaussian window (sigma 1.5, separable, normalised) with zero padding and
 // C1 = 0.01^2, C2 = 0.03^2; both terms are means over 3 H W.  With the local moments
-// mx = w*x, exx = w*x^2, exy = w*(x y) (and my, eyy),
-//   S = (2 mx my + C1)(2 (exy - mx my) + C2) / ((mx^2 + my^2 + C1)(exx - mx^2 + eyy - my^2 + C2))
+// mx = w*x, my = w*y, ess = w*(x^2 + y^2), exy = w*(x y),
+//   S = (2 mx my + C1)(2 (exy - mx my) + C2) / ((mx^2 + my^2 + C1)(ess - mx^2 - my^2 + C2))
+// (the two second moments only enter as their sum, so four windows do instead of five; variances and
+// covariance are formed of differences from a value in the window, see base_of),
 // and dL/dx(q) = l1' + (w * a)(q) + 2 x(q) (w * b)(q) + y(q) (w * c)(q), where a, b, c are
-// dL/dS times dS/dmx, dS/dexx, dS/dexy at every pixel (the window is symmetric, so correlation
+// dL/dS times dS/dmx, dS/dess, dS/dexy at every pixel (the window is symmetric, so correlation
 // with it is its own adjoint).  Two kernels: moments -> (a, b, c) maps + partial sums, then the
 // transposed convolution of the maps.  32x32 output tiles, halo 5, separable passes in shared
 // memory.  Each thread slides the 11-tap window along a run of outputs so that every staged value
@@ -55,7 +57,7 @@ __device__ __forceinline__ int qcol(int q) { return q + (q >> 3); }
 __device__ __forceinline__ int hs_at(int r, int c) { return r * LT + 2 * ((c >> 1) ^ ((r >> 1) & 3)) + (c & 1); }
 
 // Rows 2p and 2p + 1, columns c .. c + GH - 1 of F quantities, two columns a store: the moment pass is bound
-// by the shared-memory pipe, and single columns take twice its clocks for these stores (53.4 -> 51.9 us at 1080p).
+// by the shared-memory pipe, and single columns took twice its clocks for these stores (51.5 -> 47.6 us at 1080p).
 template <int F>
 __device__ __forceinline__ void store_rows(const float2 (&a)[F][GH], float (*hs)[LTH * LT], int p, int c) {
 #pragma unroll
@@ -65,6 +67,18 @@ __device__ __forceinline__ void store_rows(const float2 (&a)[F][GH], float (*hs)
       *reinterpret_cast<float2*>(&hs[f][hs_at(2 * p, c + j)]) = make_float2(a[f][j].x, a[f][j + 1].x);
       *reinterpret_cast<float2*>(&hs[f][hs_at(2 * p + 1, c + j)]) = make_float2(a[f][j].y, a[f][j + 1].y);
     }
+}
+
+__device__ __forceinline__ float2 neg(float2 v) { return make_float2(-v.x, -v.y); }
+
+// What the values of overlapping windows are taken relative to, so that a variance is no difference of large
+// numbers: of values that lie in all of these windows the one of smallest magnitude, or 0 where their signs
+// differ.  It is never far from what a window holds: |base| is at most each of the four, which have 0.15 of
+// every window's weight, so squares relative to it are at most 15 times those of the values themselves, and for
+// smooth images far smaller.  A base from outside a window (one pixel or a mean of the tile) costs it
+// its digits where that pixel is a highlight; none leaves the gradient of a photograph 3 times further off.
+__device__ __forceinline__ float base_of(float a, float b, float c, float d) {
+  return fmaxf(fminf(fminf(a, b), fminf(c, d)), 0.f) + fminf(fmaxf(fmaxf(a, b), fmaxf(c, d)), 0.f);
 }
 
 // Block sum: FP32 inside each warp (FP64 is slow on this part), FP64 across the warps.
@@ -173,10 +187,10 @@ __device__ __forceinline__ void stage_pairs(const float* const (&plane)[F], int 
 
 // Moments of a 32x32 output tile: x, y staged with a 5-pixel zero-padded halo as row pairs.  The
 // horizontal pass (21 row pairs x 4 groups of 8 columns) slides the window along a row for two
-// rows at once; the vertical pass (32 columns x 4 groups of 8 rows) slides it down a column.  The
-// values enter as they are: relative to one pixel of the tile (which halves the rounding of smooth images)
-// a pixel unlike its surroundings cost the whole tile its digits, and with x^2 + y^2 in one window instead
-// of two (four windows: 47 us instead of 52) the gradient's error was 1.12 times as large.
+// rows at once and leaves each row's means, variance sum and covariance, formed relative to a base for its 8
+// outputs; the vertical pass (32 columns x 4 groups of 8 rows) slides down a column and adds the rows' own
+// variances to that of their means, relative to another base.  49.5 us at 1080p, by the shared-memory pipe (69%)
+// and issue (66%) together; five windows of the values as they are took 51.9.
 // kMaps: the derivative maps for the gradient pass are written; without it the pass leaves the
 // partial sums alone (the evaluation needs no gradient).
 template <bool kMaps>
@@ -186,7 +200,7 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
                                                                     double* __restrict__ partials) {
   pdl_enter();
   __shared__ __align__(16) float4 s4[NRP][QP];   // (x row 2p, x row 2p + 1, y row 2p, y row 2p + 1)
-  __shared__ __align__(16) float hs[5][LTH * LT];
+  __shared__ __align__(16) float hs[4][LTH * LT];   // mx, my, sxx + syy, sxy along a row
   __shared__ double red[kLossThreads / 32];
   const int c = blockIdx.z;
   const int ox = blockIdx.x * LT, oy = blockIdx.y * LT;
@@ -200,27 +214,56 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
   __syncthreads();
   if (threadIdx.x < NH) {
     const int p = threadIdx.x >> 2, g = threadIdx.x & 3;
-    float2 a[5][GH];
-    window_pairs<5, GH>(win, [&](int i, float2 (&v)[5]) {
-      const float4 s = s4[p][qcol(GH * g + i)];
-      const float2 xv = make_float2(s.x, s.y), yv = make_float2(s.z, s.w);
-      v[0] = xv; v[1] = yv; v[2] = __fmul2_rn(xv, xv); v[3] = __fmul2_rn(yv, yv); v[4] = __fmul2_rn(xv, yv);
+    float2 a[4][GH];
+    float4 mid[4];                        // staged columns GH - 1 .. 10 of the group: in every one of its windows
+#pragma unroll
+    for (int k = 0; k < 4; ++k) mid[k] = s4[p][qcol(GH * g + GH - 1 + k)];
+    const float2 bx = make_float2(base_of(mid[0].x, mid[1].x, mid[2].x, mid[3].x),
+                                  base_of(mid[0].y, mid[1].y, mid[2].y, mid[3].y));
+    const float2 by = make_float2(base_of(mid[0].z, mid[1].z, mid[2].z, mid[3].z),
+                                  base_of(mid[0].w, mid[1].w, mid[2].w, mid[3].w));
+    const float2 nbx = neg(bx), nby = neg(by);
+    window_pairs<4, GH>(win, [&](int i, float2 (&v)[4]) {
+      const float4 s = i >= GH - 1 && i <= 10 ? mid[i - (GH - 1)] : s4[p][qcol(GH * g + i)];
+      v[0] = __fadd2_rn(make_float2(s.x, s.y), nbx);
+      v[1] = __fadd2_rn(make_float2(s.z, s.w), nby);
+      v[2] = __ffma2_rn(v[0], v[0], __fmul2_rn(v[1], v[1]));
+      v[3] = __fmul2_rn(v[0], v[1]);
     }, a);
+#pragma unroll
+    for (int j = 0; j < GH; ++j) {
+      const float2 dx = a[0][j], dy = a[1][j];
+      a[2][j] = __fadd2_rn(a[2][j], neg(__ffma2_rn(dx, dx, __fmul2_rn(dy, dy))));
+      a[3][j] = __fadd2_rn(a[3][j], neg(__fmul2_rn(dx, dy)));
+      a[0][j] = __fadd2_rn(dx, bx);
+      a[1][j] = __fadd2_rn(dy, by);
+    }
     store_rows(a, hs, p, GH * g);
   }
   __syncthreads();
   const int q = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * GV;   // column q, output rows r0 .. r0 + 7
-  float m[5][GV];
-  window_column<5>(win, [&](int i, float (&v)[5]) {
+  float m[4][GV];
+  float mid[2][4];                        // rows GV - 1 .. 10 of the column: in every window of its GV outputs
 #pragma unroll
-    for (int f = 0; f < 5; ++f) v[f] = hs[f][hs_at(r0 + i, q)];
+  for (int k = 0; k < 4; ++k) {
+    mid[0][k] = hs[0][hs_at(r0 + GV - 1 + k, q)];
+    mid[1][k] = hs[1][hs_at(r0 + GV - 1 + k, q)];
+  }
+  const float bx = base_of(mid[0][0], mid[0][1], mid[0][2], mid[0][3]);
+  const float by = base_of(mid[1][0], mid[1][1], mid[1][2], mid[1][3]);
+  window_column<4>(win, [&](int i, float (&v)[4]) {
+    const int at = hs_at(r0 + i, q);
+    const bool held = i >= GV - 1 && i <= 10;
+    v[0] = (held ? mid[0][i - (GV - 1)] : hs[0][at]) - bx;
+    v[1] = (held ? mid[1][i - (GV - 1)] : hs[1][at]) - by;
+    v[2] = fmaf(v[0], v[0], fmaf(v[1], v[1], hs[2][at]));
+    v[3] = fmaf(v[0], v[1], hs[3][at]);
   }, m);
   // the per-pixel SSIM and its three partial derivatives for two rows at once (packed FP32; the
   // reciprocals approximate, within 1 ulp)
   const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
   const float2 c1 = make_float2(C1, C1), c2 = make_float2(C2, C2), two = make_float2(2.f, 2.f);
   const float2 dl = make_float2(dLdS, dLdS);
-  auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
   float ssum = 0.f, l1sum = 0.f;
   const float* sf = reinterpret_cast<const float*>(&s4[0][0]);
   const int gx = ox + q;
@@ -236,18 +279,19 @@ __global__ void __launch_bounds__(kLossThreads) ssim_forward_kernel(const float*
       const float* cell = sf + ((sr >> 1) * QP + qcol(q + HALO)) * 4;
       l1sum += fabsf(cell[sr & 1] - cell[2 + (sr & 1)]);
     }
-    const float2 mx = make_float2(m[0][j], m[0][j + 1]), my = make_float2(m[1][j], m[1][j + 1]);
-    const float2 exx = make_float2(m[2][j], m[2][j + 1]), eyy = make_float2(m[3][j], m[3][j + 1]);
-    const float2 exy = make_float2(m[4][j], m[4][j + 1]);
-    const float2 mxx = __fmul2_rn(mx, mx), myy = __fmul2_rn(my, my), mxy = __fmul2_rn(mx, my);
-    const float2 sxx = __fadd2_rn(exx, neg(mxx)), syy = __fadd2_rn(eyy, neg(myy)), sxy = __fadd2_rn(exy, neg(mxy));
+    const float2 dx = make_float2(m[0][j], m[0][j + 1]), dy = make_float2(m[1][j], m[1][j + 1]);
+    const float2 ess = make_float2(m[2][j], m[2][j + 1]), exy = make_float2(m[3][j], m[3][j + 1]);
+    const float2 sss = __fadd2_rn(ess, neg(__ffma2_rn(dx, dx, __fmul2_rn(dy, dy))));
+    const float2 sxy = __fadd2_rn(exy, neg(__fmul2_rn(dx, dy)));
+    const float2 mx = __fadd2_rn(dx, make_float2(bx, bx)), my = __fadd2_rn(dy, make_float2(by, by));
+    const float2 mss = __ffma2_rn(mx, mx, __fmul2_rn(my, my)), mxy = __fmul2_rn(mx, my);
     const float2 N1 = __ffma2_rn(two, mxy, c1), N2 = __ffma2_rn(two, sxy, c2);
-    const float2 D1 = __fadd2_rn(__fadd2_rn(mxx, myy), c1), D2 = __fadd2_rn(__fadd2_rn(sxx, syy), c2);
+    const float2 D1 = __fadd2_rn(mss, c1), D2 = __fadd2_rn(sss, c2);
     const float2 iD1 = make_float2(rcp_approx(D1.x), rcp_approx(D1.y));
     const float2 iD2 = make_float2(rcp_approx(D2.x), rcp_approx(D2.y));
     const float2 iD = __fmul2_rn(iD1, iD2);
     const float2 S = __fmul2_rn(__fmul2_rn(N1, N2), iD);
-    // dS/dmx = 2 my (N2 - N1) iD - 2 mx S (iD1 - iD2), dS/dexx = -S iD2, dS/dexy = 2 N1 iD
+    // dS/dmx = 2 my (N2 - N1) iD - 2 mx S (iD1 - iD2), dS/dess = -S iD2, dS/dexy = 2 N1 iD
     const float2 t1 = __fmul2_rn(__fmul2_rn(__fmul2_rn(two, my), __fadd2_rn(N2, neg(N1))), iD);
     const float2 t2 = __fmul2_rn(__fmul2_rn(__fmul2_rn(two, mx), S), __fadd2_rn(iD1, neg(iD2)));
     const float2 g0 = __fmul2_rn(dl, __fadd2_rn(t1, neg(t2)));
