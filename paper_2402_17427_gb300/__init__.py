@@ -5,7 +5,7 @@ tile binning, depth sort, front-to-back alpha compositing and its adjoint — as
 CUDA kernels behind a C ABI (``include/vgrast.h``, ``libvgrast.so``).  Python modules:
 
 * ``binding``   — ctypes binding of the C ABI (same names);
-* ``rasterize`` — torch front end: workspaces, streams, ``torch.autograd.Function``;
+* ``rasterize`` — torch front end: workspaces, streams, autograd nodes;
 * ``batch``     — many cells in one launch per stage, with the per-cell autotuner;
 * ``serving``   — continuous-batching novel-view server over the merged scene;
 * ``scenes``    — seeded synthetic scenes and cameras.

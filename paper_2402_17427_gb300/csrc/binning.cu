@@ -3,7 +3,7 @@
 // The result is, per tile, the list of Gaussians whose tile rectangle contains it, ordered by
 // (FP32 depth bits, Gaussian index): exactly the order of a stable sort of the 64-bit keys
 // (tile << 32 | depth bits) emitted in index order.  It is produced in two cheaper steps:
-//   1. the visible Gaussians, compacted in index order by the projection kernel, are stably
+//   1. the visible Gaussians, compacted in index order by the projection, are stably
 //      radix-sorted by depth (V elements, not P; only the bits in which the keys differ);
 //   2. pairs (tile, depth rank) are emitted in that depth order and stably radix-sorted by tile
 //      id only (ceil(log2 tiles) bits), which keeps the depth order inside every tile.
@@ -878,7 +878,7 @@ cudaError_t launch_binning(const DevTables* tab, int n, int degree, int tiles, i
   } else {
     join = nullptr;                     // the side stream's last work is the records: rec_join
   }
-  // 1. depth sort of the visible Gaussians (compacted by the projection kernel); passes beyond
+  // 1. depth sort of the visible Gaussians (compacted by the projection); passes beyond
   //    the bits the keys differ in return at once, and the result sits in the buffer
   //    depth_order() names
   for (int pass = 0; pass < kMaxPasses; ++pass) {

@@ -203,7 +203,7 @@ struct Compact {
   float4* key_inputs;              // optional [total_n]: (u, v, r, depth) the keys were decided from
 };
 // Every kernel after the first look-back of a render checks this once: after a wait gave up the
-// compacted and sorted arrays may hold unwritten slots, so no stage may index with them.  The flag
+// sorted arrays may hold unwritten slots, so no stage may index with them.  The flag
 // is set by an earlier kernel of the stream, so a plain load sees it (kernels of one stream see
 // each other's writes); the L1 cache then merges the loads of a block's warps.
 // Programmatic dependent launch: the kernels of a call may be launched so that their blocks are

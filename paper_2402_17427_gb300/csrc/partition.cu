@@ -630,7 +630,7 @@ extern "C" vg_status vg_airspace_boxes(const float* points, const int64_t* cell_
   unsigned* ob = reinterpret_cast<unsigned*>(out_boxes);
   box_init<<<(n_cells + 127) / 128, 128, 0, s>>>(ob, n_cells);
   int launches = 2;
-  // one launch per group of up to 256 cells; a block reduces 16K points of one cell
+  // one launch per group of up to 256 cells; a block reduces 4K points of one cell
   for (int k0 = 0; k0 < n_cells; k0 += kBoxCellsPerLaunch) {
     BoxJob job{};
     job.n = n_cells - k0 < kBoxCellsPerLaunch ? n_cells - k0 : kBoxCellsPerLaunch;

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(128) record_kernel(const DevTables* __restrict
                                                      const uint32_t* __restrict__ vis_ids,
                                                      const WsHeader* __restrict__ hdr, Splat* __restrict__ splats) {
   pdl_enter();
-  const bool dead = render_dead(hdr);   // the compacted list may hold unwritten slots
+  const bool dead = render_dead(hdr);   // the depth sort beside this gave up: nobody reads the records
   const unsigned nv = hdr->visible;
   if (dead) return;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += gridDim.x * blockDim.x) {
@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(128, 4) preprocess_backward_kernel(
     const DevTables* __restrict__ tab, const uint32_t* __restrict__ vis_ids, const WsHeader* __restrict__ hdr,
     const Splat* __restrict__ splats, const float* __restrict__ g2d, int accumulate) {
   pdl_enter();
-  const bool dead = render_dead(hdr);   // the compacted list may hold unwritten slots
+  const bool dead = render_dead(hdr);   // a sort gave up: ranks and accumulators are not this render's
   const int nv = (int)hdr->visible;
   if (dead) return;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nv; t += gridDim.x * blockDim.x)

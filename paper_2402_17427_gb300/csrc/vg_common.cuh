@@ -195,15 +195,13 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
 
 // Decoupled look-back of ticketed block `blk` whose own count is `tot`, by one whole warp: publishes
 // the block's status word and returns the sum of the counts of all blocks before it (every lane).
-// Blocks only wait on blocks of smaller tickets, which are already running; each wait is bounded by
-// `limit_ns`, after which `bit` is set in *timeout (before this block's prefix is published).
-// publish = false (tests only) withholds this block's words.
+// Blocks only wait on blocks of smaller tickets, which are already running; each wait is bounded by 1 s,
+// after which *timeout is set (before this block's prefix is published).
 __device__ __forceinline__ unsigned lookback(unsigned long long* status, unsigned blk, unsigned tot,
-                                             unsigned* timeout, unsigned bit = 1u,
-                                             unsigned long long limit_ns = 1000000000ull, bool publish = true) {
+                                             unsigned* timeout) {
   const int lane = threadIdx.x & 31;
   unsigned excl = 0;
-  if (lane == 0 && publish) st_relaxed(status + blk, (blk == 0 ? kFlagPrefix : kFlagAggregate) | tot);
+  if (lane == 0) st_relaxed(status + blk, (blk == 0 ? kFlagPrefix : kFlagAggregate) | tot);
   if (blk == 0) return 0;
   long long p = (long long)blk - 1;
   const uint64_t start = global_timer_ns();
@@ -220,15 +218,15 @@ __device__ __forceinline__ unsigned lookback(unsigned long long* status, unsigne
     excl += part;
     if (done) break;
     p -= take;
-    if (take == 0 && global_timer_ns() - start > limit_ns) {   // a predecessor never published
+    if (take == 0 && global_timer_ns() - start > 1000000000ull) {   // a predecessor never published
       if (lane == 0) {
-        atomicOr(timeout, bit);
+        atomicOr(timeout, 1u);
         __threadfence();      // the flag is visible before this block's prefix is
       }
       break;
     }
   }
-  if (lane == 0 && publish) st_relaxed(status + blk, kFlagPrefix | (excl + tot));
+  if (lane == 0) st_relaxed(status + blk, kFlagPrefix | (excl + tot));
   return excl;
 }
 

@@ -33,7 +33,7 @@ class RasterSettings:
     guard: float = 1.3
     stop_rule: int = 0
     count_blends: bool = False
-    test_stall: bool = False      # diagnostic: make the compaction's look-back give up (tests only)
+    test_stall: bool = False      # diagnostic: make the depth sort's look-back give up (tests only)
 
     def c(self, accumulate: bool = False) -> B.vg_raster_opts:
         o = B.vg_raster_opts()
@@ -203,7 +203,7 @@ class Rasterizer:
 
 
 class _RasterizeFn(torch.autograd.Function):
-    """rasterize() through a Rasterizer subclass: its own forward and backward are called."""
+    """rasterize() through a Rasterizer subclass, or without the C++ nodes: its own forward and backward are called."""
 
     @staticmethod
     def use(rasterizer):
@@ -296,8 +296,8 @@ class LossL1DSSIM:
 
 
 class _LossFn(torch.autograd.Function):
-    """l1_dssim_loss() through a LossL1DSSIM subclass.  Forward computes the loss only; backward runs the
-    gradient pass scaled on the device by the incoming gradient (no separate elementwise product)."""
+    """l1_dssim_loss() through a LossL1DSSIM subclass, or without the C++ nodes.  Forward computes the loss only;
+    backward runs the gradient pass scaled on the device by the incoming gradient (no separate elementwise product)."""
 
     @staticmethod
     def forward(ctx, img, target, lossobj):
